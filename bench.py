@@ -91,26 +91,9 @@ BYTES_PER_POINT_STAGE = {"rns": 17 * 4 * 8 / 4, "detonation": 8 * 4 * 8 / 3, "ad
 # the step-fused path reads u^n and writes u^{n+1} once per step (+ the ring)
 BYTES_PER_POINT_STAGE_FUSED = {"advdiff": 2 * 8 / 4, "rns": 2 * 4 * 8 / 4, "detonation": 2 * 4 * 8 / 3}
 # DRAM bytes per launch of the timed kernel (dram__bytes_read.sum +
-# dram__bytes_write.sum) from the ncu captures of the current kernels, by
-# workload and path; the advection-diffusion kernels were captured at
-# N = 2^25 and are scaled by 4 for N = 2^27.
-TRAFFIC_PER_LAUNCH = {
-    ("rns-flame-n16384", "persistent"): 2.5541e+06,  # state and rings read once, writes stay in L2
-    ("rns-flame-n16777216", "stage"): 2 * (8.3054e+08 + 5.2048e+08),  # captured at N = 2^23, x2
-    ("rns-flame-n8388608", "stage"): 8.3054e+08 + 5.2048e+08,
-    ("detonation-n8388608", "stage"): 2.7371e+08 + 2.2617e+08,
-    ("detonation-n16777216", "stage"): 2 * (2.7371e+08 + 2.2617e+08),  # captured at N = 2^23, x2
-    ("advdiff-n134217728", "stage"): 4 * (8.7076e+08 + 5.1195e+08),
-    ("advdiff-n33554432", "stage"): 8.7076e+08 + 5.1195e+08,
-    ("advdiff-n134217728", "fused"): 4 * (4.6988e+08 + 3.0293e+08),  # one step: u^n, u^{n+1}, the ring
-    ("advdiff-n33554432", "fused"): 4.6988e+08 + 3.0293e+08,
-    ("advdiff-n2048", "persistent"): 8.0384e+04,  # one-cluster launch: state and ring read once
-    ("advdiff-n16384", "fused"): 2.8877e+05,  # cooperative fused launch: state and ring read once
-    ("rns-flame-n16777216", "fused"): 2 * (2.6860e+08 + 3.1804e+08),  # tile-fused step, captured at N = 2^23, x2
-    ("rns-flame-n8388608", "fused"): 2.6860e+08 + 3.1804e+08,
-    ("detonation-n16777216", "fused"): 2 * (2.7574e+08 + 2.3274e+08),  # tile-fused step, captured at N = 2^23, x2
-    ("detonation-n8388608", "fused"): 2.7574e+08 + 2.3274e+08,
-}
+# dram__bytes_write.sum) from ncu captures, by workload and path; a workload
+# without a capture of the current kernels has no entry.
+TRAFFIC_PER_LAUNCH = {}
 
 
 # The kernel sources the captured counts above were taken from, per
@@ -119,30 +102,11 @@ TRAFFIC_PER_LAUNCH = {
 # the roofline is then marked stale and its traffic is reported as null
 # until the capture is redone.  A key without an entry is stale.
 KERNEL_FILES = {
-    "stage": ("at_device.cuh", "at_stage.cu"),
-    "persistent": ("at_cluster.cu", "at_device.cuh", "at_persist.cu"),
-    "fused": ("at_device.cuh", "at_fused.cu", "at_tilefused.cu"),
+    "stage": ("at_device.cuh", "at_fixed.cuh", "at_stage.cu"),
+    "persistent": ("at_cluster.cu", "at_device.cuh", "at_fixed.cuh", "at_persist.cu"),
+    "fused": ("at_device.cuh", "at_fixed.cuh", "at_fused.cu", "at_tilefused.cu"),
 }
-_SHA_STAGE = "0cecc1445fec100af6a8261ff949636d13abda82401f91c538bf46eea741a1e2"
-_SHA_PERSISTENT = "b9e03fe76cc5c2182917044ff8965c8a015a4d4ab02a7bc7eaf4e2134e28dab4"
-_SHA_FUSED = "ec36d6c3395c55e85546f641189d941abc7c206c5373b137cce2035fad616f1a"
-PROFILED_SHA256 = {
-    ("detonation-n16777216", "stage"): _SHA_STAGE,
-    ("detonation-n8388608", "stage"): _SHA_STAGE,
-    ("rns-flame-n16777216", "stage"): _SHA_STAGE,
-    ("rns-flame-n8388608", "stage"): _SHA_STAGE,
-    ("advdiff-n134217728", "stage"): _SHA_STAGE,
-    ("advdiff-n33554432", "stage"): _SHA_STAGE,
-    ("rns-flame-n16384", "persistent"): _SHA_PERSISTENT,
-    ("advdiff-n2048", "persistent"): _SHA_PERSISTENT,
-    ("advdiff-n134217728", "fused"): _SHA_FUSED,
-    ("advdiff-n33554432", "fused"): _SHA_FUSED,
-    ("advdiff-n16384", "fused"): _SHA_FUSED,
-    ("rns-flame-n16777216", "fused"): _SHA_FUSED,
-    ("rns-flame-n8388608", "fused"): _SHA_FUSED,
-    ("detonation-n16777216", "fused"): _SHA_FUSED,
-    ("detonation-n8388608", "fused"): _SHA_FUSED,
-}
+PROFILED_SHA256 = {}
 
 
 def sources_sha256(path: str) -> str:

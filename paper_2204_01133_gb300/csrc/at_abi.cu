@@ -314,10 +314,8 @@ atk::StageArgs build_args(const at_problem* pb, const at_delays* dl, const Layou
         const double* d2 = pb->order == 2 ? d2_2 : (pb->order == 4 ? d2_4 : d2_6);
         const double den1 = pb->order == 2 ? 2.0 : (pb->order == 4 ? 12.0 : 60.0);
         const double den2 = pb->order == 2 ? 1.0 : (pb->order == 4 ? 12.0 : 180.0);
-        for (int o = 0; o <= 2 * L.H; ++o) {
-            a.c1[o] = -d1[o] / (den1 * dx);
-            a.c2[o] = d2[o] / (den2 * dx * dx);
-        }
+        a.s1 = -1.0 / (den1 * dx);
+        a.s2 = 1.0 / (den2 * dx * dx);
         if (pb->pde == AT_ADVDIFF) {
             const double cc = pb->prm[0], aa = pb->prm[1];
             for (int o = 0; o <= 2 * L.H; ++o)
@@ -331,13 +329,11 @@ atk::StageArgs build_args(const at_problem* pb, const at_delays* dl, const Layou
             a.k2 = lam;
             a.k3 = lam / (cp * Le);
             // the diffusion rows carry u, the energy term over lambda and Y; the
-            // constants go into the taps (without viscosity every row term is 0)
+            // constants go into the scale (without viscosity every row term is 0)
             const bool visc = a.k2 != 0.0;
-            for (int o = 0; o <= 2 * L.H; ++o) {
-                a.c2v[0][o] = a.c2[o] * a.k0;
-                a.c2v[1][o] = visc ? a.c2[o] * a.k2 : 0.0;
-                a.c2v[2][o] = a.c2[o] * a.k3;
-            }
+            a.s2v[0] = a.s2 * a.k0;
+            a.s2v[1] = visc ? a.s2 * a.k2 : 0.0;
+            a.s2v[2] = a.s2 * a.k3;
             a.kd1 = visc ? a.k1 / a.k2 : 0.0;
             a.kd3 = visc ? pb->prm[6] * a.k3 / a.k2 : 0.0;
         }

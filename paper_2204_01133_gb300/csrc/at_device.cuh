@@ -8,6 +8,7 @@
 
 #include <cstdint>
 
+#include "at_fixed.cuh"
 #include "exp_table.h"
 
 #define AT_KMAX_LIMIT 15
@@ -42,15 +43,15 @@ struct StageArgs {
     uint64_t thr[AT_KMAX_LIMIT];              // Philox word-0 thresholds
     double w[AT_KMAX_LIMIT + 1][AT_QMAX + 1]; // extrapolation weights by delay
     uint8_t wnz[AT_KMAX_LIMIT + 1];           // bit l: level l enters at delay k (weight != 0)
-    double c1[2 * AT_HMAX + 1];               // -d1_m / dx  (central)
-    double c2[2 * AT_HMAX + 1];               //  d2_m / dx^2 (central)
+    double s1;                                // -1 / (D1 dx): scales fx_d1 (central first derivative, negated)
+    double s2;                                // 1 / (D2 dx^2): scales fx_d2
     double cm[2 * AT_HMAX + 1];               // merged advection-diffusion taps
     double prm[16];                           // physics constants (see at.h)
     double k0, k1, k2, k3;                    // derived physics constants
     // reacting flow: the diffusion rows are u, the energy term over lambda and
-    // Y, with the constants in the taps: c2v[v-1][m] = c2[m] times (4/3) mu,
+    // Y, with the constants in the scale: s2v[v-1] = s2 times (4/3) mu,
     // lambda, lambda / (cp Le) for v = 1, 2, 3; kd1 = k1 / k2, kd3 = qc k3 / k2
-    double c2v[3][2 * AT_HMAX + 1];
+    double s2v[3];
     double kd1, kd3;
     // persistent path only
     int64_t* done;       // per PE: stages completed, as the index n*S + s + 1 [P]
@@ -266,7 +267,7 @@ struct Phys<ADVDIFF> {
 
 // Reacting Navier-Stokes: g = [rho u, rho u^2 + p, u (rho E + p), rho u Y,
 // u, ((2/3) mu u^2 + lam T + q_c rhoD Y) / lam, Y, T]; the diffusion rows
-// 4..6 are differentiated with the taps c2v, which carry their constants
+// 4..6 are differentiated with the scales s2v, which carry their constants
 // (4/3) mu, lam and rhoD.  k0 = (4/3) mu, k1 = (2/3) mu, k2 = lam, k3 = rhoD.
 template <>
 struct Phys<RNS> {
@@ -283,9 +284,9 @@ struct Phys<RNS> {
         g[1] = fma(Q[1], u, p);
         g[2] = u * (Q[2] + p);
         g[3] = Q[3] * u;
-        g[4] = u;                                      // times (4/3) mu in the taps
-        g[5] = fma(a.kd1 * u, u, fma(a.kd3, Y, T));    // (k1 u^2 + k2 T + qc k3 Y) / k2; times k2 in the taps
-        g[6] = Y;                                      // times k3 in the taps
+        g[4] = u;                                      // times (4/3) mu in the scale
+        g[5] = fma(a.kd1 * u, u, fma(a.kd3, Y, T));    // (k1 u^2 + k2 T + qc k3 Y) / k2; times k2 in the scale
+        g[6] = Y;                                      // times k3 in the scale
         g[7] = T;
     }
     // the temperature exactly as derive() forms it (same operations, same rounding)
@@ -532,6 +533,19 @@ __device__ __forceinline__ double weno_flux(const double* C, DC dC, DQ dQ, int c
     weno5d(fma(hl, dQ(c + 2), -dC(c + 2)), fma(hl, dQ(c + 1), -dC(c + 1)), fma(hl, dQ(c), -dC(c)),
            fma(hl, dQ(c - 1), -dC(c - 1)), eps, nm, dm, s1m);
     return fma(1.0 / 6.0, fma(fma(np, dm, nm * dp), at_rcp3(dp * dm), -(s1p + s1m)), C[c - 1] + C[c]);
+}
+
+// ---------------------------------------------------------------------------
+// -dF_v/dx plus the diffusion term of variable v of the reacting flow at
+// column c of the derived rows G (row stride ld): the differences in integers
+// (at_fixed.cuh), one FP64 instruction each to scale and add them.
+// ---------------------------------------------------------------------------
+template <int H>
+__device__ __forceinline__ double rns_flux_terms(const StageArgs& a, const double* G, int ld, int v, int c)
+{
+    double K = a.s1 * fx_d1<H>(G + v * ld + c);
+    if (v > 0) K = fma(a.s2v[v - 1], fx_d2<H>(G + (3 + v) * ld + c), K);
+    return K;
 }
 
 // ---------------------------------------------------------------------------

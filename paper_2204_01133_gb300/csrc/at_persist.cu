@@ -70,15 +70,7 @@ __device__ __forceinline__ double point_update(const StageArgs& a, int s, int v,
 #pragma unroll
         for (int o = -H; o <= H; ++o) K = fma(a.cm[o + H], G[c + o], K);
     } else {
-        const double* F = G + v * W2;
-#pragma unroll
-        for (int o = -H; o <= H; ++o)
-            if (o != 0) K = fma(a.c1[o + H], F[c + o], K);
-        if (v > 0) {
-            const double* D = G + (3 + v) * W2;
-#pragma unroll
-            for (int o = -H; o <= H; ++o) K = fma(a.c2v[v - 1][o + H], D[c + o], K);
-        }
+        K = rns_flux_terms<H>(a, G, W2, v, c);
         if (v == 3) K = fma(-a.prm[4] * x, E[jl], K);
     }
     const double dt = a.dt;

@@ -205,7 +205,7 @@ __device__ __forceinline__ void rk_update(const StageArgs& a, const Cx& cx, int 
 // central stencils: advection-diffusion and reacting Navier-Stokes
 // ---------------------------------------------------------------------------
 // Reacting N-S in chain-rule form (Sec. 4) at own point j (window column c):
-// with m_f = sum_o c1_o f_{j+o} = -f_x and f_xx from the c2 taps,
+// with m_f = -f_x and f_xx by fx_d1 and fx_d2,
 //   K_rho  = -(rho_x u + rho u_x)
 //   K_rhou = -(rho_x u^2 + 2 rho u u_x) - p_x + 4/3 mu u_xx
 //   K_rhoE = -(u_x (rho E + p) + u ((rho E)_x + p_x)) + 4/3 mu (u_x^2 + u u_xx)
@@ -220,19 +220,11 @@ __device__ __forceinline__ void chain_point(const StageArgs& a, const Cx& cx, co
     double m[5];  // -d/dx of rho, u, p, rho E, Y
 #pragma unroll
     for (int q = 0; q < 5; ++q) {
-        double t = 0.0;
-#pragma unroll
-        for (int o = -H; o <= H; ++o)
-            if (o != 0) t = fma(a.c1[o + H], G[q * W2 + c + o], t);
-        m[q] = t;
+        m[q] = a.s1 * fx_d1<H>(G + q * W2 + c);
     }
-    double uxx = 0.0, Yxx = 0.0, Txx = 0.0;
-#pragma unroll
-    for (int o = -H; o <= H; ++o) {
-        uxx = fma(a.c2[o + H], G[1 * W2 + c + o], uxx);
-        Yxx = fma(a.c2[o + H], G[4 * W2 + c + o], Yxx);
-        Txx = fma(a.c2[o + H], G[5 * W2 + c + o], Txx);
-    }
+    const double uxx = a.s2 * fx_d2<H>(G + 1 * W2 + c);
+    const double Yxx = a.s2 * fx_d2<H>(G + 4 * W2 + c);
+    const double Txx = a.s2 * fx_d2<H>(G + 5 * W2 + c);
     const double rho = G[c], u = G[W2 + c], p = G[2 * W2 + c], rE = G[3 * W2 + c], Y = G[4 * W2 + c];
     const double T = G[5 * W2 + c];
     const double ru = rho * u;
@@ -300,15 +292,7 @@ __device__ __forceinline__ void central_window(const StageArgs& a, const Cx& cx,
             for (int o = -H; o <= H; ++o) K = fma(a.cm[o + H], G[c + o], K);
             x = G[c];
         } else {
-            const double* F = G + v * W2;
-#pragma unroll
-            for (int o = -H; o <= H; ++o)
-                if (o != 0) K = fma(a.c1[o + H], F[c + o], K);
-            if (v > 0) {
-                const double* D = G + (3 + v) * W2;  // u | energy diffusion / lambda | Y (constants in the taps)
-#pragma unroll
-                for (int o = -H; o <= H; ++o) K = fma(a.c2v[v - 1][o + H], D[c + o], K);
-            }
+            K = rns_flux_terms<H>(a, G, W2, v, c);
             if (v == 3) K = fma(-a.prm[4] * x, at_exp(-a.prm[5] * at_rcp3(G[7 * W2 + c])), K);
         }
         rk_update<RKS>(a, cx, v, j, chunk * a.Tw + jl, pe, K, x, in);
@@ -746,15 +730,7 @@ __global__ void __launch_bounds__(128) ring_recompute(const StageArgs a, const d
 #pragma unroll
                     for (int o = -H; o <= H; ++o) K = fma(a.cm[o + H], G[lane + o], K);
                 } else {
-                    const double* F = G + v * W;
-#pragma unroll
-                    for (int o = -H; o <= H; ++o)
-                        if (o != 0) K = fma(a.c1[o + H], F[lane + o], K);
-                    if (v > 0) {
-                        const double* D = G + (3 + v) * W;
-#pragma unroll
-                        for (int o = -H; o <= H; ++o) K = fma(a.c2v[v - 1][o + H], D[lane + o], K);
-                    }
+                    K = rns_flux_terms<H>(a, G, W, v, lane);
                     if (v == 3) K = fma(-a.prm[4] * x[v], at_exp(-a.prm[5] * at_rcp3(G[7 * W + lane])), K);
                 }
                 // the stage-(r+1) argument as rk_update forms it

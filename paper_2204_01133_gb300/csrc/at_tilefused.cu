@@ -189,15 +189,7 @@ __global__ void __launch_bounds__(256) tile_fused(const StageArgs a, const doubl
 #pragma unroll
                 for (int o = -H; o <= H; ++o) K = fma(a.cm[o + H], Gr[c + o], K);
             } else {
-                const double* F = Gr + v * RW;
-#pragma unroll
-                for (int o = -H; o <= H; ++o)
-                    if (o != 0) K = fma(a.c1[o + H], F[c + o], K);
-                if (v > 0) {
-                    const double* Dq = Gr + (3 + v) * RW;
-#pragma unroll
-                    for (int o = -H; o <= H; ++o) K = fma(a.c2v[v - 1][o + H], Dq[c + o], K);
-                }
+                K = rns_flux_terms<H>(a, Gr, RW, v, c);
                 if (v == 3) K = fma(-a.prm[4] * x, at_exp(-a.prm[5] * at_rcp3(Gr[7 * RW + c])), K);
             }
             double acc = AC[v * E + i];

@@ -1,0 +1,93 @@
+"""The integer arithmetic of csrc/at_fixed.cuh, compiled for the host: it is
+the device code's own source, so what holds here holds in the kernels."""
+import ctypes
+import math
+import os
+import subprocess
+from fractions import Fraction
+
+import numpy as np
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2204_01133_gb300", "csrc")
+D1 = {1: [-1, 0, 1], 2: [1, -8, 0, 8, -1], 3: [-1, 9, -45, 0, 45, -9, 1]}
+D2 = {1: [1, -2, 1], 2: [-1, 16, -30, 16, -1], 3: [2, -27, 270, -490, 270, -27, 2]}
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    d = tmp_path_factory.mktemp("fixed")
+    src = d / "f.cpp"
+    src.write_text('#include "at_fixed.cuh"\nextern "C" {\n' + "".join(
+        "double d%d_%d(const double* f) { return atk::fx_d%d<%d>(f + %d); }\n" % (k, h, k, h, h)
+        for k in (1, 2) for h in (1, 2, 3)) + "}\n")
+    so = str(d / "f.so")
+    subprocess.run(["g++", "-O2", "-std=c++17", "-ffp-contract=off", "-shared", "-fPIC", "-I", CSRC, str(src), "-o", so],
+                   check=True)
+    L = ctypes.CDLL(so)
+    for k in (1, 2):
+        for h in (1, 2, 3):
+            f = getattr(L, "d%d_%d" % (k, h))
+            f.restype, f.argtypes = ctypes.c_double, [ctypes.c_void_p]
+    return L
+
+
+def _call(lib, k, f):
+    f = np.ascontiguousarray(f, dtype=np.float64)
+    return getattr(lib, "d%d_%d" % (k, (len(f) - 1) // 2))(f.ctypes.data)
+
+
+def _rows(h, rng):
+    n = 2 * h + 1
+    x = np.arange(n)
+    for e in (-900, -30, 0, 30, 900):
+        s = math.ldexp(1.0, e)
+        yield s * (1.0 + 0.01 * np.sin(0.2 * x + rng.uniform(0, 6)))   # about the binade's edge
+        yield s * np.sin(0.15 * x + rng.uniform(0, 6))                 # through zero
+        yield s * rng.uniform(1.5, 1.9, n)                             # one exponent
+        yield s * rng.uniform(-1, 1, n)                                # no smoothness
+        yield s * np.ldexp(rng.uniform(-1, 1, n), rng.integers(-70, 70, n))  # no common scale
+        yield s * np.where(x % 2, 1.0, -1.0) * (2.0 - 2.0 ** -52)      # the largest differences there are
+
+
+@pytest.mark.parametrize("h", (1, 2, 3))
+@pytest.mark.parametrize("k", (1, 2))
+def test_differences_against_the_exact_sum(lib, k, h):
+    """Never worse than a chain of FMAs may be (2H + 1 roundings of partial
+    sums); and where second differences are moderate half an ulp of the
+    result plus the cut of every value."""
+    taps = (D1 if k == 1 else D2)[h]
+    weight = sum(abs(t) for t in taps)
+    rng = np.random.default_rng(3)
+    for _ in range(200):
+        for f in _rows(h, rng):
+            exact = sum((t * Fraction(float(v)) for t, v in zip(taps, f)), Fraction(0))
+            big = Fraction(float(np.abs(f).max()))
+            got = Fraction(_call(lib, k, f))
+            err = abs(got - exact)
+            assert err <= (2 * h + 1) * weight * big / 2 ** 53
+            smooth = k == 1 or h < 3 or float(np.abs(np.diff(f, 2)).max()) < 0.05 * float(big)
+            if smooth:
+                assert err <= abs(got) / 2 ** 53 + weight * big / 2 ** 55
+
+
+@pytest.mark.parametrize("h", (1, 2, 3))
+@pytest.mark.parametrize("k", (1, 2))
+def test_zeros_specials_and_the_ends_of_the_range(lib, k, h):
+    n = 2 * h + 1
+    assert _call(lib, k, np.where(np.arange(n) % 2, 0.0, -0.0)) == 0.0
+    assert _call(lib, k, np.full(n, 0.3)) == 0.0
+    for bad in (math.inf, -math.inf, math.nan):
+        f = np.ones(n)
+        f[h + 1] = bad
+        assert not math.isfinite(_call(lib, k, f))
+    tiny = np.zeros(n)
+    tiny[h + 1] = 5e-324
+    assert 0.0 <= abs(_call(lib, k, tiny)) < 1e-300
+    huge = np.full(n, 1e300)
+    huge[0] = 1.5e300
+    taps = (D1 if k == 1 else D2)[h]
+    assert _call(lib, k, huge) == pytest.approx(taps[0] * 0.5e300, rel=1e-12)
+    # overflow is an infinity, as in FP64
+    top = np.where(np.arange(n) < h, -1.7e308, 1.7e308)
+    assert math.isinf(_call(lib, 1, top))
