@@ -91,3 +91,62 @@ def test_zeros_specials_and_the_ends_of_the_range(lib, k, h):
     # overflow is an infinity, as in FP64
     top = np.where(np.arange(n) < h, -1.7e308, 1.7e308)
     assert math.isinf(_call(lib, 1, top))
+
+
+@pytest.fixture(scope="module")
+def soft(tmp_path_factory):
+    d = tmp_path_factory.mktemp("soft")
+    src = d / "s.cpp"
+    src.write_text('#include "at_fixed.cuh"\nextern "C" {\n'
+                   "uint64_t recip(uint64_t m) { return atk::fx_recip(m); }\n"
+                   "double terms(const double* p, const double* m) "
+                   "{ return atk::fx_weno_terms(p, p[3], p[4], m, m[3], m[4]); }\n}\n")
+    so = str(d / "s.so")
+    subprocess.run(["g++", "-O2", "-std=c++17", "-ffp-contract=off", "-shared", "-fPIC", "-I", CSRC, str(src), "-o", so],
+                   check=True)
+    L = ctypes.CDLL(so)
+    L.recip.restype, L.recip.argtypes = ctypes.c_uint64, [ctypes.c_uint64]
+    L.terms.restype, L.terms.argtypes = ctypes.c_double, [ctypes.c_void_p, ctypes.c_void_p]
+    return L
+
+
+def test_integer_reciprocal(soft):
+    rng = np.random.default_rng(5)
+    top = 1 << 63
+    ms = [top + i for i in range(600)] + [(1 << 64) - 1 - i for i in range(600)] + [top | 1 << i for i in range(63)]
+    ms += [top | int(v) for v in rng.integers(0, top, 20000, dtype=np.uint64)]
+    for m in ms:
+        r = soft.recip(m)
+        assert 1 << 62 <= r <= 1 << 63
+        assert abs(r * m - (1 << 126)) <= 1 << 66
+
+
+def _terms_exact(side):
+    d0, d1, d2, x, y = (Fraction(float(v)) for v in side)
+    e0, e1, e2 = d0 * d0, d1 * d1, d2 * d2
+    den = e1 * (3 * e0 + e2) + 6 * e0 * e2
+    return e1 * (2 * e2 * x + 3 * e0 * y) / den, e1 * (2 * e2 * abs(x) + 3 * e0 * abs(y)) / den
+
+
+def test_weno_terms_against_the_exact_quotients(soft):
+    """Seven products of 57 or more bits, three sums and a reciprocal: below
+    2 ulps of the terms' size; the FP64 sequence had 16 roundings of half an
+    ulp each."""
+    rng = np.random.default_rng(9)
+    for i in range(4000):
+        amp = 10.0 ** rng.uniform(-9, 4)
+        sides = []
+        for _ in range(2):
+            s0, s1, s2, a2 = amp * rng.uniform(-1, 1, 4) * 10.0 ** rng.uniform(-4 if i % 2 else 0, 0, 4)
+            a3 = a2 + s1
+            d = [s * (4 / 3 * s + a) + a * a + 1e-6 for s, a in ((s0, a2), (s1, a2), (s2, -a3))]
+            sides.append(np.array(d + [s0 - s1, s1 - s2]))
+        got = Fraction(soft.terms(sides[0].ctypes.data, sides[1].ctypes.data))
+        (tp, sp), (tm, sm) = map(_terms_exact, sides)
+        assert abs(got - tp - tm) <= 2 * (sp + sm) / 2 ** 53
+    flat = np.array([1e-12, 1e-12, 1e-12, 0.0, -0.0])
+    assert soft.terms(flat.ctypes.data, flat.ctypes.data) == 0.0
+    for bad in (np.zeros(5), np.array([1.0, math.nan, 1.0, 0.0, 0.0]), np.array([1.0, math.inf, 1.0, 0.0, 0.0])):
+        assert math.isnan(soft.terms(bad.ctypes.data, bad.ctypes.data))
+        if bad[1] != 0.0:
+            assert math.isnan(soft.terms(flat.ctypes.data, bad.ctypes.data))
