@@ -149,29 +149,37 @@ __device__ __forceinline__ int keff(const StageArgs& a, int64_t pe, int side)
 }
 
 // exp(x) by Tang's table-driven method (P. T. P. Tang, ACM TOMS 15(2), 1989)
-// with 256 table entries: x = (256 M + j) ln2/256 + r, |r| <= ln2/512, and
-// exp(x) = 2^M 2^(j/256) (1 + expm1(r)), expm1(r) by its Taylor polynomial of
-// degree 4 (the first omitted term, r^5/120, is below 4e-17).  The product
+// with 512 table entries: x = (512 M + j) ln2/512 + r, |r| <= ln2/1024, and
+// exp(x) = 2^M 2^(j/512) (1 + expm1(r)), expm1(r) by its Taylor polynomial of
+// degree 4 (the first omitted term, r^5/120, is below 2e-18).  The product
 // with 2^M is an integer add to the exponent field, exact while the result is
 // normal, which the fast path |x| < 512 guarantees (tested on the high word
 // with integer instructions); every other x (and Inf, NaN) goes to exp().
-// Nine FP64 instructions; within 2 ulp of the correctly rounded value.
+// What only needs FP32's 24 bits is done there (1 cycle against 64): the
+// nearest multiple (a slip by one at a tie leaves |r| a hair larger) and the
+// polynomial's terms above r^2/2, at most 6e-11 of the result, so that their
+// 3e-7 relative error is 2e-17.  Five FP64 instructions; within 2 ulp of the
+// correctly rounded value.
 __device__ __forceinline__ double at_exp(double x)
 {
-    static_assert(AT_EXP_N == 256, "the table has 256 entries");
-    if ((__double2hiint(x) & 0x7fffffff) >= 0x40800000) return exp(x);
-    const double shift = 0x1.8p52;                  // round to integer, result in the low word
-    const double t = fma(x, AT_EXP_INV_L, shift);
-    const int n = __double2loint(t);                // 256 M + j
-    const double nf = t - shift;
-    double r = fma(-nf, AT_EXP_L_HI, x);
-    r = fma(-nf, AT_EXP_L_LO, r);
-    double c = fma(r, 1.0 / 24.0, 1.0 / 6.0);
-    c = fma(c, r, 0.5);
-    const double em1 = fma(c, r * r, r);            // expm1(r)
-    const double tj = __ldg(&at_exp_tab[n & 255]);  // 2^(j/256)
+    static_assert(AT_EXP_N == 512, "the table has 512 entries");
+    const uint32_t hi = fx_hi(x), ah = hi & 0x7fffffffu;
+    if (ah >= 0x40800000u) return exp(x);
+    const float xf = fx_float(x);
+    const float t = fmaf(xf, (float)AT_EXP_INV_L, 12582912.0f);  // 1.5 2^23: the integer lands in the low bits
+    const int n = __float_as_int(t) - 0x4b400000;                // 512 M + j
+    const uint32_t nb = __float_as_uint(t - 12582912.0f);
+    // -n as a double (at most 19 bits: its low word is zero)
+    const double nd = fx_double(n == 0 ? 0u : (((nb & 0x7fffffffu) >> 3) + 0x38000000u) | (~nb & 0x80000000u), 0u);
+    double r = fma(nd, AT_EXP_L_HI, x);
+    r = fma(nd, AT_EXP_L_LO, r);
+    const float rf = fx_float(r);
+    const uint32_t qb = __float_as_uint(rf * rf * fmaf(rf, 1.0f / 24.0f, 1.0f / 6.0f));  // r^2/6 + r^3/24
+    const double w = fma(0.5, r, fx_double((qb >> 3) + 0x38000000u, qb << 29));
+    const double em1 = fma(r, w, r);                // expm1(r)
+    const double tj = __ldg(&at_exp_tab[n & 511]);  // 2^(j/512)
     const double e = fma(tj, em1, tj);
-    return __hiloint2double(__double2hiint(e) + ((n >> 8) << 20), __double2loint(e));
+    return fx_double(fx_hi(e) + ((uint32_t)(n >> 9) << 20), fx_lo(e));
 }
 
 // 1/x by two Newton-Raphson steps r <- r + r (1 - x r) from the hardware's
@@ -200,13 +208,35 @@ __device__ __forceinline__ double at_rcp(double x)
 // instruction fewer than at_rcp's two quadratic steps, within about an ulp
 // of 1/x for normal, finite, nonzero x (both are tested against 1/x).  The
 // kernels' reciprocals (densities, temperatures, pressures, WENO weight
-// sums) all use this one.
+// sums) outside the normal range go through this one (at_rcpi below).
 __device__ __forceinline__ double at_rcp3(double x)
 {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
     const double e = fma(-x, r, 1.0);
     return fma(r, fma(e, e, e), r);
+}
+
+// 1/x in integers (fx_rcp, at_fixed.cuh: correctly rounded up to 2^-60), the
+// kernels' reciprocals of densities, temperatures and pressures: about 75 issue
+// cycles beside the FP64 unit instead of three FP64 instructions, 192 cycles
+// of it.  Zero, Inf, NaN and the ends of the range go to at_rcp3.
+__device__ __forceinline__ double at_rcpi(double x)
+{
+    bool ok;
+    double r = fx_rcp(x, &ok);
+    if (!ok) r = at_rcp3(x);
+    return r;
+}
+
+// sqrt(x) in integers (fx_sqrt), about 105 issue cycles against some ten FP64
+// instructions; everything but positive normal numbers goes to sqrt().
+__device__ __forceinline__ double at_sqrt(double x)
+{
+    bool ok;
+    double r = fx_sqrt(x, &ok);
+    if (!ok) r = sqrt(x);
+    return r;
 }
 
 // Inf or NaN: exponent field all ones, tested on the high word with integer
@@ -275,9 +305,9 @@ struct Phys<RNS> {
     __device__ static void derive(const StageArgs& a, const double* Q, double* g)
     {
         const double gm1 = a.prm[0] - 1.0, qc = a.prm[6];
-        const double rinv = at_rcp3(Q[0]);
+        const double rinv = at_rcpi(Q[0]);
         const double u = Q[1] * rinv;
-        const double p = gm1 * (Q[2] - fma(0.5 * Q[1], u, qc * Q[3]));
+        const double p = gm1 * (Q[2] - fma(fx_half(Q[1]), u, qc * Q[3]));
         const double T = p * rinv;
         const double Y = Q[3] * rinv;
         g[0] = Q[1];
@@ -293,9 +323,9 @@ struct Phys<RNS> {
     __device__ static double temperature(const StageArgs& a, const double* Q)
     {
         const double gm1 = a.prm[0] - 1.0, qc = a.prm[6];
-        const double rinv = at_rcp3(Q[0]);
+        const double rinv = at_rcpi(Q[0]);
         const double u = Q[1] * rinv;
-        const double p = gm1 * (Q[2] - fma(0.5 * Q[1], u, qc * Q[3]));
+        const double p = gm1 * (Q[2] - fma(fx_half(Q[1]), u, qc * Q[3]));
         return p * rinv;
     }
 };
@@ -309,9 +339,9 @@ struct Phys<RNS_CHAIN> {
     __device__ static void derive(const StageArgs& a, const double* Q, double* g)
     {
         const double gm1 = a.prm[0] - 1.0, qc = a.prm[6];
-        const double rinv = at_rcp3(Q[0]);
+        const double rinv = at_rcpi(Q[0]);
         const double u = Q[1] * rinv;
-        const double p = gm1 * (Q[2] - fma(0.5 * Q[1], u, qc * Q[3]));
+        const double p = gm1 * (Q[2] - fma(fx_half(Q[1]), u, qc * Q[3]));
         g[0] = Q[0];
         g[1] = u;
         g[2] = p;
@@ -328,15 +358,15 @@ struct Phys<EULER> {
     static constexpr int NV = 4, ND = 8;
     __device__ static double pressure(const StageArgs& a, const double* Q, double u)
     {
-        return (a.prm[0] - 1.0) * (Q[2] - fma(0.5 * Q[1], u, a.prm[3] * Q[3]));
+        return (a.prm[0] - 1.0) * (Q[2] - fma(fx_half(Q[1]), u, a.prm[3] * Q[3]));
     }
     __device__ static void derive(const StageArgs& a, const double* Q, double* g)
     {
-        const double u = Q[1] * at_rcp3(Q[0]);
-        const double uh = 0.5 * u;
+        const double u = Q[1] * at_rcpi(Q[0]);
+        const double uh = fx_half(u);
         const double p = pressure(a, Q, u);
-        g[0] = 0.5 * Q[1];
-        g[1] = 0.5 * fma(Q[1], u, p);
+        g[0] = fx_half(Q[1]);
+        g[1] = fx_half(fma(Q[1], u, p));
         g[2] = uh * (Q[2] + p);  // = (u (E + p)) / 2 exactly
         g[3] = Q[3] * uh;
         g[4] = Q[0];
@@ -349,24 +379,24 @@ struct Phys<EULER> {
     // Arrhenius factor exp(-Ea rho / p) of the point's reaction source.
     // Halving is exact, so g[2] = (u/2)(E + p), g[3] = rho Y (u/2) and the half
     // speed |u/2| + sqrt(gamma p / (4 rho)) equal the halved products and the
-    // halved speed bit for bit (sqrt is correctly rounded).
+    // halved speed up to the root's rounding.
     template <bool ARR>
     __device__ static void derive_weno(const StageArgs& a, const double* Q, double* g, double& sph, double& arr)
     {
-        const double rinv = at_rcp3(Q[0]);
+        const double rinv = at_rcpi(Q[0]);
         const double u = Q[1] * rinv;
-        const double uh = 0.5 * u;
+        const double uh = fx_half(u);
         const double p = pressure(a, Q, u);
-        g[0] = 0.5 * Q[1];
-        g[1] = 0.5 * fma(Q[1], u, p);
+        g[0] = fx_half(Q[1]);
+        g[1] = fx_half(fma(Q[1], u, p));
         g[2] = uh * (Q[2] + p);
         g[3] = Q[3] * uh;
         g[4] = Q[0];
         g[5] = Q[1];
         g[6] = Q[2];
         g[7] = Q[3];
-        sph = fabs(uh) + sqrt((0.25 * a.prm[0]) * p * rinv);
-        if constexpr (ARR) arr = at_exp(-a.prm[2] * Q[0] * at_rcp3(p));
+        sph = fabs(uh) + at_sqrt((0.25 * a.prm[0]) * p * rinv);
+        if constexpr (ARR) arr = at_exp(-a.prm[2] * Q[0] * at_rcpi(p));
     }
 };
 

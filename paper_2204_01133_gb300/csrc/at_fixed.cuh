@@ -69,6 +69,20 @@ AT_HD double fx_double(uint32_t hi, uint32_t lo)
 AT_HD uint32_t fx_max(uint32_t a, uint32_t b) { return a > b ? a : b; }
 AT_HD uint32_t fx_min(uint32_t a, uint32_t b) { return a < b ? a : b; }
 
+// x cut to FP32 (|x| < 2^128; below 2^-127 zero or a subnormal)
+AT_HD float fx_float(double x)
+{
+    const uint32_t hi = fx_hi(x), ah = hi & 0x7fffffffu;
+    const uint32_t b = ((fx_max(ah, 0x38000000u) - 0x38000000u) << 3) | (fx_lo(x) >> 29) | (hi & 0x80000000u);
+    float f;
+#ifdef __CUDA_ARCH__
+    f = __uint_as_float(b);
+#else
+    std::memcpy(&f, &b, 4);
+#endif
+    return f;
+}
+
 AT_HD uint64_t fx_mulhi(uint64_t a, uint64_t b)
 {
 #ifdef __CUDA_ARCH__
@@ -325,6 +339,69 @@ AT_HD uint64_t fx_recip(uint64_t m)
     const int32_t e2 = (int32_t)(0x4000000000000000ll - (int64_t)fx_mulhi(m, r1));   // units of 2^-62
     const int64_t c2 = (int64_t)e2 * (int32_t)(r1 >> 33);                            // units of 2^-92
     return r1 + (uint64_t)(c2 >> 29);
+}
+
+// 1/x of a normal x whose reciprocal is normal, within half an ulp and 2^-60;
+// *ok is cleared for every other x
+AT_HD double fx_rcp(double x, bool* ok)
+{
+    const uint32_t hi = fx_hi(x), t = hi & FX_EXP;
+    *ok = t - 0x100000u < 0x7fc00000u;  // exponent fields 1..2044
+    const uint64_t m = ((uint64_t)((hi & 0xfffffu) | 0x100000u) << 32 | fx_lo(x)) << 11;
+    const uint64_t r = fx_recip(m);  // 2^62 (x nearly twice a power of two) .. 2^63 (a power of two)
+    const uint64_t v = (r >> 10) + ((r >> 9) & 1u);
+    return fx_double((uint32_t)(v >> 32) + (0x7fc00000u - t) + (hi & 0x80000000u), (uint32_t)v);
+}
+
+// sqrt(x) of a positive normal x, within half an ulp and 2^-58: two Newton
+// steps s <- s + (x - s^2) y / 2 in integers, y the hardware's approximate
+// FP32 reciprocal root; *ok is cleared for every other x
+AT_HD double fx_sqrt(double x, bool* ok)
+{
+    const uint32_t hi = fx_hi(x);
+    *ok = hi - 0x100000u < 0x7fe00000u;
+    // x = X 4^k, X in [1, 4) in units of 2^-62
+    const uint32_t odd = 1u - ((hi >> 20) & 1u);  // 1: the unbiased exponent is odd
+    const uint64_t X = ((uint64_t)((hi & 0xfffffu) | 0x100000u) << 32 | fx_lo(x)) << (10 + odd);
+    const uint32_t xh = (uint32_t)(X >> 32);
+    const uint32_t fb = (0x3f800000u + (odd << 23)) | ((hi << 3) & 0x7fffffu) | (fx_lo(x) >> 29);
+#ifdef __CUDA_ARCH__
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(__uint_as_float(fb)));
+    const uint32_t rb = __float_as_uint(r);
+#else
+    float f;
+    std::memcpy(&f, &fb, 4);
+    f = 1.0f / std::sqrt(f);
+    uint32_t rb;
+    std::memcpy(&rb, &f, 4);
+#endif
+    const uint32_t y = fx_seed(rb);                                                     // units of 2^-32
+    const uint64_t s1 = (uint64_t)xh * y + fx_mulhi32((uint32_t)X, y);                  // units of 2^-62
+    const int32_t e1 = (int32_t)((int64_t)((X >> 2) - fx_mulhi(s1, s1)) >> 12);         // units of 2^-48
+    const uint64_t s2 = s1 + (uint64_t)((int64_t)e1 * (int32_t)(y >> 1) >> 18);
+    const int32_t e2 = (int32_t)((X >> 2) - fx_mulhi(s2, s2));                          // units of 2^-60
+    const uint64_t s3 = s2 + (uint64_t)((int64_t)e2 * (int32_t)(y >> 1) >> 30);
+    const uint64_t v = (s3 >> 10) + ((s3 >> 9) & 1u);  // implicit bit at 52
+    return fx_double((uint32_t)(v >> 32) + ((((hi >> 20) + 1021u - odd) >> 1) << 20), (uint32_t)v);
+}
+
+// x / 2 (exact; what would be subnormal is zero)
+AT_HD double fx_half(double x)
+{
+    const uint32_t hi = fx_hi(x), t = hi & FX_EXP;
+    const bool in = t - 0x200000u < FX_EXP - 0x200000u;
+    const bool keep = t == FX_EXP;
+    return fx_double(in ? hi - 0x100000u : (keep ? hi : hi & 0x80000000u), in || keep ? fx_lo(x) : 0u);
+}
+
+// fmax of two numbers that are not negative (or not a number)
+AT_HD double fx_fmax(double a, double b)
+{
+    const uint64_t inf = (uint64_t)FX_EXP << 32;
+    const uint64_t ka = ((uint64_t)fx_hi(a) << 32 | fx_lo(a)) & 0x7fffffffffffffffull;
+    const uint64_t kb = ((uint64_t)fx_hi(b) << 32 | fx_lo(b)) & 0x7fffffffffffffffull;
+    return (kb > inf || (ka <= inf && ka >= kb)) ? a : b;
 }
 
 // the sum np/dp + nm/dm of the two reconstructions of a WENO edge (num and

@@ -233,7 +233,7 @@ __device__ __forceinline__ void chain_point(const StageArgs& a, const Cx& cx, co
     K[1] = fma(m[0] * u, u, fma(2.0 * ru, m[1], fma(a.k0, uxx, m[2])));
     K[2] = fma(m[1], rE + p, fma(u, m[3] + m[2], fma(a.k0, fma(m[1], m[1], u * uxx), fma(a.k2, Txx, a.prm[6] * a.k3 * Yxx))));
     const double x3 = cx.X[3 * a.N + j];
-    K[3] = fma(m[0] * u, Y, fma(rho * m[1], Y, fma(ru, m[4], fma(a.k3, Yxx, -a.prm[4] * x3 * at_exp(-a.prm[5] * at_rcp3(T))))));
+    K[3] = fma(m[0] * u, Y, fma(rho * m[1], Y, fma(ru, m[4], fma(a.k3, Yxx, -a.prm[4] * x3 * at_exp(-a.prm[5] * at_rcpi(T))))));
 #pragma unroll
     for (int v = 0; v < 4; ++v) {
         const double x = v == 3 ? x3 : cx.X[v * a.N + j];
@@ -293,7 +293,7 @@ __device__ __forceinline__ void central_window(const StageArgs& a, const Cx& cx,
             x = G[c];
         } else {
             K = rns_flux_terms<H>(a, G, W2, v, c);
-            if (v == 3) K = fma(-a.prm[4] * x, at_exp(-a.prm[5] * at_rcp3(G[7 * W2 + c])), K);
+            if (v == 3) K = fma(-a.prm[4] * x, at_exp(-a.prm[5] * at_rcpi(G[7 * W2 + c])), K);
         }
         rk_update<RKS>(a, cx, v, j, chunk * a.Tw + jl, pe, K, x, in);
     }
@@ -399,7 +399,7 @@ __device__ __forceinline__ void weno_window(const StageArgs& a, const Cx& cx, in
     fill_window<PDE, true>(a, cx, G, SP, HS, pe, chunk, t0, W2, threadIdx.x, blockDim.x, ARR);
     __syncthreads();
     for (int e = threadIdx.x; e < E; e += blockDim.x)
-        LAM[e] = fmax(SP[e - 1 + H], SP[e + H]);  // half the edge's local wave speed (SP: half speeds)
+        LAM[e] = fx_fmax(SP[e - 1 + H], SP[e + H]);  // half the edge's local wave speed (SP: half speeds)
     for (int it = threadIdx.x; it < ND * (W2 - 1); it += blockDim.x) {
         const int d = it / (W2 - 1);
         const int j = 1 + it - d * (W2 - 1);
@@ -464,7 +464,7 @@ __device__ __forceinline__ double weno5_interp(double f0, double f1, double f2, 
     const double num = e1 * fma(3.0 * e2, s0 - s1, (5.0 * e0) * (s1 - s2));
     const double den = fma(e1, fma(8.0, e2, 40.0 * e0), 80.0 * (e0 * e2));
     const double u1 = fma(-0.125, f1, fma(0.75, f2, 0.375 * f3));
-    return fma(num, at_rcp3(den), u1);
+    return fma(num, at_rcpi(den), u1);
 }
 
 // A window of Tw points with a halo of H = 4: the edge values F of the
@@ -493,7 +493,7 @@ __device__ __forceinline__ void weno_interp_window(const StageArgs& a, const Cx&
     fill_window<PDE, true>(a, cx, G, SP, HS, pe, chunk, t0, W2, threadIdx.x, blockDim.x, ARR);
     __syncthreads();
     for (int t = threadIdx.x; t < E; t += blockDim.x)
-        LAM[t] = fmax(SP[t + 2], SP[t + 3]);  // SP holds half speeds
+        LAM[t] = fx_fmax(SP[t + 2], SP[t + 3]);  // SP holds half speeds
     __syncthreads();
     const double eps4 = 4.0 * ((PDE == EULER) ? a.prm[4] : a.prm[1]);
     const int items = NV * 2 * E;
@@ -731,7 +731,7 @@ __global__ void __launch_bounds__(128) ring_recompute(const StageArgs a, const d
                     for (int o = -H; o <= H; ++o) K = fma(a.cm[o + H], G[lane + o], K);
                 } else {
                     K = rns_flux_terms<H>(a, G, W, v, lane);
-                    if (v == 3) K = fma(-a.prm[4] * x[v], at_exp(-a.prm[5] * at_rcp3(G[7 * W + lane])), K);
+                    if (v == 3) K = fma(-a.prm[4] * x[v], at_exp(-a.prm[5] * at_rcpi(G[7 * W + lane])), K);
                 }
                 // the stage-(r+1) argument as rk_update forms it
                 if (RK == RK4) y[v] = fma(r == 2 ? a.dt : a.hdt, K, un[v]);

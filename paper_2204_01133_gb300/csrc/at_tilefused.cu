@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(256) tile_fused(const StageArgs a, const doubl
                 for (int o = -H; o <= H; ++o) K = fma(a.cm[o + H], Gr[c + o], K);
             } else {
                 K = rns_flux_terms<H>(a, Gr, RW, v, c);
-                if (v == 3) K = fma(-a.prm[4] * x, at_exp(-a.prm[5] * at_rcp3(Gr[7 * RW + c])), K);
+                if (v == 3) K = fma(-a.prm[4] * x, at_exp(-a.prm[5] * at_rcpi(Gr[7 * RW + c])), K);
             }
             double acc = AC[v * E + i];
             const double y = fused_update<RK>(a, s, K, x, UN[v * E + i], acc);
@@ -400,7 +400,7 @@ __global__ void __launch_bounds__(256) tile_fused_weno(const StageArgs a, const 
             const int r = t < ne[0] ? 0 : (t < ne[0] + ne[1] ? 1 : 2);
             const int e = t - (r == 0 ? 0 : (r == 1 ? ne[0] : ne[0] + ne[1]));
             const int c = H + ka[r] + e - row_lo(r);  // column of the point right of the edge
-            LAM[roff(r) + c] = fmax(SP[roff(r) + c - 1], SP[roff(r) + c]);  // SP holds half speeds
+            LAM[roff(r) + c] = fx_fmax(SP[roff(r) + c - 1], SP[roff(r) + c]);  // SP holds half speeds
         }
         __syncthreads();
         const double eps = (PDE == EULER) ? a.prm[4] : a.prm[1];

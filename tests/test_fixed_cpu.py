@@ -100,14 +100,50 @@ def soft(tmp_path_factory):
     src.write_text('#include "at_fixed.cuh"\nextern "C" {\n'
                    "uint64_t recip(uint64_t m) { return atk::fx_recip(m); }\n"
                    "double terms(const double* p, const double* m) "
-                   "{ return atk::fx_weno_terms(p, p[3], p[4], m, m[3], m[4]); }\n}\n")
+                   "{ return atk::fx_weno_terms(p, p[3], p[4], m, m[3], m[4]); }\n"
+                   "int one(int f, double x, double* y) { bool ok = true; "
+                   "*y = f == 0 ? atk::fx_rcp(x, &ok) : f == 1 ? atk::fx_sqrt(x, &ok) : atk::fx_half(x); return ok; }\n"
+                   "double most(double a, double b) { return atk::fx_fmax(a, b); }\n}\n")
     so = str(d / "s.so")
     subprocess.run(["g++", "-O2", "-std=c++17", "-ffp-contract=off", "-shared", "-fPIC", "-I", CSRC, str(src), "-o", so],
                    check=True)
     L = ctypes.CDLL(so)
     L.recip.restype, L.recip.argtypes = ctypes.c_uint64, [ctypes.c_uint64]
     L.terms.restype, L.terms.argtypes = ctypes.c_double, [ctypes.c_void_p, ctypes.c_void_p]
+    L.one.argtypes = [ctypes.c_int, ctypes.c_double, ctypes.c_void_p]
+    L.most.restype, L.most.argtypes = ctypes.c_double, [ctypes.c_double, ctypes.c_double]
     return L
+
+
+def _one(L, f, x):
+    y = ctypes.c_double()
+    return bool(L.one(f, x, ctypes.byref(y))), y.value
+
+
+def test_reciprocal_root_half_and_maximum(soft):
+    """Half an ulp and 2^-58 relative, that is 0.52 ulp; everything outside
+    the normal range is handed back."""
+    rng = np.random.default_rng(6)
+    xs = [math.ldexp(float(m), int(e)) for m, e in zip(rng.uniform(1, 2, 4000), rng.integers(-1020, 1020, 4000))]
+    for e in (-1, 0, 1, 2):  # both sides of a power of two, of both parities
+        xs += [math.ldexp(1.0, e) * (1 + i * 2.0 ** -52) for i in range(-40, 41)]
+    for x in xs:
+        ok, r = _one(soft, 0, -x)
+        assert ok and abs(Fraction(r) + 1 / Fraction(x)) <= Fraction(math.ulp(r)) * 52 / 100
+        ok, r = _one(soft, 1, x)
+        lo, hi = Fraction(r) - Fraction(math.ulp(r)) * 52 / 100, Fraction(r) + Fraction(math.ulp(r)) * 52 / 100
+        assert ok and lo * lo <= Fraction(x) <= hi * hi
+        assert _one(soft, 2, x)[1] == 0.5 * x
+    for x in (0.0, -0.0, math.inf, -math.inf, math.nan, 1e-310):
+        assert not _one(soft, 0, x)[0] and not _one(soft, 1, x)[0]
+        h = _one(soft, 2, x)[1]
+        assert h == (0.0 if abs(x) < 1 else 0.5 * x) or h != h
+    assert not _one(soft, 1, -1.0)[0] and not _one(soft, 0, 1.7e308)[0]
+    for a in (0.0, 1.0, 2.0, math.inf, math.nan):
+        for b in (0.0, 1.0, 2.0, math.inf, math.nan):
+            want = b if a != a else a if b != b else max(a, b)
+            got = soft.most(a, b)
+            assert got == want or (got != got and want != want)
 
 
 def test_integer_reciprocal(soft):
