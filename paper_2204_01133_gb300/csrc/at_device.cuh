@@ -47,7 +47,7 @@ struct StageArgs {
     double s2;                                // 1 / (D2 dx^2): scales fx_d2
     double cm[2 * AT_HMAX + 1];               // merged advection-diffusion taps
     double prm[16];                           // physics constants (see at.h)
-    double k0, k1, k2, k3;                    // derived physics constants
+    double k0, k1, k2, k3;                    // derived physics constants (WENO: k0 = 1/dx, k1 = 3 eps)
     // reacting flow: the diffusion rows are u, the energy term over lambda and
     // Y, with the constants in the scale: s2v[v-1] = s2 times (4/3) mu,
     // lambda, lambda / (cp Le) for v = 1, 2, 3; kd1 = k1 / k2, kd3 = qc k3 / k2
@@ -489,81 +489,57 @@ __device__ __forceinline__ int64_t place_rank(const StageArgs& a)
 }
 
 // ---------------------------------------------------------------------------
-// WENO5-JS reconstruction at the right edge of f[2] from f[0..4]
-// (candidates of Eq. atRecon at k = 0, ideal weights {1/10, 3/5, 3/10},
-// indicators of Eq. betaS, weights of Eq. omg with power 2), taken from the
-// first differences a_k = f[k] - f[k-1] (k = 1..4), and arranged for few
-// FP64 instructions without changing the mathematics:
-//  * the second differences s_i (centred on f[i+1]) are s_0 = a_2 - a_1,
-//    s_1 = a_3 - a_2, s_2 = a_4 - a_3, and the first-difference terms of the
-//    indicators r_0 = f0 - 4 f1 + 3 f2 = s_0 + 2 a_2, r_1 = f1 - f3 =
-//    -(a_2 + a_3) = -(s_1 + 2 a_2), r_2 = 3 f2 - 4 f3 + f4 = s_2 - 2 a_3;
-//    then beta_i = (13 s_i^2 + 3 r_i^2) / 12, and with r_i expanded
+// The LLF-split WENO5-JS flux at the edge left of column c of a row: the
+// reconstruction of f+ = C + hl Q from columns c-3..c+1 plus that of
+// f- = C - hl Q from columns c+2..c-2 (mirrored), hl half the edge's wave
+// speed (Eq. Csplit).  One reconstruction, at the right edge of f[2] from
+// f[0..4] (candidates of Eq. atRecon at k = 0, ideal weights {1/10, 3/5, 3/10},
+// indicators of Eq. betaS, weights of Eq. omg with power 2), is taken from
+// the first differences a_k = f[k] - f[k-1] (k = 1..4):
+//  * with the second differences s_i (centred on f[i+1]) s_0 = a_2 - a_1,
+//    s_1 = a_3 - a_2, s_2 = a_4 - a_3 and the first-difference terms
+//    r_0 = f0 - 4 f1 + 3 f2 = s_0 + 2 a_2, r_1 = f1 - f3 = -(s_1 + 2 a_2),
+//    r_2 = 3 f2 - 4 f3 + f4 = s_2 - 2 a_3 the indicators
+//    beta_i = (13 s_i^2 + 3 r_i^2) / 12 give
 //      D_0 = eps + beta_0 = s_0 ((4/3) s_0 + a_2) + a_2^2 + eps,
 //      D_1 = eps + beta_1 = s_1 ((4/3) s_1 + a_2) + a_2^2 + eps,
-//      D_2 = eps + beta_2 = s_2 ((4/3) s_2 - a_3) + a_3^2 + eps
-//    (each a positive definite form in (s_i, a), so the sum does not
-//    cancel), D_0 and D_1 sharing a_2^2 + eps;
+//      D_2 = eps + beta_2 = s_2 ((4/3) s_2 - a_3) + a_3^2 + eps;
 //  * the middle candidate p_1 = (-f1 + 5 f2 + 2 f3) / 6 = f2 + a_2/6 + a_3/3,
 //    and the others differ from it by third differences,
 //    p_0 - p_1 = (s_0 - s_1) / 3 and p_2 - p_1 = (s_1 - s_2) / 6, so
 //    sum omega_i p_i = p_1 + omega_0 (p_0 - p_1) + omega_2 (p_2 - p_1);
 //  * alpha_i ~ gamma_i / D_i^2 times the common factor D_0^2 D_1^2 D_2^2, and
 //    numerator and denominator scaled by 10 (ideal weights 1 : 6 : 3); with
-//    E_i = D_i^2, A = 3 E_0 and B = 2 E_2,
-//      num = E_1 (B (s_0 - s_1) + A (s_1 - s_2))   (6 times the corrections'
-//            numerator E_1 (E_2 (s_0 - s_1) / 3 + E_0 (s_1 - s_2) / 2)),
-//      den = E_1 (A + E_2) + A B                   (= E_1 (3 E_0 + E_2) + 6 E_0 E_2),
-//    so the reconstruction is p_1 + num / (6 den).
-// Returned: the D_i, x = s_0 - s_1, y = s_1 - s_2 and s_1; num and den of both
-// signs, and the quotients, are formed in integers (fx_weno_terms,
-// at_fixed.cuh): 30 of the 66 FP64 instructions of an edge and variable, 64
-// cycles each, become about 800 issue cycles of integer work beside the rest.
-// Measured on GB300: the detonation of 2^23 points 16.3 -> 11.1 ms per RK3
-// step, of 61,440 points 168 -> 123 us; within 1.4 ulps of the exact terms
-// where the FP64 sequence was within 5.7.
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ void weno5d(double a1, double a2, double a3, double a4, double eps, double* d, double& x,
-                                       double& y, double& s1)
-{
-    const double s0 = a2 - a1;
-    s1 = a3 - a2;
-    const double s2 = a4 - a3;
-    const double t2 = fma(a2, a2, eps);
-    d[0] = fma(s0, fma(4.0 / 3.0, s0, a2), t2);
-    d[1] = fma(s1, fma(4.0 / 3.0, s1, a2), t2);
-    d[2] = fma(s2, fma(4.0 / 3.0, s2, -a3), fma(a3, a3, eps));
-    x = s0 - s1;
-    y = s1 - s2;
-}
-
-// The LLF-split WENO5 flux at the edge left of column c of a row: the
-// reconstruction of f+ = C + hl Q from columns c-3..c+1 plus that of
-// f- = C - hl Q from columns c+2..c-2 (mirrored), hl half the edge's wave
-// speed (Eq. Csplit).  The split fluxes' first differences are those of C
-// and Q combined, P(j) = dC(j) + hl dQ(j) and M(j) = hl dQ(j) - dC(j) with
+//    E_i = D_i^2 and A = 3 E_0, den = E_1 (A + E_2) + 2 A E_2,
+//      p = p_1 + (2 E_1 E_2 / den (s_0 - s_1) + E_1 A / den (s_1 - s_2)) / 6.
+// The split fluxes' first differences are those of C and Q combined,
+// P(j) = hl dQ(j) + dC(j) and M(j) = hl dQ(j) - dC(j) with
 // dC(j) = C[j] - C[j-1], so they come from the rows' own first differences,
 // formed once per column and shared by every edge and both signs; dC(j),
-// dQ(j) are callables returning them.
-// The two middle candidates add up to a centred value: p+ = f+(c-1) +
-// P(c-1)/6 + P(c)/3 and p- = f-(c) + M(c+1)/6 + M(c)/3, and with
-// f+(c-1) + f-(c) = C[c-1] + C[c] - hl dQ(c) and P(c) + M(c) = 2 hl dQ(c),
+// dQ(j) are callables returning them.  The two middle candidates add up to a
+// centred value: p+ = f+(c-1) + P(c-1)/6 + P(c)/3 and p- = f-(c) + M(c+1)/6 +
+// M(c)/3, and with f+(c-1) + f-(c) = C[c-1] + C[c] - hl dQ(c) and
+// P(c) + M(c) = 2 hl dQ(c),
 //   p+ + p- = C[c-1] + C[c] + (P(c-1) - P(c) + M(c+1) - M(c)) / 6
 //           = C[c-1] + C[c] - (s1+ + s1-) / 6,
 // s1+ = P(c) - P(c-1) and s1- = M(c) - M(c+1) being the two
-// reconstructions' middle second differences.  The 1/6 of the corrections
-// num+ / (6 den+) + num- / (6 den-) and of the second differences is applied
-// once.
+// reconstructions' middle second differences.
+//
+// What bounds it: an FP64 warp instruction holds a sub-partition's FP64 unit
+// for 64 cycles, and the whole flux took 66 of them.  Seven are left: the
+// products hl dQ and the last sum.  Everything between is integer arithmetic
+// on the aligned differences (fx_weno_sum, at_fixed.cuh).
+// ---------------------------------------------------------------------------
 template <class DC, class DQ>
-__device__ __forceinline__ double weno_flux(const double* C, DC dC, DQ dQ, int c, double hl, double eps)
+__device__ __forceinline__ double weno_flux(const StageArgs& a, const double* C, DC dC, DQ dQ, int c, double hl)
 {
-    double dp[3], xp, yp, s1p, dm[3], xm, ym, s1m;
-    weno5d(fma(hl, dQ(c - 2), dC(c - 2)), fma(hl, dQ(c - 1), dC(c - 1)), fma(hl, dQ(c), dC(c)),
-           fma(hl, dQ(c + 1), dC(c + 1)), eps, dp, xp, yp, s1p);
-    // mirrored: a_k of f- is M at columns c+2, c+1, c, c-1
-    weno5d(fma(hl, dQ(c + 2), -dC(c + 2)), fma(hl, dQ(c + 1), -dC(c + 1)), fma(hl, dQ(c), -dC(c)),
-           fma(hl, dQ(c - 1), -dC(c - 1)), eps, dm, xm, ym, s1m);
-    return fma(1.0 / 6.0, fx_weno_terms(dp, xp, yp, dm, xm, ym) - (s1p + s1m), C[c - 1] + C[c]);
+    double d[5], q[5];
+#pragma unroll
+    for (int j = 0; j < 5; ++j) {
+        d[j] = dC(c - 2 + j);
+        q[j] = hl * dQ(c - 2 + j);
+    }
+    return fma(1.0 / 6.0, fx_weno_sum(d, q, fx_unpack(a.k1)), C[c - 1] + C[c]);
 }
 
 // ---------------------------------------------------------------------------

@@ -403,7 +403,6 @@ __global__ void __launch_bounds__(256) tile_fused_weno(const StageArgs a, const 
             LAM[roff(r) + c] = fx_fmax(SP[roff(r) + c - 1], SP[roff(r) + c]);  // SP holds half speeds
         }
         __syncthreads();
-        const double eps = (PDE == EULER) ? a.prm[4] : a.prm[1];
         const int nrec = NV * (ne[0] + ne[1] + ne[2]);
         for (int it = threadIdx.x; it < nrec; it += blockDim.x) {
             const int t = it % (ne[0] + ne[1] + ne[2]);
@@ -416,8 +415,8 @@ __global__ void __launch_bounds__(256) tile_fused_weno(const StageArgs a, const 
             // the rows' first differences formed where they are used: the same
             // operations, so the same values, as the per-stage kernels' stored ones
             REC[NV * roff(r) + v * rstride(r) + c] =
-                weno_flux(Cr, [&](int j) { return Cr[j] - Cr[j - 1]; }, [&](int j) { return Qr[j] - Qr[j - 1]; }, c,
-                          LAM[roff(r) + c], eps);
+                weno_flux(a, Cr, [&](int j) { return Cr[j] - Cr[j - 1]; }, [&](int j) { return Qr[j] - Qr[j - 1]; },
+                          c, LAM[roff(r) + c]);
         }
         __syncthreads();
         const double rdx = a.k0;

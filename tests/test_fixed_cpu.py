@@ -99,8 +99,8 @@ def soft(tmp_path_factory):
     src = d / "s.cpp"
     src.write_text('#include "at_fixed.cuh"\nextern "C" {\n'
                    "uint64_t recip(uint64_t m) { return atk::fx_recip(m); }\n"
-                   "double terms(const double* p, const double* m) "
-                   "{ return atk::fx_weno_terms(p, p[3], p[4], m, m[3], m[4]); }\n"
+                   "double weno(const double* c, const double* q, double eps3) "
+                   "{ return atk::fx_weno_sum(c, q, atk::fx_unpack(eps3)); }\n"
                    "int one(int f, double x, double* y) { bool ok = true; "
                    "*y = f == 0 ? atk::fx_rcp(x, &ok) : f == 1 ? atk::fx_sqrt(x, &ok) : atk::fx_half(x); return ok; }\n"
                    "double most(double a, double b) { return atk::fx_fmax(a, b); }\n}\n")
@@ -109,7 +109,7 @@ def soft(tmp_path_factory):
                    check=True)
     L = ctypes.CDLL(so)
     L.recip.restype, L.recip.argtypes = ctypes.c_uint64, [ctypes.c_uint64]
-    L.terms.restype, L.terms.argtypes = ctypes.c_double, [ctypes.c_void_p, ctypes.c_void_p]
+    L.weno.restype, L.weno.argtypes = ctypes.c_double, [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_double]
     L.one.argtypes = [ctypes.c_int, ctypes.c_double, ctypes.c_void_p]
     L.most.restype, L.most.argtypes = ctypes.c_double, [ctypes.c_double, ctypes.c_double]
     return L
@@ -157,32 +157,51 @@ def test_integer_reciprocal(soft):
         assert abs(r * m - (1 << 126)) <= 1 << 66
 
 
-def _terms_exact(side):
-    d0, d1, d2, x, y = (Fraction(float(v)) for v in side)
-    e0, e1, e2 = d0 * d0, d1 * d1, d2 * d2
-    den = e1 * (3 * e0 + e2) + 6 * e0 * e2
-    return e1 * (2 * e2 * x + 3 * e0 * y) / den, e1 * (2 * e2 * abs(x) + 3 * e0 * abs(y)) / den
+def _weno_exact(c, q, eps):
+    """six times (the weighted corrections) minus the middle second differences, both signs, exactly"""
+    c, q = [Fraction(float(v)) for v in c], [Fraction(float(v)) for v in q]
+    total = Fraction(0)
+    for a in ([q[j] + c[j] for j in (0, 1, 2, 3)], [q[j] - c[j] for j in (4, 3, 2, 1)]):
+        s0, s1, s2 = a[1] - a[0], a[2] - a[1], a[3] - a[2]
+        e = Fraction(eps)
+        d0 = s0 * (Fraction(4, 3) * s0 + a[1]) + a[1] ** 2 + e
+        d1 = s1 * (Fraction(4, 3) * s1 + a[1]) + a[1] ** 2 + e
+        d2 = s2 * (Fraction(4, 3) * s2 - a[2]) + a[2] ** 2 + e
+        e0, e1, e2 = d0 ** 2, d1 ** 2, d2 ** 2
+        den = e1 * (3 * e0 + e2) + 6 * e0 * e2
+        total += (2 * e1 * e2 * (s0 - s1) + 3 * e0 * e1 * (s1 - s2)) / den - s1
+    return total
 
 
-def test_weno_terms_against_the_exact_quotients(soft):
-    """Seven products of 57 or more bits, three sums and a reciprocal: below
-    2 ulps of the terms' size; the FP64 sequence had 16 roundings of half an
-    ulp each."""
+def test_weno_sum_against_the_exact_weights(soft):
+    """Every difference is cut below 2^-57 of the largest; a cut of one unit
+    moves the sum by at most some tens of units (four taps of up to 8 with
+    weights up to 2, and the weights' own response, of the same size), two
+    signs: 32 2^-53 of the largest difference bounds it with room."""
     rng = np.random.default_rng(9)
     for i in range(4000):
-        amp = 10.0 ** rng.uniform(-9, 4)
-        sides = []
-        for _ in range(2):
-            s0, s1, s2, a2 = amp * rng.uniform(-1, 1, 4) * 10.0 ** rng.uniform(-4 if i % 2 else 0, 0, 4)
-            a3 = a2 + s1
-            d = [s * (4 / 3 * s + a) + a * a + 1e-6 for s, a in ((s0, a2), (s1, a2), (s2, -a3))]
-            sides.append(np.array(d + [s0 - s1, s1 - s2]))
-        got = Fraction(soft.terms(sides[0].ctypes.data, sides[1].ctypes.data))
-        (tp, sp), (tm, sm) = map(_terms_exact, sides)
-        assert abs(got - tp - tm) <= 2 * (sp + sm) / 2 ** 53
-    flat = np.array([1e-12, 1e-12, 1e-12, 0.0, -0.0])
-    assert soft.terms(flat.ctypes.data, flat.ctypes.data) == 0.0
-    for bad in (np.zeros(5), np.array([1.0, math.nan, 1.0, 0.0, 0.0]), np.array([1.0, math.inf, 1.0, 0.0, 0.0])):
-        assert math.isnan(soft.terms(bad.ctypes.data, bad.ctypes.data))
-        if bad[1] != 0.0:
-            assert math.isnan(soft.terms(flat.ctypes.data, bad.ctypes.data))
+        amp = 10.0 ** rng.uniform(-12, 6)
+        kind = i % 4
+        c, q = amp * rng.uniform(-1, 1, 5), amp * rng.uniform(-1, 1, 5)
+        if kind == 1:    # smooth
+            c, q = amp * (1 + 0.1 * np.sin(0.2 * np.arange(5) + rng.uniform(0, 6))), 0.7 * amp * np.cos(0.1 * np.arange(5))
+        elif kind == 2:  # a front at one end, quiet at the other
+            c, q = c * 10.0 ** -np.arange(0, 15, 3.0), q * 10.0 ** -np.arange(0, 15, 3.0)
+        elif kind == 3:  # one family only
+            q = np.zeros(5)
+        got = Fraction(soft.weno(c.ctypes.data, q.ctypes.data, 3e-6))
+        big = Fraction(float(max(np.abs(c).max(), np.abs(q).max())))
+        assert abs(got - _weno_exact(c, q, 1e-6)) <= 32 * big / 2 ** 53
+    zero = np.zeros(5)
+    assert soft.weno(zero.ctypes.data, zero.ctypes.data, 3e-6) == 0.0
+    assert math.isnan(soft.weno(zero.ctypes.data, zero.ctypes.data, 0.0))
+    for bad in (math.nan, math.inf, -math.inf):
+        for j in range(5):
+            f = np.ones(5)
+            f[j] = bad
+            assert math.isnan(soft.weno(f.ctypes.data, zero.ctypes.data, 3e-6))
+            assert math.isnan(soft.weno(zero.ctypes.data, f.ctypes.data, 3e-6))
+    for amp in (1e-300, 1e250):  # no intermediate leaves its range
+        f = amp * np.array([1.0, -2.0, 3.0, 0.5, 1.0])
+        big = Fraction(3 * amp)
+        assert abs(Fraction(soft.weno(f.ctypes.data, zero.ctypes.data, 3e-6)) - _weno_exact(f, zero, 1e-6)) <= 32 * big / 2 ** 53
