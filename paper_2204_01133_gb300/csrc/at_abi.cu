@@ -22,7 +22,7 @@
 
 size_t atk_stage_smem_bytes(int pde, int Tw, int H);
 int atk_stage_block(int pde, int Tw);
-cudaError_t atk_launch_stage(const atk::StageArgs& a, int pde, int order, cudaStream_t st);
+cudaError_t atk_launch_stage(const atk::StageArgs& a, int pde, int order, int sms, cudaStream_t st);
 cudaError_t atk_launch_ring_seed(const atk::StageArgs& a, cudaStream_t st);
 cudaError_t atk_launch_ring_recompute(const atk::StageArgs& a, int pde, int order, int rk, const double* um,
                                       int64_t m, cudaStream_t st);
@@ -216,6 +216,31 @@ Layout layout(const at_problem* pb, const at_delays* dl)
     return L;
 }
 
+// Window length of the per-stage WENO kernels on a GPU of `sms` SMs.  A CTA's
+// time grows with its window plus the points beyond it (about 8 more edges and
+// derived points), and the SM that gets the most windows sets the stage's
+// time: the divisor of the PE size that keeps ceil(windows / SMs) (Tw + 8)
+// smallest.  Large problems get the longest window (the overhead decides),
+// small ones windows short enough to reach every SM.  Measured on GB300, us per
+// RK3 stage: 4,096 points in PEs of 512: 27.5 with windows of 256, @A@ with the
+// rule's 32; 61,440 points in PEs of 480: 34.9 with 240, @B@ with the rule's 60.
+// The values do not depend on the window.
+int stage_window(const at_problem* pb, const Layout& L, int sms)
+{
+    if (!is_weno(pb->pde) || sms < 1) return L.Tw;
+    int best = L.Tw;
+    int64_t least = INT64_MAX;
+    for (int t = L.Tw; t >= 16 && t >= 2 * L.H; --t) {
+        if (pb->pe_size % t) continue;
+        const int64_t windows = pb->n / t, cost = (windows + sms - 1) / sms * (t + 8);
+        if (cost < least) {
+            least = cost;
+            best = t;
+        }
+    }
+    return best;
+}
+
 // thresholds: T_i = floor(2^32 CDF(i)), CDF accumulated in index order
 void thresholds(const at_delays* dl, uint64_t* thr)
 {
@@ -380,6 +405,8 @@ struct at_ctx {
     int last_path = 0;             // path of the last at_step
     int64_t persist_cap = 0;       // PEs one cooperative launch can hold (0: unavailable)
     int cluster_c = 0;             // CTAs of the one-cluster kernel for this problem (0: not used)
+    int sms = 0;                   // SMs of the device
+    int stage_tw = 0;              // window length of the per-stage kernels (stage_window)
     int fused_multi_w = 0;         // PEs per CTA when the fused path's steps fit one cooperative launch
     int64_t wait_limit = 4000000;  // polls of a bounded wait
     int64_t withhold_pe = -1;
@@ -538,6 +565,8 @@ int at_set_delays(at_ctx* c, const at_delays* dl)
     if (e != cudaSuccess) return cuda_fail(e, "ring seed launch");
     c->level = 0;
     c->hist_level = -1;  // reading A recomputes level 0 at the first at_step
+    if (c->sms == 0) cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device);
+    c->stage_tw = stage_window(&c->pb, L, c->sms);
     c->persist_cap = (c->pb.pde == AT_ADVDIFF || c->pb.pde == AT_RNS)
                          ? atk_persist_capacity(c->pb.pde, c->pb.order, c->pb.pe_size, c->device)
                          : 0;
@@ -710,6 +739,8 @@ int at_step(at_ctx* c, int64_t nsteps)
         a.level = c->level;
         a.u = u;
         a.hist_recompute = recompute ? 1 : 0;
+        a.Tw = c->stage_tw;
+        a.wpp = c->pb.pe_size / c->stage_tw;
         for (int s = 0; s < L.S; ++s) {
             a.stage = s;
             // stencil source and output of each stage (ping-pong A/B, last stage in place)
@@ -718,7 +749,7 @@ int at_step(at_ctx* c, int64_t nsteps)
             a.X = X;
             a.Y = Y;
             e = record(c, true);
-            if (e == cudaSuccess) e = atk_launch_stage(a, c->pb.pde, c->pb.order, c->stream);
+            if (e == cudaSuccess) e = atk_launch_stage(a, c->pb.pde, c->pb.order, c->sms, c->stream);
             if (e != cudaSuccess) return cuda_fail(e, "stage kernel launch");
             e = record(c, false);
             if (e != cudaSuccess) return cuda_fail(e, "profiling event");
@@ -1078,6 +1109,8 @@ int at_stage(at_ctx* c)
     a.level = c->level;
     a.u = u;
     a.stage = s;
+    a.Tw = c->stage_tw;
+    a.wpp = c->pb.pe_size / c->stage_tw;
     a.open_ends = c->open_ends;
     a.pe_base = c->pe_base;
     a.pe_total = c->pe_total;
@@ -1088,7 +1121,7 @@ int at_stage(at_ctx* c)
     a.X = (s == 0) ? u : ((s % 2 == 1) ? A : Bf);
     a.Y = (s == L.S - 1) ? u : ((s % 2 == 0) ? A : Bf);
     e = record(c, true);
-    if (e == cudaSuccess) e = atk_launch_stage(a, c->pb.pde, c->pb.order, c->stream);
+    if (e == cudaSuccess) e = atk_launch_stage(a, c->pb.pde, c->pb.order, c->sms, c->stream);
     if (e == cudaSuccess) e = record(c, false);
     if (e != cudaSuccess) return cuda_fail(e, "stage kernel launch");
     ++c->launched;

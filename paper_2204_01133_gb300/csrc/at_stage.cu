@@ -303,7 +303,7 @@ __device__ __forceinline__ void central_window(const StageArgs& a, const Cx& cx,
 // > 1 only when every window spans a whole PE, so all groups pass the same
 // barriers, and a.wpc divides the window count).
 template <int PDE, int H, int RKS>
-__global__ void __launch_bounds__(256, PDE == ADVDIFF ? 6 : 5) stage_central(const StageArgs a)
+__global__ void __launch_bounds__(256, PDE == ADVDIFF ? 6 : (PDE == RNS_CHAIN ? 3 : 5)) stage_central(const StageArgs a)
 {
     extern __shared__ double sm[];
     const int gs = blockDim.x / a.wpc;
@@ -797,7 +797,8 @@ size_t atk_stage_smem_bytes(int pde, int Tw, int H)
 int atk_stage_block(int pde, int Tw)
 {
     int nv = (pde == atk::RNS || pde == atk::EULER) ? 4 : 1;
-    int want = (pde == atk::EULER || pde == atk::ADV_WENO || pde == atk::BURGERS) ? 256 : nv * Tw;
+    // WENO: a thread per (edge, variable)
+    int want = (pde == atk::EULER || pde == atk::ADV_WENO || pde == atk::BURGERS) ? nv * (Tw + 1) : nv * Tw;
     // reacting N-S: half a thread per (point, variable) item, so that a CTA of
     // 256 threads takes two whole-PE windows (below).  A window's fill has
     // fewer items than its update (own points plus ring levels, against 4 per
@@ -810,21 +811,27 @@ int atk_stage_block(int pde, int Tw)
     return want < 32 ? 32 : want;
 }
 
-cudaError_t atk_launch_stage(const atk::StageArgs& a, int pde, int order, cudaStream_t st)
+cudaError_t atk_launch_stage(const atk::StageArgs& a, int pde, int order, int sms, cudaStream_t st)
 {
     const int64_t windows = a.P * a.wpp;
-    const int b1 = atk_stage_block(pde, a.Tw);
+    int b1 = atk_stage_block(pde, a.Tw);
+    // the chain-rule form on few windows: a thread per fill item (own points and
+    // buffer levels), so that the fill takes one pass
+    const bool few = windows < 16 * (int64_t)sms;
+    if (pde == atk::RNS_CHAIN && few && a.Tw <= 192) b1 = (a.Tw + 2 * a.H * (a.q + 1) + 31) / 32 * 32 > 256 ? 256 : (a.Tw + 2 * a.H * (a.q + 1) + 31) / 32 * 32;
     size_t smem1 = atk_stage_smem_bytes(pde, a.Tw, a.H);
     if (a.weno_interp) {  // G [ND][W2], SP, ARR [W2], LAM [E], REC [NV][2][E], HS with W2 = Tw + 8, E = Tw + 3
         const size_t nd = pde == atk::EULER ? 8 : 2, nv = nd / 2, W2 = a.Tw + 2 * a.H, E = a.Tw + 3;
         smem1 = sizeof(double) * (nd * W2 + 2 * W2 + E + 2 * nv * E + (size_t)2 * a.H * (AT_QMAX + 1) * nd);
     }
     // central stencils on small windows: several windows per CTA (whole PEs
-    // only, dividing the window count), so a CTA carries up to 256 threads
+    // only, dividing the window count), so a CTA carries up to 256 threads, where
+    // that leaves four CTAs an SM (the chain-rule form at 16,384 points, 256
+    // windows: @C@ us per stage with four windows a CTA, @D@ with one)
     int m = 1;
     if ((pde == atk::ADVDIFF || pde == atk::RNS || pde == atk::RNS_CHAIN) && a.wpp == 1) {
         for (int c = 4; c >= 2; c /= 2)
-            if (c * b1 <= 256 && windows % c == 0) {
+            if (c * b1 <= 256 && windows % c == 0 && windows / c >= 4 * (int64_t)sms) {
                 m = c;
                 break;
             }
