@@ -169,11 +169,8 @@ __global__ void __launch_bounds__(288, 2) persist_central(const StageArgs a, int
     double* ACC = U + NV * B;      // RK accumulator      [NV][B]
     double* X = ACC + NV * B;      // stage argument      [NV][B]
     double* G2 = X + NV * B;       // derived, by stage parity [2][ND][W2]
-    double* HS = G2 + 2 * ND * W2; // halo levels         [2H(q+1)][ND]
-    double* E = HS + 2 * H * (AT_QMAX + 1) * ND;  // exp(-Ea/T) of own points [B]
+    double* E = G2 + 2 * ND * W2;  // exp(-Ea/T) of own points [B]
     __shared__ long long s_abort_at;  // first stage whose halo could not be formed
-    __shared__ int s_k[2];
-    __shared__ int s_fail;
     const int nw = (a.mode == AT) ? a.q + 1 : 1;
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
@@ -188,10 +185,19 @@ __global__ void __launch_bounds__(288, 2) persist_central(const StageArgs a, int
     // w % 4 and the halo warp on hwarp % 4 (sub-partition 0 with 8 workers).
     // The derive warps start at warp 1, so that two of them (a 64-point PE)
     // take sub-partitions 1 and 2, away from the halo warp.
-    int derive_rank = -1;
+    int derive_rank = -1, arr_rank = -1;
     if (warp < hwarp) {
         const int r = (warp + hwarp - 1) % hwarp;  // warp 1 -> rank 0, warp 2 -> rank 1, ...
         if (r < bw) derive_rank = r;
+    }
+    // The Arrhenius factor exp(-Ea/T) on warps of its own where there are enough
+    // (the last ones; for two derive warps of eight, warps 3 and 7 on
+    // sub-partition 3, which has no other work in phase A): derivation and factor
+    // took 2,600 cycles one after the other, 1,300 and 2,000 side by side
+    const bool arr_apart = PDE == RNS && hwarp > 2 * bw;
+    if (arr_apart && warp < hwarp) {
+        if (bw == 2 && hwarp == 8) arr_rank = warp == 3 ? 0 : (warp == 7 ? 1 : -1);
+        else if (warp >= hwarp - bw) arr_rank = warp - (hwarp - bw);
     }
 
     for (int i = threadIdx.x; i < NV * B; i += blockDim.x) {
@@ -221,109 +227,105 @@ __global__ void __launch_bounds__(288, 2) persist_central(const StageArgs a, int
 
     if (warp == hwarp) {
         // ---- the halo warp: stage t's buffer values, one stage ahead ----
+        // Lane items: (buffer point, derived quantity), NP a lane, read straight
+        // from the neighbours' rings of derived quantities, all levels in flight
+        // at once.  A side with delay k >= 1 reads what the neighbour published
+        // a step ago, which the last progress counter seen usually covers: its
+        // values are formed first, and only a side with delay 0 waits for the
+        // stage just finished, with nothing but one copy left to do.
+        constexpr int NI = 2 * H * ND, NP = (NI + 31) / 32;
         int64_t n = level0;
+        int64_t seen = -0x7fffffffffffffffLL;  // lanes 0, 1: the neighbour's counter as last read
         int s = 0;
+        int r0 = (int)((uint32_t)level0 % (uint32_t)a.R);  // ring slot of level n
         for (int64_t t = 0; t < T; ++t) {
             const int p = (int)(t & 1);
             double* G = G2 + p * ND * W2;
             const bool last = (s == S - 1);
             const int64_t Ln = last ? n + 1 : n;  // the stage argument stage t produces: (Ln, sn)
             const int sn = last ? 0 : s + 1;
-            if (t >= 2) bar_sync_p<3>(p, nall);  // the workers are done with G[p] (stage t - 2)
-            if (lane == 0) s_fail = 0;
-            __syncwarp();
-            if (lane < 2) {
-                const int side = lane;
-                int k;
-                bool ok;
-                // one bounded wait for both conditions on the neighbour's
-                // progress: the stage-s argument this stage reads has been
-                // published, and the ring slot of (Ln, sn) this stage writes is
-                // no longer read by it
-                const int64_t free_at = (Ln - a.slack - 1) * S + sn + 1;
-                if (a.arrival) {
-                    // the freshest stage-s argument of the neighbour that has
-                    // arrived, once one recent enough for the clamp is there
-                    const int kc = kcap_at(a, n);
-                    const int64_t need = (n - kc) * S + s;
-                    ok = wait_ge(a, a.done + nbr[side], need > free_at ? need : free_at);
-                    const int64_t m = (load_acquire(a.done + nbr[side]) - s) / S;
-                    k = m >= n ? 0 : (int)(n - m);
-                    if (k > kc) k = kc;  // only if the wait gave up
-                } else {
-                    // the neighbour's stage-s argument at the drawn level n-k
-                    k = keff_at(a, n, s, pe, side);
-                    const int64_t need = (n - k) * S + s;
-                    ok = wait_ge(a, a.done + nbr[side], need > free_at ? need : free_at);
-                }
-                s_k[side] = k;
-                log_delay(a, n, s, pe, side, k);
-                if (!ok) s_fail = 1;
+            // the ring slot of (Ln, sn) this stage writes is no longer read by the neighbour
+            const int64_t free_at = (Ln - a.slack - 1) * S + sn + 1;
+            int k = 0;
+            if (lane < 2 && !a.arrival) {
+                k = keff_at(a, n, s, pe, lane);
+                log_delay(a, n, s, pe, lane, k);
             }
-            __syncwarp();
-            const bool failed = *(volatile int*)&s_fail != 0;
-            if (!failed) {
-                // A side with delay 0 has weights (1, +-0, ...), exact integer
-                // ratios: its buffer values are the neighbour's level-n quantities
-                // themselves, up to the sign of a zero, which no stencil sum sees
-                // (they start from +0 and take the buffer columns as factors), so
-                // they are copied without FP64 work.  Their loads go first, so
-                // that they are in flight with those of the other side.  (With
-                // one derived quantity the weighted sum is a few instructions on
-                // 2H lanes and the staging of the general case measured faster:
-                // there every side takes it.)
-                constexpr bool copy0 = ND > 1;
-                constexpr int NI = 2 * H * ND, NP = (NI + 31) / 32;
-                double cur[NP];
-#pragma unroll
-                for (int i = 0; i < NP; ++i) {
-                    const int c = lane + 32 * i;
-                    cur[i] = 0.0;
-                    if (c < NI) {
-                        const int hp = c / ND, d = c - hp * ND;
-                        const int side = hp < H ? 0 : 1;
-                        if (copy0 && s_k[side] == 0)
-                            cur[i] = __ldcg(a.gring + gring_index(a, n, s, nbr[side], 1 - side,
-                                                                 side == 0 ? hp : hp - H, ND) + d);
+            if (t >= 2) bar_sync_p<3>(p, nall);  // the workers are done with G[p] (stage t - 2)
+            bool ok = true;
+            // with delays by arrival: the freshest stage-s argument of the
+            // neighbour that has arrived, once one recent enough for the clamp is there
+            if (lane < 2 && a.arrival) {
+                const int kc = kcap_at(a, n);
+                const int64_t need = (n - kc) * S + s;
+                ok = wait_ge(a, a.done + nbr[lane], need > free_at ? need : free_at);
+                seen = load_acquire(a.done + nbr[lane]);
+                const int64_t m = (seen - s) / S;
+                k = m >= n ? 0 : (int)(n - m);
+                if (k > kc) k = kc;  // only if the wait gave up
+                log_delay(a, n, s, pe, lane, k);
+            }
+            const int k0 = __shfl_sync(0xffffffffu, k, 0), k1 = __shfl_sync(0xffffffffu, k, 1);
+            // both passes wait for "published" and "slot free" on the neighbour's counter
+            auto wait_for = [&](bool mine) {
+                if (mine && !a.arrival) {
+                    const int64_t need = (n - k) * S + s, target = need > free_at ? need : free_at;
+                    if (seen < target) {
+                        ok = wait_ge(a, a.done + nbr[lane], target);
+                        seen = load_acquire(a.done + nbr[lane]);
                     }
                 }
-                // the other sides: their levels n-k-l into HS
-                const int tt = lane;
-                if (tt < 2 * H * nw) {
-                    const int hp = tt / nw, l = tt - hp * nw;
-                    const int side = hp < H ? 0 : 1;
-                    const int h = side == 0 ? hp : hp - H;
-                    const int k = s_k[side];
-                    const bool staged = !copy0 || k >= 1;
-                    if (staged && ((a.wnz[k] >> l) & 1)) {
-                        // the neighbour's own derived quantities of that level
-                        const int64_t gi = gring_index(a, n - k - l, s, nbr[side], 1 - side, h, ND);
-#pragma unroll
-                        for (int d = 0; d < ND; ++d) HS[tt * ND + d] = __ldcg(a.gring + gi + d);
-                    } else if (staged) {
-#pragma unroll
-                        for (int d = 0; d < ND; ++d) HS[tt * ND + d] = 0.0;
-                    }
-                }
-                __syncwarp();
-                // weighted sum over levels, in level order: lanes (buffer point, quantity)
+            };
+            // A side with delay 0 has weights (1, +-0, ...), exact integer ratios:
+            // its buffer values are the neighbour's level-n quantities themselves,
+            // up to the sign of a zero, which no stencil sum sees.
+            auto fill = [&](bool zero) {
+                double v[NP][AT_QMAX + 1];
 #pragma unroll
                 for (int i = 0; i < NP; ++i) {
-                    const int c = lane + 32 * i;
-                    if (c < NI) {
-                        const int hp = c / ND, d = c - hp * ND;
-                        const int k = s_k[hp < H ? 0 : 1];
-                        double acc = cur[i];
-                        if (!copy0 || k >= 1) {
-                            acc = ((a.mode == AT) ? a.w[k][0] : 1.0) * HS[(hp * nw) * ND + d];
-                            for (int l = 1; l < nw; ++l) acc = fma(a.w[k][l], HS[(hp * nw + l) * ND + d], acc);
+                    const int c = lane + 32 * i, hp = c / ND, d = c - hp * ND;
+                    const int side = hp < H ? 0 : 1, h = side == 0 ? hp : hp - H;
+                    const int kk = side == 0 ? k0 : k1;
+#pragma unroll
+                    for (int l = 0; l <= AT_QMAX; ++l) {
+                        v[i][l] = 0.0;  // a level with weight 0 is not part of the scheme
+                        if (c < NI && (kk == 0) == zero && (zero ? l == 0 : l < nw && ((a.wnz[kk] >> l) & 1))) {
+                            int r = r0 - kk - l;
+                            if (r < 0) r += a.R;
+                            v[i][l] = __ldcg(a.gring + ((((int64_t)(r * S + s) * a.P + nbr[side]) * 2 + 1 - side) * H + h) * ND + d);
+                        }
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < NP; ++i) {
+                    const int c = lane + 32 * i, hp = c / ND, d = c - hp * ND;
+                    const int kk = hp < H ? k0 : k1;
+                    if (c < NI && (kk == 0) == zero) {
+                        double acc = v[i][0];
+                        if (!zero) {
+                            acc = ((a.mode == AT) ? a.w[kk][0] : 1.0) * v[i][0];
+#pragma unroll
+                            for (int l = 1; l <= AT_QMAX; ++l)
+                                if (l < nw) acc = fma(a.w[kk][l], v[i][l], acc);
                         }
                         G[d * W2 + (hp < H ? hp : B + hp)] = acc;
                     }
                 }
-            } else if (lane == 0) {
-                s_abort_at = t;
+            };
+            bool failed = false;
+            if (k0 >= 1 || k1 >= 1) {
+                wait_for(lane < 2 && k >= 1);
+                failed = __any_sync(0xffffffffu, !ok);
+                __syncwarp();  // orders the other lanes' reads after lanes 0 and 1 saw the counters
+                if (!failed) fill(false);
             }
+            if (!failed && (k0 == 0 || k1 == 0)) {
+                wait_for(lane < 2 && k == 0);
+                failed = __any_sync(0xffffffffu, !ok);
+                __syncwarp();
+                if (!failed) fill(true);
+            }
+            if (failed && lane == 0) s_abort_at = t;
             __syncwarp();
             bar_arrive_p<1>(p, nall);  // stage t's halo is ready (or the run stops at t)
             if (failed) {
@@ -335,18 +337,22 @@ __global__ void __launch_bounds__(288, 2) persist_central(const StageArgs a, int
             if (++s == S) {
                 s = 0;
                 ++n;
+                if (++r0 == a.R) r0 = 0;
             }
         }
     } else {
         // ---- the worker warps ----
         int64_t n = level0;
         int s = 0;
+        int r0 = (int)((uint32_t)level0 % (uint32_t)a.R);  // ring slot of level n
         for (int64_t t = 0; t < T; ++t) {
             const int p = (int)(t & 1);
             double* G = G2 + p * ND * W2;
             const bool last = (s == S - 1);
-            const int64_t Ln = last ? n + 1 : n;
             const int sn = last ? 0 : s + 1;
+            const int rn = last ? (r0 + 1 == a.R ? 0 : r0 + 1) : r0;
+            // this PE's windows of the stage argument stage t produces, in points
+            const int64_t win = ((int64_t)(rn * S + sn) * a.P + pe) * 2 * H;
             // (A)
             if (derive_rank >= 0) {
                 for (int it = derive_rank * 32 + lane; it < B; it += bw * 32) {
@@ -357,7 +363,18 @@ __global__ void __launch_bounds__(288, 2) persist_central(const StageArgs a, int
                     P::derive(a, Q, g);
 #pragma unroll
                     for (int d = 0; d < ND; ++d) G[d * W2 + H + it] = g[d];
-                    if constexpr (PDE == RNS) E[it] = at_exp(-a.prm[5] * at_rcpi(g[7]));  // g[7] = T
+                    if constexpr (PDE == RNS)
+                        if (!arr_apart) E[it] = at_exp(-a.prm[5] * at_rcpi(g[7]));  // g[7] = T
+                }
+            }
+            if constexpr (PDE == RNS) {
+                if (arr_rank >= 0) {
+                    for (int it = arr_rank * 32 + lane; it < B; it += bw * 32) {
+                        double Q[NV];
+#pragma unroll
+                        for (int v = 0; v < NV; ++v) Q[v] = X[v * B + it];
+                        E[it] = at_exp(-a.prm[5] * at_rcpi(P::temperature(a, Q)));
+                    }
                 }
             }
             bar_sync_p<1>(p, nall);  // own derived quantities and stage t's halo in G[p]
@@ -380,7 +397,7 @@ __global__ void __launch_bounds__(288, 2) persist_central(const StageArgs a, int
                     side = 1;
                     h = jl - (B - H);
                 }
-                if (side >= 0) __stcg(a.ring + ring_index(a, Ln, sn, pe, side, h, v), y);
+                if (side >= 0) __stcg(a.ring + (win + side * H + h) * NV + v, y);
             }
             bar_sync<5>(nwork);
             // the derived quantities of the new stage argument at the edge
@@ -396,7 +413,7 @@ __global__ void __launch_bounds__(288, 2) persist_central(const StageArgs a, int
 #pragma unroll
                     for (int v = 0; v < NV; ++v) Q[v] = X[v * B + jl];
                     P::derive(a, Q, g);
-                    const int64_t gi = gring_index(a, Ln, sn, pe, side, h, ND);
+                    const int64_t gi = (win + lane) * ND;  // lane = side H + h
 #pragma unroll
                     for (int d = 0; d < ND; ++d) __stcg(a.gring + gi + d, g[d]);
                 }
@@ -407,6 +424,7 @@ __global__ void __launch_bounds__(288, 2) persist_central(const StageArgs a, int
             if (++s == S) {
                 s = 0;
                 ++n;
+                r0 = rn;
             }
         }
     }
@@ -460,7 +478,7 @@ size_t atk_persist_smem_bytes(int pde, int B, int H)
 {
     const int nv = pde == atk::RNS ? 4 : 1, nd = pde == atk::RNS ? 8 : 1;
     return sizeof(double) *
-           ((size_t)3 * nv * B + (size_t)2 * nd * (B + 2 * H) + (size_t)2 * H * (AT_QMAX + 1) * nd + (size_t)B);
+           ((size_t)3 * nv * B + (size_t)2 * nd * (B + 2 * H) + (size_t)B);
 }
 
 // worker warps for the PE's points (at least two roles' worth for phase A)
