@@ -291,7 +291,7 @@ struct Phys;
 // u_t + c u_x = a u_xx: the only derived quantity is u itself.
 template <>
 struct Phys<ADVDIFF> {
-    static constexpr int NV = 1, ND = 1;
+    static constexpr int NV = 1, ND = 1, SPLIT = 0;
     __device__ static void derive(const StageArgs&, const double* Q, double* g) { g[0] = Q[0]; }
 };
 
@@ -301,7 +301,7 @@ struct Phys<ADVDIFF> {
 // (4/3) mu, lam and rhoD.  k0 = (4/3) mu, k1 = (2/3) mu, k2 = lam, k3 = rhoD.
 template <>
 struct Phys<RNS> {
-    static constexpr int NV = 4, ND = 8;
+    static constexpr int NV = 4, ND = 8, SPLIT = 7;  // SPLIT rows are differentiated, the last is T
     __device__ static void derive(const StageArgs& a, const double* Q, double* g)
     {
         const double gm1 = a.prm[0] - 1.0, qc = a.prm[6];
@@ -335,7 +335,7 @@ struct Phys<RNS> {
 // T] are differentiated (and extrapolated at buffer points).
 template <>
 struct Phys<RNS_CHAIN> {
-    static constexpr int NV = 4, ND = 6;
+    static constexpr int NV = 4, ND = 6, SPLIT = 6;
     __device__ static void derive(const StageArgs& a, const double* Q, double* g)
     {
         const double gm1 = a.prm[0] - 1.0, qc = a.prm[6];
@@ -355,7 +355,7 @@ struct Phys<RNS_CHAIN> {
 // u (rho E + p), rho u Y); the split fluxes are C/2 +- (lam/2) Q.
 template <>
 struct Phys<EULER> {
-    static constexpr int NV = 4, ND = 8;
+    static constexpr int NV = 4, ND = 8, SPLIT = 0;
     __device__ static double pressure(const StageArgs& a, const double* Q, double u)
     {
         return (a.prm[0] - 1.0) * (Q[2] - fma(fx_half(Q[1]), u, a.prm[3] * Q[3]));
@@ -403,7 +403,7 @@ struct Phys<EULER> {
 // Scalar linear advection, WENO form: g = [c u / 2, u].
 template <>
 struct Phys<ADV_WENO> {
-    static constexpr int NV = 1, ND = 2;
+    static constexpr int NV = 1, ND = 2, SPLIT = 0;
     __device__ static void derive(const StageArgs& a, const double* Q, double* g)
     {
         g[0] = 0.5 * a.prm[0] * Q[0];
@@ -420,7 +420,7 @@ struct Phys<ADV_WENO> {
 // Inviscid Burgers, WENO form: g = [u^2 / 4, u] (C/2 with C = u^2/2); wave speed |u|.
 template <>
 struct Phys<BURGERS> {
-    static constexpr int NV = 1, ND = 2;
+    static constexpr int NV = 1, ND = 2, SPLIT = 0;
     __device__ static void derive(const StageArgs&, const double* Q, double* g)
     {
         g[0] = 0.5 * (0.5 * Q[0] * Q[0]);
@@ -547,13 +547,36 @@ __device__ __forceinline__ double weno_flux(const StageArgs& a, const double* C,
 // column c of the derived rows G (row stride ld): the differences in integers
 // (at_fixed.cuh), one FP64 instruction each to scale and add them.
 // ---------------------------------------------------------------------------
-template <int H>
-__device__ __forceinline__ double rns_flux_terms(const StageArgs& a, const double* G, int ld, int v, int c)
+template <int H, class ROWS>
+__device__ __forceinline__ double rns_flux_terms(const StageArgs& a, const ROWS& G, int v, int c)
 {
-    double K = a.s1 * fx_d1<H>(G + v * ld + c);
-    if (v > 0) K = fma(a.s2v[v - 1], fx_d2<H>(G + (3 + v) * ld + c), K);
+    double K = a.s1 * fx_d1<H>(G.row(v, c));
+    if (v > 0) K = fma(a.s2v[v - 1], fx_d2<H>(G.row(3 + v, c)), K);
     return K;
 }
+
+// Rows of derived quantities in shared memory, row stride ld: as doubles, or
+// (the reacting flow) split for the integer differences where they are written
+struct DoubleRows {
+    double* g;
+    int ld;
+    __device__ __forceinline__ void put(int d, int c, double x) const { g[d * ld + c] = x; }
+    __device__ __forceinline__ FxDoubles row(int d, int c) const { return FxDoubles{g + d * ld + c}; }
+};
+struct SplitRows {
+    int64_t* m;
+    uint32_t* e;
+    int ld;
+    __device__ __forceinline__ void put(int d, int c, double x) const
+    {
+        const FxV v = fx_split(x);
+        m[d * ld + c] = v.m;
+        e[d * ld + c] = v.e;
+    }
+    __device__ __forceinline__ FxRow row(int d, int c) const { return FxRow{m + d * ld + c, e + d * ld + c}; }
+};
+// 8-byte words of `rows` split rows of ld columns
+__host__ __device__ constexpr int split_words(int rows, int ld) { return rows * ld + (rows * ld + 1) / 2; }
 
 // ---------------------------------------------------------------------------
 // The RK update of the step-fused kernels, stage by stage: the next stage

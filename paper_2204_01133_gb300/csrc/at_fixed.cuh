@@ -116,20 +116,43 @@ AT_HD int fx_clz(uint64_t v)
 constexpr uint32_t FX_EXP = 0x7ff00000u;
 constexpr int FX_GUARD = 3;  // bits kept below the last bit of the largest value
 
-// x as a signed integer in units of 2^-GUARD ulp at the exponent field
-// emax (>= x's own; in place, bits 20..30 of the high word), cut towards zero;
-// a zero or subnormal has no implicit bit
+// A double as a signed integer in units of 2^-FX_GUARD of its last place and its
+// exponent field (in place, bits 20..30 of the high word); a zero or subnormal
+// has no implicit bit.  Inf and NaN keep their bits, marked by the field.
+struct FxV {
+    int64_t m;
+    uint32_t e;
+};
+
 template <int GUARD = FX_GUARD>
-AT_HD int64_t fx_align(double x, uint32_t emax)
+AT_HD FxV fx_split(double x)
 {
     const uint32_t hi = fx_hi(x), t = hi & FX_EXP;
     const uint64_t m = ((uint64_t)((hi & 0xfffffu) | fx_min(t, 0x100000u)) << 32 | fx_lo(x)) << GUARD;
-    const uint64_t v = m >> fx_min((emax - t) >> 20, 63u);
     const int64_t s = (int32_t)hi >> 31;
-    return (int64_t)(v ^ (uint64_t)s) - s;
+    return FxV{t == FX_EXP ? (int64_t)((uint64_t)hi << 32 | fx_lo(x)) : (int64_t)(m ^ (uint64_t)s) - s, t};
 }
 
-// the integer x in fx_align's units as a double, rounded to nearest; *ok is
+// the double that fx_split took apart (the sign of a zero aside)
+AT_HD double fx_join(FxV v)
+{
+    const uint64_t a = (v.m < 0 ? 0u - (uint64_t)v.m : (uint64_t)v.m) >> FX_GUARD;
+    const uint32_t s = (uint32_t)((uint64_t)v.m >> 32) & 0x80000000u;
+    const uint64_t r = (a & 0xfffffffffffffull) | ((uint64_t)(v.e | s) << 32);
+    const uint64_t x = v.e == FX_EXP ? (uint64_t)v.m : r;
+    return fx_double((uint32_t)(x >> 32), (uint32_t)x);
+}
+
+// its integer at the exponent field emax (at least its own), cut downwards
+AT_HD int64_t fx_at(FxV v, uint32_t emax) { return v.m >> fx_min((emax - v.e) >> 20, 63u); }
+
+template <int GUARD>
+AT_HD int64_t fx_align(double x, uint32_t emax)
+{
+    return fx_at(fx_split<GUARD>(x), emax);
+}
+
+// the integer x in fx_at's units as a double, rounded to nearest; *ok is
 // cleared where the result is not a normal number or zero
 AT_HD double fx_result(int64_t x, uint32_t emax, bool* ok)
 {
@@ -161,8 +184,8 @@ AT_HD constexpr int fx_t2(int o)
 // to the ends of the exponent range, second differences that could overflow),
 // the combination by FMAs.  Loops that stay loops: straight-line code could be
 // predicated, and FP64 instructions take their issue slots also when off.
-template <int H, int ORDER>
-AT_HD double fx_chain(const double* F)
+template <int H, int ORDER, class ROW>
+AT_HD double fx_chain(const ROW& F)
 {
     double x = 0.0;
 #ifdef __CUDA_ARCH__
@@ -176,27 +199,40 @@ AT_HD double fx_chain(const double* F)
         } else {
             t = o == 0 ? (H == 3 ? -490.0 : (H == 2 ? -30.0 : -2.0)) : (double)fx_t2<H>(o > 0 ? o : -o);
         }
-        x = ::fma(t, F[o], x);
+        x = ::fma(t, fx_join(F[o]), x);
     }
     return x;
 }
 
+// A row around a point: F[o] the split value o points on.  Of doubles, split
+// where they are read; or of values split once where they were formed (a
+// mantissa and an exponent row), which leaves 8 of the 24 issue cycles a tap
+// (the flame of 2^22 points 2.13 -> 1.99 ms per step, of 2,048 points 16.6 -> 15.7 us).
+struct FxDoubles {
+    const double* f;
+    AT_HD FxV operator[](int o) const { return fx_split(f[o]); }
+};
+struct FxRow {
+    const int64_t* m;
+    const uint32_t* e;
+    AT_HD FxV operator[](int o) const { return FxV{m[o], e[o]}; }
+};
+
 // D1 times the first difference at F[0]
-template <int H>
-AT_HD double fx_d1(const double* F)
+template <int H, class ROW>
+AT_HD double fx_d1(const ROW& F)
 {
-    double f[2 * H];
+    FxV f[2 * H];
     uint32_t emax = 0;
 #pragma unroll
     for (int o = 0; o < H; ++o) {
         f[2 * o] = F[o + 1];
         f[2 * o + 1] = F[-o - 1];
-        emax = fx_max(emax, fx_max(fx_hi(f[2 * o]) & FX_EXP, fx_hi(f[2 * o + 1]) & FX_EXP));
+        emax = fx_max(emax, fx_max(f[2 * o].e, f[2 * o + 1].e));
     }
     int64_t x = 0;
 #pragma unroll
-    for (int o = 0; o < H; ++o)
-        x += fx_t1<H>(o + 1) * (fx_align(f[2 * o], emax) - fx_align(f[2 * o + 1], emax));
+    for (int o = 0; o < H; ++o) x += fx_t1<H>(o + 1) * (fx_at(f[2 * o], emax) - fx_at(f[2 * o + 1], emax));
     bool ok = emax != FX_EXP;
     double r = fx_result(x, emax, &ok);
     if (!ok) r = fx_chain<H, 1>(F);
@@ -204,25 +240,25 @@ AT_HD double fx_d1(const double* F)
 }
 
 // D2 times the second difference at F[0]
-template <int H>
-AT_HD double fx_d2(const double* F)
+template <int H, class ROW>
+AT_HD double fx_d2(const ROW& F)
 {
-    const double f0 = F[0];
-    double f[2 * H];
-    uint32_t emax = fx_hi(f0) & FX_EXP;
+    const FxV f0 = F[0];
+    FxV f[2 * H];
+    uint32_t emax = f0.e;
 #pragma unroll
     for (int o = 0; o < H; ++o) {
         f[2 * o] = F[o + 1];
         f[2 * o + 1] = F[-o - 1];
-        emax = fx_max(emax, fx_max(fx_hi(f[2 * o]) & FX_EXP, fx_hi(f[2 * o + 1]) & FX_EXP));
+        emax = fx_max(emax, fx_max(f[2 * o].e, f[2 * o + 1].e));
     }
-    const int64_t two0 = 2 * fx_align(f0, emax);
+    const int64_t two0 = 2 * fx_at(f0, emax);
     bool ok = emax != FX_EXP;
     int64_t x = 0;
 #pragma unroll
     for (int o = 0; o < H; ++o) {
-        const int64_t s = fx_align(f[2 * o], emax) + fx_align(f[2 * o + 1], emax) - two0;
-        // |s| < 2^58; with the taps of H = 3 the sum stays below 2^63 when
+        const int64_t s = fx_at(f[2 * o], emax) + fx_at(f[2 * o + 1], emax) - two0;
+        // |s| <= 2^58; with the taps of H = 3 the sum stays below 2^63 when
         // |s_1| < 2^53 (an eighth of the largest value) and |s_2| < 2^57
         if (H == 3 && o < 2) {
             const int32_t sh = (int32_t)((uint64_t)s >> 32);

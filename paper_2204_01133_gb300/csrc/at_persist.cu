@@ -57,9 +57,9 @@ __device__ bool wait_ge(const StageArgs& a, int64_t* ctr, int64_t target)
 // stencil, source and RK update of own point (v, jl) for stage s, in shared
 // memory: the same arithmetic, in the same order, as the per-stage kernels
 // (the Arrhenius factor exp(-Ea/T) arrives precomputed in E)
-template <int PDE, int H>
-__device__ __forceinline__ double point_update(const StageArgs& a, int s, int v, int jl, const double* G,
-                                               const double* E, double* X, double* U, double* ACC, int W2, int B,
+template <int PDE, int H, class ROWS>
+__device__ __forceinline__ double point_update(const StageArgs& a, int s, int v, int jl, const ROWS& G,
+                                               const double* E, double* X, double* U, double* ACC, int B,
                                                bool last)
 {
     const int it = v * B + jl;
@@ -68,9 +68,9 @@ __device__ __forceinline__ double point_update(const StageArgs& a, int s, int v,
     const double x = X[it];
     if constexpr (PDE == ADVDIFF) {
 #pragma unroll
-        for (int o = -H; o <= H; ++o) K = fma(a.cm[o + H], G[c + o], K);
+        for (int o = -H; o <= H; ++o) K = fma(a.cm[o + H], G.g[c + o], K);
     } else {
-        K = rns_flux_terms<H>(a, G, W2, v, c);
+        K = rns_flux_terms<H>(a, G, v, c);
         if (v == 3) K = fma(-a.prm[4] * x, E[jl], K);
     }
     const double dt = a.dt;
@@ -168,8 +168,19 @@ __global__ void __launch_bounds__(288, 2) persist_central(const StageArgs a, int
     double* U = sm;                // u^n                 [NV][B]
     double* ACC = U + NV * B;      // RK accumulator      [NV][B]
     double* X = ACC + NV * B;      // stage argument      [NV][B]
-    double* G2 = X + NV * B;       // derived, by stage parity [2][ND][W2]
-    double* E = G2 + 2 * ND * W2;  // exp(-Ea/T) of own points [B]
+    double* E = X + NV * B;        // exp(-Ea/T) of own points [B]
+    double* G2 = E + B;            // derived rows by stage parity: [2][W2] doubles, or the
+                                   // reacting flow's split rows
+    constexpr int NG = P::SPLIT > 0 ? P::SPLIT : ND;
+    const int gwords = P::SPLIT > 0 ? split_words(NG, W2) : NG * W2;
+    auto rows = [&](int p) {
+        if constexpr (P::SPLIT > 0) {
+            int64_t* m = (int64_t*)(G2 + p * gwords);
+            return SplitRows{m, (uint32_t*)(m + NG * W2), W2};
+        } else {
+            return DoubleRows{G2 + p * gwords, W2};
+        }
+    };
     __shared__ long long s_abort_at;  // first stage whose halo could not be formed
     const int nw = (a.mode == AT) ? a.q + 1 : 1;
     const int lane = threadIdx.x & 31;
@@ -233,14 +244,14 @@ __global__ void __launch_bounds__(288, 2) persist_central(const StageArgs a, int
         // a step ago, which the last progress counter seen usually covers: its
         // values are formed first, and only a side with delay 0 waits for the
         // stage just finished, with nothing but one copy left to do.
-        constexpr int NI = 2 * H * ND, NP = (NI + 31) / 32;
+        constexpr int NI = 2 * H * NG, NP = (NI + 31) / 32;
         int64_t n = level0;
         int64_t seen = -0x7fffffffffffffffLL;  // lanes 0, 1: the neighbour's counter as last read
         int s = 0;
         int r0 = (int)((uint32_t)level0 % (uint32_t)a.R);  // ring slot of level n
         for (int64_t t = 0; t < T; ++t) {
             const int p = (int)(t & 1);
-            double* G = G2 + p * ND * W2;
+            const auto G = rows(p);
             const bool last = (s == S - 1);
             const int64_t Ln = last ? n + 1 : n;  // the stage argument stage t produces: (Ln, sn)
             const int sn = last ? 0 : s + 1;
@@ -283,7 +294,7 @@ __global__ void __launch_bounds__(288, 2) persist_central(const StageArgs a, int
                 double v[NP][AT_QMAX + 1];
 #pragma unroll
                 for (int i = 0; i < NP; ++i) {
-                    const int c = lane + 32 * i, hp = c / ND, d = c - hp * ND;
+                    const int c = lane + 32 * i, hp = c / NG, d = c - hp * NG;
                     const int side = hp < H ? 0 : 1, h = side == 0 ? hp : hp - H;
                     const int kk = side == 0 ? k0 : k1;
 #pragma unroll
@@ -298,7 +309,7 @@ __global__ void __launch_bounds__(288, 2) persist_central(const StageArgs a, int
                 }
 #pragma unroll
                 for (int i = 0; i < NP; ++i) {
-                    const int c = lane + 32 * i, hp = c / ND, d = c - hp * ND;
+                    const int c = lane + 32 * i, hp = c / NG, d = c - hp * NG;
                     const int kk = hp < H ? k0 : k1;
                     if (c < NI && (kk == 0) == zero) {
                         double acc = v[i][0];
@@ -308,7 +319,7 @@ __global__ void __launch_bounds__(288, 2) persist_central(const StageArgs a, int
                             for (int l = 1; l <= AT_QMAX; ++l)
                                 if (l < nw) acc = fma(a.w[kk][l], v[i][l], acc);
                         }
-                        G[d * W2 + (hp < H ? hp : B + hp)] = acc;
+                        G.put(d, hp < H ? hp : B + hp, acc);
                     }
                 }
             };
@@ -347,7 +358,7 @@ __global__ void __launch_bounds__(288, 2) persist_central(const StageArgs a, int
         int r0 = (int)((uint32_t)level0 % (uint32_t)a.R);  // ring slot of level n
         for (int64_t t = 0; t < T; ++t) {
             const int p = (int)(t & 1);
-            double* G = G2 + p * ND * W2;
+            const auto G = rows(p);
             const bool last = (s == S - 1);
             const int sn = last ? 0 : s + 1;
             const int rn = last ? (r0 + 1 == a.R ? 0 : r0 + 1) : r0;
@@ -362,7 +373,7 @@ __global__ void __launch_bounds__(288, 2) persist_central(const StageArgs a, int
                     for (int v = 0; v < NV; ++v) Q[v] = X[v * B + it];
                     P::derive(a, Q, g);
 #pragma unroll
-                    for (int d = 0; d < ND; ++d) G[d * W2 + H + it] = g[d];
+                    for (int d = 0; d < NG; ++d) G.put(d, H + it, g[d]);
                     if constexpr (PDE == RNS)
                         if (!arr_apart) E[it] = at_exp(-a.prm[5] * at_rcpi(g[7]));  // g[7] = T
                 }
@@ -387,7 +398,7 @@ __global__ void __launch_bounds__(288, 2) persist_central(const StageArgs a, int
             for (int it = threadIdx.x; it < NV * B; it += nwork) {
                 const int v = by_warp ? warp % NV : it / B;
                 const int jl = by_warp ? (warp / NV) * 32 + lane : it - v * B;
-                const double y = point_update<PDE, H>(a, s, v, jl, G, E, X, U, ACC, W2, B, last);
+                const double y = point_update<PDE, H>(a, s, v, jl, G, E, X, U, ACC, B, last);
                 if (nonfinite(y)) bad = 1;
                 int side = -1, h = 0;
                 if (jl < H) {
@@ -415,7 +426,7 @@ __global__ void __launch_bounds__(288, 2) persist_central(const StageArgs a, int
                     P::derive(a, Q, g);
                     const int64_t gi = (win + lane) * ND;  // lane = side H + h
 #pragma unroll
-                    for (int d = 0; d < ND; ++d) __stcg(a.gring + gi + d, g[d]);
+                    for (int d = 0; d < NG; ++d) __stcg(a.gring + gi + d, g[d]);
                 }
                 __syncwarp();
                 if (lane == 0 && pe != a.withhold_pe) store_release(a.done + pe, n * S + s + 1);
@@ -476,9 +487,9 @@ void* persist_kernel(int pde, int order)
 
 size_t atk_persist_smem_bytes(int pde, int B, int H)
 {
-    const int nv = pde == atk::RNS ? 4 : 1, nd = pde == atk::RNS ? 8 : 1;
-    return sizeof(double) *
-           ((size_t)3 * nv * B + (size_t)2 * nd * (B + 2 * H) + (size_t)B);
+    const int nv = pde == atk::RNS ? 4 : 1, W2 = B + 2 * H;
+    const size_t rows = pde == atk::RNS ? atk::split_words(atk::Phys<atk::RNS>::SPLIT, W2) : W2;
+    return sizeof(double) * ((size_t)3 * nv * B + 2 * rows + (size_t)B);
 }
 
 // worker warps for the PE's points (at least two roles' worth for phase A)

@@ -53,7 +53,8 @@ __device__ __forceinline__ Cx launch_cx(const StageArgs& a) { return Cx{a.level,
 template <int PDE, bool WENO>
 __device__ __forceinline__ void fill_window(const StageArgs& a, const Cx& cx, double* __restrict__ G,
                                             double* __restrict__ SP, double* __restrict__ HS, int64_t pe, int chunk,
-                                            int64_t t0, int W2, int lt, int gs, double* __restrict__ ARR = nullptr)
+                                            int64_t t0, int W2, int lt, int gs, double* __restrict__ ARR = nullptr,
+                                            SplitRows SR = SplitRows{nullptr, nullptr, 0})
 {
     using P = Phys<PDE>;
     constexpr int NV = P::NV, ND = P::ND;
@@ -79,8 +80,14 @@ __device__ __forceinline__ void fill_window(const StageArgs& a, const Cx& cx, do
             } else {
                 P::derive(a, Q, g);
             }
+            if constexpr (P::SPLIT > 0) {  // G: the temperature (flux form); the rest split
 #pragma unroll
-            for (int d = 0; d < ND; ++d) G[d * W2 + i] = g[d];
+                for (int d = 0; d < P::SPLIT; ++d) SR.put(d, i, g[d]);
+                if constexpr (P::SPLIT < ND) G[i] = g[P::SPLIT];
+            } else {
+#pragma unroll
+                for (int d = 0; d < ND; ++d) G[d * W2 + i] = g[d];
+            }
         } else {
             const int t = it - own;
             const int hp = t / nw, l = t - hp * nw;         // buffer point, level
@@ -120,7 +127,11 @@ __device__ __forceinline__ void fill_window(const StageArgs& a, const Cx& cx, do
         double acc = ((a.mode == AT) ? a.w[k][0] : 1.0) * HS[(hp * nw) * ND + d];
         for (int l = 1; l < nw; ++l) acc = fma(a.w[k][l], HS[(hp * nw + l) * ND + d], acc);
         const int i = hp < L0 ? hp : W2 - R0 + (hp - L0);
-        G[d * W2 + i] = acc;
+        if constexpr (P::SPLIT > 0) {
+            if (d < P::SPLIT) SR.put(d, i, acc);
+        } else {
+            G[d * W2 + i] = acc;
+        }
     }
 }
 
@@ -214,19 +225,19 @@ __device__ __forceinline__ void rk_update(const StageArgs& a, const Cx& cx, int 
 // (tau = 4/3 mu u_x, q = -lam T_x + q_c J_F, J_F = -rhoD Y_x), the factors
 // being the point's own current values; then the four RK updates.
 template <int H, int RKS>
-__device__ __forceinline__ void chain_point(const StageArgs& a, const Cx& cx, const double* G, int W2, int64_t pe,
-                                            int jpe, int64_t j, int c)
+__device__ __forceinline__ void chain_point(const StageArgs& a, const Cx& cx, const SplitRows& G, int64_t pe, int jpe,
+                                            int64_t j, int c)
 {
     double m[5];  // -d/dx of rho, u, p, rho E, Y
 #pragma unroll
     for (int q = 0; q < 5; ++q) {
-        m[q] = a.s1 * fx_d1<H>(G + q * W2 + c);
+        m[q] = a.s1 * fx_d1<H>(G.row(q, c));
     }
-    const double uxx = a.s2 * fx_d2<H>(G + 1 * W2 + c);
-    const double Yxx = a.s2 * fx_d2<H>(G + 4 * W2 + c);
-    const double Txx = a.s2 * fx_d2<H>(G + 5 * W2 + c);
-    const double rho = G[c], u = G[W2 + c], p = G[2 * W2 + c], rE = G[3 * W2 + c], Y = G[4 * W2 + c];
-    const double T = G[5 * W2 + c];
+    const double uxx = a.s2 * fx_d2<H>(G.row(1, c));
+    const double Yxx = a.s2 * fx_d2<H>(G.row(4, c));
+    const double Txx = a.s2 * fx_d2<H>(G.row(5, c));
+    auto at = [&](int q) { return fx_join(G.row(q, c)[0]); };
+    const double rho = at(0), u = at(1), p = at(2), rE = at(3), Y = at(4), T = at(5);
     const double ru = rho * u;
     double K[4];
     K[0] = fma(m[0], u, rho * m[1]);
@@ -241,6 +252,15 @@ __device__ __forceinline__ void chain_point(const StageArgs& a, const Cx& cx, co
     }
 }
 
+// the reacting flow's shared memory: T [W2] (flux form), the level items HS, then the split rows
+template <int PDE>
+__device__ __forceinline__ SplitRows split_rows(const StageArgs& a, double* sm, int W2)
+{
+    using P = Phys<PDE>;
+    int64_t* m = (int64_t*)(sm + (P::ND - P::SPLIT) * W2 + 2 * a.H * (AT_QMAX + 1) * P::ND);
+    return SplitRows{m, (uint32_t*)(m + P::SPLIT * W2), W2};
+}
+
 template <int PDE, int H, int RKS = RKS_ANY>
 __device__ __forceinline__ void central_window(const StageArgs& a, const Cx& cx, int64_t win, double* sm, int lt,
                                                int gs)
@@ -249,15 +269,16 @@ __device__ __forceinline__ void central_window(const StageArgs& a, const Cx& cx,
     constexpr int NV = P::NV;
     const int W2 = a.Tw + 2 * H;
     double* G = sm;
-    double* HS = G + P::ND * W2;
+    double* HS = G + (P::ND - P::SPLIT) * W2;
     const int64_t pe = a.wpp == 1 ? win : win / a.wpp;  // a 64-bit division only where PEs hold several windows
     const int chunk = (int)(win - pe * a.wpp);
     const int64_t t0 = pe * a.B + (int64_t)chunk * a.Tw;
     if constexpr (PDE == RNS_CHAIN) {  // one item per point: its derivatives feed all four equations
-        fill_window<PDE, false>(a, cx, G, nullptr, HS, pe, chunk, t0, W2, lt, gs);
+        const SplitRows SR = split_rows<PDE>(a, sm, W2);
+        fill_window<PDE, false>(a, cx, G, nullptr, HS, pe, chunk, t0, W2, lt, gs, nullptr, SR);
         __syncthreads();
         for (int jl = lt; jl < a.Tw; jl += gs)
-            chain_point<H, RKS>(a, cx, G, W2, pe, chunk * a.Tw + jl, t0 + jl, jl + H);
+            chain_point<H, RKS>(a, cx, SR, pe, chunk * a.Tw + jl, t0 + jl, jl + H);
         return;
     }
     const int items = NV * a.Tw;
@@ -273,7 +294,10 @@ __device__ __forceinline__ void central_window(const StageArgs& a, const Cx& cx,
         if constexpr (PDE != ADVDIFF) x0 = cx.X[idx];
         in0 = rk_load<RKS>(a, cx, idx);
     }
-    fill_window<PDE, false>(a, cx, G, nullptr, HS, pe, chunk, t0, W2, lt, gs);
+    if constexpr (PDE == RNS)
+        fill_window<PDE, false>(a, cx, G, nullptr, HS, pe, chunk, t0, W2, lt, gs, nullptr, split_rows<PDE>(a, sm, W2));
+    else
+        fill_window<PDE, false>(a, cx, G, nullptr, HS, pe, chunk, t0, W2, lt, gs);
     __syncthreads();
     for (int it = lt; it < items; it += gs) {
         const int v = it / a.Tw;
@@ -292,8 +316,8 @@ __device__ __forceinline__ void central_window(const StageArgs& a, const Cx& cx,
             for (int o = -H; o <= H; ++o) K = fma(a.cm[o + H], G[c + o], K);
             x = G[c];
         } else {
-            K = rns_flux_terms<H>(a, G, W2, v, c);
-            if (v == 3) K = fma(-a.prm[4] * x, at_exp(-a.prm[5] * at_rcpi(G[7 * W2 + c])), K);
+            K = rns_flux_terms<H>(a, split_rows<PDE>(a, sm, W2), v, c);
+            if (v == 3) K = fma(-a.prm[4] * x, at_exp(-a.prm[5] * at_rcpi(G[c])), K);
         }
         rk_update<RKS>(a, cx, v, j, chunk * a.Tw + jl, pe, K, x, in);
     }
@@ -729,7 +753,7 @@ __global__ void __launch_bounds__(128) ring_recompute(const StageArgs a, const d
 #pragma unroll
                     for (int o = -H; o <= H; ++o) K = fma(a.cm[o + H], G[lane + o], K);
                 } else {
-                    K = rns_flux_terms<H>(a, G, W, v, lane);
+                    K = rns_flux_terms<H>(a, DoubleRows{G, W}, v, lane);
                     if (v == 3) K = fma(-a.prm[4] * x[v], at_exp(-a.prm[5] * at_rcpi(G[7 * W + lane])), K);
                 }
                 // the stage-(r+1) argument as rk_update forms it
@@ -785,8 +809,8 @@ size_t atk_stage_smem_bytes(int pde, int Tw, int H)
     const size_t hs = (size_t)2 * H * (AT_QMAX + 1);  // ring-halo (point, level) items
     switch (pde) {
     case atk::ADVDIFF: return sizeof(double) * (W2 + hs * 1);
-    case atk::RNS: return sizeof(double) * (8 * W2 + hs * 8);
-    case atk::RNS_CHAIN: return sizeof(double) * (6 * W2 + hs * 6);
+    case atk::RNS: return sizeof(double) * (W2 + hs * 8 + atk::split_words(7, (int)W2));
+    case atk::RNS_CHAIN: return sizeof(double) * (hs * 6 + atk::split_words(6, (int)W2));
     // WENO: G and its first differences (2 ND W2), SP, ARR (2 W2), LAM (E),
     // the edge fluxes (NV E), HS
     case atk::EULER: return sizeof(double) * (18 * W2 + E + 4 * E + hs * 8);

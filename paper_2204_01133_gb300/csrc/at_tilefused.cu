@@ -189,7 +189,7 @@ __global__ void __launch_bounds__(256) tile_fused(const StageArgs a, const doubl
 #pragma unroll
                 for (int o = -H; o <= H; ++o) K = fma(a.cm[o + H], Gr[c + o], K);
             } else {
-                K = rns_flux_terms<H>(a, Gr, RW, v, c);
+                K = rns_flux_terms<H>(a, DoubleRows{const_cast<double*>(Gr), RW}, v, c);
                 if (v == 3) K = fma(-a.prm[4] * x, at_exp(-a.prm[5] * at_rcpi(Gr[7 * RW + c])), K);
             }
             double acc = AC[v * E + i];

@@ -19,7 +19,7 @@ def lib(tmp_path_factory):
     d = tmp_path_factory.mktemp("fixed")
     src = d / "f.cpp"
     src.write_text('#include "at_fixed.cuh"\nextern "C" {\n' + "".join(
-        "double d%d_%d(const double* f) { return atk::fx_d%d<%d>(f + %d); }\n" % (k, h, k, h, h)
+        "double d%d_%d(const double* f) { return atk::fx_d%d<%d>(atk::FxDoubles{f + %d}); }\n" % (k, h, k, h, h)
         for k in (1, 2) for h in (1, 2, 3)) + "}\n")
     so = str(d / "f.so")
     subprocess.run(["g++", "-O2", "-std=c++17", "-ffp-contract=off", "-shared", "-fPIC", "-I", CSRC, str(src), "-o", so],
