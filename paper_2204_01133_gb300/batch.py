@@ -89,9 +89,8 @@ class Batch:
         if init is not None:
             src = init if isinstance(init, torch.Tensor) else torch.from_numpy(np.ascontiguousarray(init))
             state.copy_(src.reshape(nvar, n))
-        nb = api.workspace_bytes(pb)
         if workspace is None:
-            workspace = torch.empty(nb, dtype=torch.uint8, device=self.device)
+            workspace = torch.empty(api.workspace_bytes(pb), dtype=torch.uint8, device=self.device)
         inst = Instance()
         inst.pb = api.problem_struct(pb)
         inst.dl = api.delays_struct(pb)

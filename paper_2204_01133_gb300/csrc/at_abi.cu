@@ -23,7 +23,7 @@
 size_t atk_stage_smem_bytes(int pde, int Tw, int H);
 int atk_stage_block(int pde, int Tw);
 cudaError_t atk_launch_stage(const atk::StageArgs& a, int pde, int order, int sms, cudaStream_t st);
-cudaError_t atk_launch_ring_seed(const atk::StageArgs& a, cudaStream_t st);
+cudaError_t atk_launch_reset(const atk::StageArgs& a, const atk::ResetArgs& z, cudaStream_t st);
 cudaError_t atk_launch_ring_recompute(const atk::StageArgs& a, int pde, int order, int rk, const double* um,
                                       int64_t m, cudaStream_t st);
 cudaError_t atk_set_smem_limits();
@@ -406,6 +406,7 @@ struct at_ctx {
     int64_t persist_cap = 0;       // PEs one cooperative launch can hold (0: unavailable)
     int cluster_c = 0;             // CTAs of the one-cluster kernel for this problem (0: not used)
     int sms = 0;                   // SMs of the device
+    int64_t fit_key[8] = {-1};     // what the capacities below were asked for
     int stage_tw = 0;              // window length of the per-stage kernels (stage_window)
     int fused_multi_w = 0;         // PEs per CTA when the fused path's steps fit one cooperative launch
     int64_t wait_limit = 4000000;  // polls of a bounded wait
@@ -550,33 +551,39 @@ int at_set_delays(at_ctx* c, const at_delays* dl)
     c->base.wait_limit = c->wait_limit;
     c->base.withhold_pe = c->withhold_pe;
     atk::StageArgs& a = c->base;
-    // reset the run: zero ring, delay log and status, then seed level 0
-    e = cudaMemsetAsync(a.ring, 0, sizeof(double) * L.ring_elems, c->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(a.dlog, 0, (size_t)L.S * L.P * 2, c->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(a.status, 0, 2 * sizeof(int), c->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(a.ext, 0, sizeof(double) * L.ext_elems, c->stream);
-    for (int g = 0; g < L.nguard && e == cudaSuccess; ++g)
-        e = cudaMemsetAsync(c->ws + L.guard[g], kGuardByte, kGuardBytes, c->stream);
-    if (e != cudaSuccess) return cuda_fail(e, "workspace reset");
+    // reset the run: zero ring, delay log and status, seed level 0
     c->stage_pos = 0;
     atk::StageArgs s = a;
     s.u = c->state;
-    e = atk_launch_ring_seed(s, c->stream);
-    if (e != cudaSuccess) return cuda_fail(e, "ring seed launch");
+    atk::ResetArgs z{};
+    z.ring_elems = (int64_t)L.ring_elems;
+    z.ext_elems = (int64_t)L.ext_elems;
+    z.ws = c->ws;
+    z.nguard = L.nguard;
+    for (int g = 0; g < L.nguard; ++g) z.guard[g] = L.guard[g];
+    z.guard_word = kGuardByte * 0x01010101u;
+    e = atk_launch_reset(s, z, c->stream);
+    if (e != cudaSuccess) return cuda_fail(e, "reset launch");
     c->level = 0;
     c->hist_level = -1;  // reading A recomputes level 0 at the first at_step
-    if (c->sms == 0) cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device);
-    c->stage_tw = stage_window(&c->pb, L, c->sms);
-    c->persist_cap = (c->pb.pde == AT_ADVDIFF || c->pb.pde == AT_RNS)
-                         ? atk_persist_capacity(c->pb.pde, c->pb.order, c->pb.pe_size, c->device)
-                         : 0;
-    if (c->persist_cap > kPersistMaxPE) c->persist_cap = kPersistMaxPE;
-    c->cluster_c = c->pb.pde == AT_ADVDIFF
-                       ? atk_cluster_size(c->pb.pde, c->pb.order, c->pb.pe_size, L.P, L.R, L.S, c->device)
-                       : 0;
-    c->fused_multi_w = atk_fused_supported(c->pb.pde, c->pb.order, c->pb.pe_size, L.S)
-                           ? atk_fused_multi_w(c->pb.order, c->pb.rk, c->pb.pe_size, L.S, L.P, c->device)
+    // what fits on the device depends on these alone: asked again only when one
+    // of them changes (the occupancy queries take some tens of microseconds)
+    const int64_t key[8] = {c->pb.pde, c->pb.order, c->pb.rk, c->pb.pe_size, c->pb.n, c->pb.weno, L.R, L.S};
+    if (std::memcmp(key, c->fit_key, sizeof key) != 0) {
+        if (c->sms == 0) cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device);
+        c->stage_tw = stage_window(&c->pb, L, c->sms);
+        c->persist_cap = (c->pb.pde == AT_ADVDIFF || c->pb.pde == AT_RNS)
+                             ? atk_persist_capacity(c->pb.pde, c->pb.order, c->pb.pe_size, c->device)
+                             : 0;
+        if (c->persist_cap > kPersistMaxPE) c->persist_cap = kPersistMaxPE;
+        c->cluster_c = c->pb.pde == AT_ADVDIFF
+                           ? atk_cluster_size(c->pb.pde, c->pb.order, c->pb.pe_size, L.P, L.R, L.S, c->device)
                            : 0;
+        c->fused_multi_w = atk_fused_supported(c->pb.pde, c->pb.order, c->pb.pe_size, L.S)
+                               ? atk_fused_multi_w(c->pb.order, c->pb.rk, c->pb.pe_size, L.S, L.P, c->device)
+                               : 0;
+        std::memcpy(c->fit_key, key, sizeof key);
+    }
     cudaGetLastError();  // an unavailable persistent path is not an error
     c->have_delays = true;
     g_err[0] = 0;
@@ -1268,7 +1275,6 @@ struct at_batch {
     std::vector<int> variant, bound;
     std::vector<size_t> smem;
     std::vector<int> order_h, slots_h, status_h;
-    std::vector<int64_t> lvl_h, left_h;  // staging for uploads
     int group_begin[kVariants + 1] = {0};
     size_t group_smem[kVariants] = {0};
     std::vector<int> wslot_h, widx_h;
@@ -1432,8 +1438,6 @@ int at_batch_create(at_batch** out, int device, void* cuda_stream, int64_t capac
     b->bound.assign(capacity, 0);
     b->smem.assign(capacity, 0);
     b->windows.assign(capacity, 0);
-    b->lvl_h.assign(capacity, 0);
-    b->left_h.assign(capacity, 0);
     e = cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming);
     for (int g = 0; g < kVariants && e == cudaSuccess; ++g) {
@@ -1473,22 +1477,14 @@ int at_batch_bind(at_batch* b, int64_t slot, const at_instance* in)
     cudaError_t e = cudaSetDevice(b->device);
     if (e != cudaSuccess) return cuda_fail(e, "cudaSetDevice");
     atk::StageArgs a = build_args(&in->pb, &in->dl, L, (unsigned char*)in->workspace_dev, in->state_dev);
-    e = cudaMemsetAsync(a.ring, 0, sizeof(double) * L.ring_elems, b->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(a.dlog, 0, (size_t)L.S * L.P * 2, b->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(a.status, 0, 2 * sizeof(int), b->stream);
-    if (e == cudaSuccess) e = atk_launch_ring_seed(a, b->stream);
     b->args[slot] = a;
-    b->lvl_h[slot] = 0;
-    b->left_h[slot] = in->nsteps;
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(b->tab + b->T.off_args + sizeof(atk::StageArgs) * slot, &b->args[slot],
-                            sizeof(atk::StageArgs), cudaMemcpyHostToDevice, b->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(b->tab + b->T.off_lvl + sizeof(int64_t) * slot, &b->lvl_h[slot], sizeof(int64_t),
-                            cudaMemcpyHostToDevice, b->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(b->tab + b->T.off_left + sizeof(int64_t) * slot, &b->left_h[slot], sizeof(int64_t),
-                            cudaMemcpyHostToDevice, b->stream);
+    atk::ResetArgs z{};
+    z.ring_elems = (int64_t)L.ring_elems;
+    z.slot_args = (atk::StageArgs*)(b->tab + b->T.off_args) + slot;
+    z.slot_level = (int64_t*)(b->tab + b->T.off_lvl) + slot;
+    z.slot_left = (int64_t*)(b->tab + b->T.off_left) + slot;
+    z.nsteps = in->nsteps;
+    e = atk_launch_reset(a, z, b->stream);
     if (e != cudaSuccess) return cuda_fail(e, "batch bind");
     b->level[slot] = 0;
     b->left[slot] = in->nsteps;

@@ -80,6 +80,17 @@ struct StageArgs {
     double* state;
 };
 
+// what a solve's reset takes besides its StageArgs
+struct ResetArgs {
+    int64_t ring_elems, ext_elems;
+    unsigned char* ws;    // canary zones of 256 bytes at ws + guard[i]
+    size_t guard[10];
+    int nguard;
+    uint32_t guard_word;
+    StageArgs* slot_args; // a batch slot's table entries (null: none)
+    int64_t *slot_level, *slot_left, nsteps;
+};
+
 // ---------------------------------------------------------------------------
 // Philox4x32-10 (Salmon et al., SC'11): ten rounds of two 32x32->64 products
 // with a Weyl key schedule; only output word 0 is used.
