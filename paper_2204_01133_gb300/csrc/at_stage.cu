@@ -624,7 +624,7 @@ __global__ void __launch_bounds__(256) batch_run(const StageArgs* __restrict__ t
 // of one CTA, as on the per-stage path.
 constexpr int AT_BATCH_WIN_MASK = 0x3fffffff;
 template <int PDE, int H, bool WENO>
-__global__ void __launch_bounds__(256, 4) batch_stage(const StageArgs* __restrict__ tab, const int64_t* __restrict__ lvl,
+__global__ void __launch_bounds__(256, PDE == RNS ? 5 : 4) batch_stage(const StageArgs* __restrict__ tab, const int64_t* __restrict__ lvl,
                                                    const int64_t* __restrict__ left, const int* __restrict__ win_slot,
                                                    const int* __restrict__ win_idx, int stage, int win_smem)
 {
