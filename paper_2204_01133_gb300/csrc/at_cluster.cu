@@ -53,10 +53,6 @@ __global__ void __launch_bounds__(256) cluster_advdiff(const StageArgs a, int64_
     double* ACC = X + 2 * m * B;                    // RK accumulator               [m][B]
     double* W = ACC + m * B;                        // stencil row of each warp     [m * WPP][SW + 2H]
     double* RING = W + m * WPP * (SW + 2 * H);      // edge windows                 [R][S][m][2][H]
-    auto ridx = [&](int64_t level, int stage, int l, int side, int h) {
-        const int r = (int)((uint32_t)level % (uint32_t)R);
-        return (((r * S + stage) * m + l) * 2 + side) * H + h;
-    };
     for (int i = threadIdx.x; i < m * B; i += blockDim.x) {
         const int l = i / B, j = i - l * B;
         const double x = a.u[(int64_t)blockIdx.x * m * B + (int64_t)l * B + j];
@@ -83,32 +79,58 @@ __global__ void __launch_bounds__(256) cluster_advdiff(const StageArgs a, int64_
     const int64_t nbr = side == 0 ? (pe == 0 ? a.P - 1 : pe - 1) : (pe == a.P - 1 ? 0 : pe + 1);
     const int rank = (int)(nbr / m), nl = (int)(nbr - (int64_t)rank * m);
     const double* src = rank == (int)blockIdx.x ? RING : cl.map_shared_rank(RING, rank);
+    // Lane s H' + i of a warp with buffer points draws the delay of its side at
+    // stage s and forms its point's value where the delay is 1 or more, for all
+    // stages of a step at once (H' = 2 H points on a one-warp PE, else H): those
+    // levels are a step old.  S H' <= 24 lanes.
+    const int HB = WPP == 1 ? 2 * H : H;
+    const bool pre = (WPP == 1 || hw == 0 || hw == WPP - 1) && lane < S * HB;
+    const int ps = lane / HB, pi = lane - ps * HB;
+    const int pside = WPP == 1 ? (pi < H ? 0 : 1) : side, ph = WPP == 1 ? pi - pside * H : pi;
+    const int64_t pnbr = pside == 0 ? (pe == 0 ? a.P - 1 : pe - 1) : (pe == a.P - 1 ? 0 : pe + 1);
+    const int prank = (int)(pnbr / m), pnl = (int)(pnbr - (int64_t)prank * m);
+    const double* psrc = prank == (int)blockIdx.x ? RING : cl.map_shared_rank(RING, prank);
     bool bad = false;
     int par = 0;  // parity of the stage argument this stage reads
+    int r0 = (int)((uint32_t)level0 % (uint32_t)R);  // ring slot of level n
     for (int64_t n = level0; n < level0 + nsteps; ++n) {
+        const int r1 = r0 + 1 == R ? 0 : r0 + 1;
+        const bool log = a.trace || n == level0 + nsteps - 1;  // the log keeps the last step's delays
+        int pk = 0;
+        double pv = 0.0;
         for (int s = 0; s < S; ++s) {
             const bool last = (s == S - 1);
-            const int64_t Ln = last ? n + 1 : n;
+            const int rn = last ? r1 : r0;
             const int sn = last ? 0 : s + 1;
             const double* Xc = X + par * m * B + lp * B;      // this stage's argument of the PE
             double* Xn = X + (1 - par) * m * B + lp * B;      // the next one
-            // Before the previous stage's cluster barrier completes: the delays,
-            // the neighbour's levels for delays k >= 1 (written at least a step
-            // ago, and their slots are not written in the stage in flight) and
-            // the warp's own points of the stencil row (written by the same
-            // lanes in the previous stage).
-            int k = 0;
-            double bv = 0.0;
-            double v[AT_QMAX + 1];
-            if (buf) {
-                k = keff_at(a, n, s, pe, side);
-                if (h == 0) log_delay(a, n, s, pe, side, k);
+            // Before the previous stage's cluster barrier completes: at the first
+            // stage the step's delays and the neighbour's levels for delays k >= 1
+            // (stage s of level n - 1 was written by stage s - 1 of that step, at
+            // least a barrier ago, and their slots are not written in the stage in
+            // flight), and the warp's own points of the stencil row (written by
+            // the same lanes in the previous stage).
+            if (s == 0 && pre) {
+                pk = keff_at(a, n, ps, pe, pside);
+                if (ph == 0 && log) log_delay(a, n, ps, pe, pside, pk);
+                if (pk >= 1) {
+                    double v[AT_QMAX + 1];
 #pragma unroll
-                for (int l = 0; l <= AT_QMAX; ++l) {
-                    v[l] = 0.0;  // a level with weight 0 is not part of the scheme (and may not exist yet)
-                    if (k >= 1 && l < nw && ((a.wnz[k] >> l) & 1)) v[l] = src[ridx(n - k - l, s, nl, 1 - side, h)];
+                    for (int l = 0; l <= AT_QMAX; ++l) {
+                        v[l] = 0.0;  // a level with weight 0 is not part of the scheme (and may not exist yet)
+                        int r = r0 - pk - l;
+                        if (r < 0) r += R;
+                        if (l < nw && ((a.wnz[pk] >> l) & 1))
+                            v[l] = psrc[(((r * S + ps) * m + pnl) * 2 + 1 - pside) * H + ph];
+                    }
+                    pv = ((a.mode == AT) ? a.w[pk][0] : 1.0) * v[0];
+#pragma unroll
+                    for (int l = 1; l <= AT_QMAX; ++l)
+                        if (l < nw) pv = fma(a.w[pk][l], v[l], pv);
                 }
             }
+            const int k = __shfl_sync(0xffffffffu, pk, (s * HB + lane) & 31);
+            double bv = __shfl_sync(0xffffffffu, pv, (s * HB + lane) & 31);
 #pragma unroll
             for (int i = 0; i < PPW; ++i) Wr[H + lane + 32 * i] = Xc[j0 + lane + 32 * i];
             // every CTA's ring writes and the other warps' stage arguments of the
@@ -119,13 +141,7 @@ __global__ void __launch_bounds__(256) cluster_advdiff(const StageArgs a, int64_
                 // so the extrapolation is this level's value, just written, up to
                 // the sign of a zero; the stencil sum starts from +0, where a zero
                 // adds nothing whatever its sign (bitwise the per-stage results)
-                if (k == 0) bv = src[ridx(n, s, nl, 1 - side, h)];
-                else {
-                    bv = ((a.mode == AT) ? a.w[k][0] : 1.0) * v[0];
-#pragma unroll
-                    for (int l = 1; l <= AT_QMAX; ++l)
-                        if (l < nw) bv = fma(a.w[k][l], v[l], bv);
-                }
+                if (k == 0) bv = src[(((r0 * S + s) * m + nl) * 2 + 1 - side) * H + h];
                 Wr[side == 0 ? h : H + SW + h] = bv;
             }
             if (halo_l) Wr[lane] = Xc[j0 - H + lane];
@@ -167,13 +183,14 @@ __global__ void __launch_bounds__(256) cluster_advdiff(const StageArgs a, int64_
                 Xn[j] = y;
                 if (last) U[it] = y;
                 if (nonfinite(y)) bad = true;
-                if (j < H) RING[ridx(Ln, sn, lp, 0, j)] = y;
-                else if (j >= B - H) RING[ridx(Ln, sn, lp, 1, j - (B - H))] = y;
+                if (j < H) RING[((rn * S + sn) * m + lp) * 2 * H + j] = y;
+                else if (j >= B - H) RING[(((rn * S + sn) * m + lp) * 2 + 1) * H + j - (B - H)] = y;
             }
             __syncwarp();  // the row is read by all lanes before the next stage rewrites it
             cl.barrier_arrive();  // this stage's ring and stage-argument writes done: release to the cluster
             par = 1 - par;
         }
+        r0 = r1;
     }
     if (nsteps > 0) cl.barrier_wait();  // no CTA leaves while another may still read its ring
     for (int i = threadIdx.x; i < m * B; i += blockDim.x) {
