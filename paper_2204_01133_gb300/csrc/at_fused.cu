@@ -84,9 +84,18 @@ __device__ __forceinline__ double fused_buffer_old(const StageArgs& a, int64_t n
 // one warp instruction for all stages and both sides of a PE; a stage only
 // reads shared memory, and fills a k = 0 buffer point with the neighbour's
 // stage argument itself (no FP64 instruction).
-template <int H, int PPL, int RK, int W>
-__device__ __forceinline__ void fused_step(const StageArgs& a, const double* __restrict__ uin,
-                                           double* __restrict__ uout, int64_t n, double* sm, int64_t cta)
+//
+// In a launch of many steps (MULTI) the PE warps keep u^n in registers (x) from
+// step to step, only what the neighbours read goes out before the last step
+// (`final`), and wait(side) blocks the calling lane until the neighbour CTA on
+// that side has finished step n-1: only the warps that read something of that
+// CTA call it, while the others draw their delays and fill their rows.  A wait
+// that fails raises *fail before the step's first barrier; every thread then
+// returns false from there.
+template <int H, int PPL, int RK, int W, bool MULTI, class WAIT>
+__device__ __forceinline__ bool fused_step(const StageArgs& a, const double* __restrict__ uin,
+                                           double* __restrict__ uout, int64_t n, double* sm, int64_t cta,
+                                           double (&x)[PPL], bool final, bool log, int* fail, WAIT wait)
 {
     constexpr int B = 32 * PPL;
     constexpr int S = RkS<RK>::S;
@@ -112,11 +121,11 @@ __device__ __forceinline__ void fused_step(const StageArgs& a, const double* __r
         // ---------------- PE warps ----------------
         const bool active = wid < nW;
         const int64_t pe = p0 + wid;
-        double x[PPL], un[PPL], ac[PPL];
+        double un[PPL], ac[PPL];
         if (active) {
 #pragma unroll
             for (int i = 0; i < PPL; ++i) {
-                const double v = uin[pe * B + lane + 32 * i];
+                const double v = MULTI ? x[i] : uin[pe * B + lane + 32 * i];
                 x[i] = v;
                 un[i] = v;
                 ac[i] = 0.0;
@@ -131,10 +140,13 @@ __device__ __forceinline__ void fused_step(const StageArgs& a, const double* __r
             const int64_t nb = side == 0 ? (pe == 0 ? P - 1 : pe - 1) : (pe == P - 1 ? 0 : pe + 1);
             const int k = keff_at(a, n, s, pe, side);
             if (h == 0) {
-                log_delay(a, n, s, pe, side, k);
+                if (log) log_delay(a, n, s, pe, side, k);
                 KS[(wid * S + s) * 2 + side] = k;
             }
-            if (k >= 1) BV[((wid * S + s) * 2 + side) * H + h] = fused_buffer_old(a, n, s, k, nb, 1 - side, h);
+            bool ok = true;  // the levels of a PE of the next CTA
+            if (MULTI && k >= 1 && (side == 0 ? wid == 0 : wid == nW - 1)) ok = wait(side);
+            if (!ok) *fail = 1;
+            if (k >= 1 && ok) BV[((wid * S + s) * 2 + side) * H + h] = fused_buffer_old(a, n, s, k, nb, 1 - side, h);
         }
         // buffer lanes of the stages: left side on lanes 0..H-1, right side on H..2H-1
         const bool buf = active && lane < 2 * H;
@@ -147,6 +159,7 @@ __device__ __forceinline__ void fused_step(const StageArgs& a, const double* __r
             double* R1 = ROW + (par ^ 1) * W * RW;
             double* Rw = R0 + wid * RW;
             __syncthreads();  // the stage arguments of stage s, of every warp and strip
+            if (MULTI && s == 0 && *(volatile int*)fail) return false;
             if (buf) {
                 const int k = KS[(wid * S + s) * 2 + side];
                 // k = 0: the neighbour's stage argument at the point facing this
@@ -180,9 +193,9 @@ __device__ __forceinline__ void fused_step(const StageArgs& a, const double* __r
                         a.ring[ring_index(a, last ? n + 1 : n, last ? 0 : s + 1, pe, 0, j, 0)] = y;
                     else if (j >= B - H)
                         a.ring[ring_index(a, last ? n + 1 : n, last ? 0 : s + 1, pe, 1, j - (B - H), 0)] = y;
-                    if (last)
-                        uout[pe * B + j] = y;
-                    else
+                    if (last) {  // before the last step only the neighbours' strips read it
+                        if (!MULTI || final || j < D || j >= B - D) uout[pe * B + j] = y;
+                    } else
                         R1[wid * RW + H + j] = y;
                     x[i] = y;
                 }
@@ -197,6 +210,11 @@ __device__ __forceinline__ void fused_step(const StageArgs& a, const double* __r
         const int sl = lane & 15;          // lane within the strip
         const int64_t spe = st == 0 ? pl : pr;
         const int64_t soff = st == 0 ? (int64_t)(B - D) : 0;  // first strip point within spe
+        if (MULTI) {
+            const bool ok = sl == 0 ? wait(st) : true;
+            if (!ok) *fail = 1;
+            __syncwarp();
+        }
         if (sl < D) {
             const double v = __ldcg(uin + spe * B + soff + sl);  // written by another CTA
             SUN[st * D + sl] = v;
@@ -222,6 +240,7 @@ __device__ __forceinline__ void fused_step(const StageArgs& a, const double* __r
             double* Rs = SROW + (par * 2 + st) * SW;
             double* Rn = SROW + ((par ^ 1) * 2 + st) * SW;
             __syncthreads();
+            if (MULTI && s == 0 && *(volatile int*)fail) return false;
             if (buf) {
                 const int k = SKS[st * (S - 1) + s];
                 double b;
@@ -249,6 +268,7 @@ __device__ __forceinline__ void fused_step(const StageArgs& a, const double* __r
         // the PE warps' last stage has one more barrier
         __syncthreads();
     }
+    return true;
 }
 
 // one step n: u^n from uin, u^{n+1} to uout
@@ -257,7 +277,9 @@ __global__ void __launch_bounds__(32 * (W + 1)) step_fused_advdiff(const StageAr
                                                                    double* __restrict__ uout, int64_t n)
 {
     extern __shared__ double sm[];
-    fused_step<H, PPL, RK, W>(a, uin, uout, n, sm, blockIdx.x);
+    double x[PPL];
+    fused_step<H, PPL, RK, W, false>(a, uin, uout, n, sm, blockIdx.x, x, true, true, nullptr,
+                                     [](int) { return true; });
 }
 
 __device__ __forceinline__ int64_t fused_load_acquire(int64_t* p)
@@ -308,14 +330,20 @@ __global__ void __launch_bounds__(32 * (W + 1)) steps_fused_advdiff(const StageA
     const int64_t C = gridDim.x, c = place_rank(a);  // CTA c takes PEs c W .. c W + W - 1
     const int64_t cl = c == 0 ? C - 1 : c - 1, cr = c == C - 1 ? 0 : c + 1;
     const bool withheld = a.withhold_pe >= 0 && a.withhold_pe / W == c;  // fault injection: never publishes
+    if (threadIdx.x == 0) s_fail = 0;
+    double x[PPL];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int64_t pe = c * W + wid;
+#pragma unroll
+    for (int i = 0; i < PPL; ++i) x[i] = wid < W && pe < a.P ? b0[pe * (32 * PPL) + lane + 32 * i] : 0.0;
+    __syncthreads();
     for (int64_t i = 0; i < nsteps; ++i) {
         const int64_t n = level0 + i;
-        if (i > 0) {
-            if (threadIdx.x == 0) s_fail = (fused_wait_ge(a, a.done + cl, n) && fused_wait_ge(a, a.done + cr, n)) ? 0 : 1;
-            __syncthreads();
-            if (s_fail) break;
-        }
-        fused_step<H, PPL, RK, W>(a, (i & 1) ? b1 : b0, (i & 1) ? b0 : b1, n, sm, c);
+        const bool final = i == nsteps - 1;
+        const bool ok = fused_step<H, PPL, RK, W, true>(
+            a, (i & 1) ? b1 : b0, (i & 1) ? b0 : b1, n, sm, c, x, final, final || a.trace, &s_fail,
+            [&](int side) { return i == 0 || fused_wait_ge(a, a.done + (side == 0 ? cl : cr), n); });
+        if (!ok) break;
         __syncthreads();  // every thread's writes of step n
         if (threadIdx.x == 0 && !withheld) {
             __threadfence();

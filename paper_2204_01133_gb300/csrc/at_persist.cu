@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(288, 2) persist_central(const StageArgs a, int
             int k = 0;
             if (lane < 2 && !a.arrival) {
                 k = keff_at(a, n, s, pe, lane);
-                log_delay(a, n, s, pe, lane, k);
+                if (a.trace || n == level0 + nsteps - 1) log_delay(a, n, s, pe, lane, k);  // the log keeps the last step
             }
             if (t >= 2) bar_sync_p<3>(p, nall);  // the workers are done with G[p] (stage t - 2)
             bool ok = true;
