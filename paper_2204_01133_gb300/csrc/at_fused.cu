@@ -92,10 +92,14 @@ __device__ __forceinline__ double fused_buffer_old(const StageArgs& a, int64_t n
 // CTA call it, while the others draw their delays and fill their rows.  A wait
 // that fails raises *fail before the step's first barrier; every thread then
 // returns false from there.
-template <int H, int PPL, int RK, int W, bool MULTI, class WAIT>
+//
+// A PE takes WPP warps, PPL / WPP points a lane; its row is complete at the
+// barrier that opens a stage, and each side's buffer points belong to the warp
+// that has the points beside them.
+template <int H, int PPL, int RK, int W, int WPP, bool MULTI, class WAIT>
 __device__ __forceinline__ bool fused_step(const StageArgs& a, const double* __restrict__ uin,
                                            double* __restrict__ uout, int64_t n, double* sm, int64_t cta,
-                                           double (&x)[PPL], bool final, bool log, int* fail, WAIT wait)
+                                           double (&x)[PPL / WPP], bool final, bool log, int* fail, WAIT wait)
 {
     constexpr int B = 32 * PPL;
     constexpr int S = RkS<RK>::S;
@@ -117,64 +121,68 @@ __device__ __forceinline__ bool fused_step(const StageArgs& a, const double* __r
     const int64_t pr = p0 + nW == P ? 0 : p0 + nW;
     const int64_t plast = p0 + nW - 1;
 
-    if (wid < W) {
+    if (wid < W * WPP) {
         // ---------------- PE warps ----------------
-        const bool active = wid < nW;
-        const int64_t pe = p0 + wid;
-        double un[PPL], ac[PPL];
+        constexpr int PPW = PPL / WPP;
+        const int pw = wid / WPP, hw = wid - pw * WPP;  // PE of the CTA, warp of the PE
+        const int j0 = 32 * PPW * hw;                    // the warp's first point
+        const bool active = pw < nW;
+        const int64_t pe = p0 + pw;
+        double un[PPW], ac[PPW];
         if (active) {
 #pragma unroll
-            for (int i = 0; i < PPL; ++i) {
-                const double v = MULTI ? x[i] : uin[pe * B + lane + 32 * i];
+            for (int i = 0; i < PPW; ++i) {
+                const double v = MULTI ? x[i] : uin[pe * B + j0 + lane + 32 * i];
                 x[i] = v;
                 un[i] = v;
                 ac[i] = 0.0;
-                ROW[wid * RW + H + lane + 32 * i] = v;
+                ROW[pw * RW + H + j0 + lane + 32 * i] = v;
             }
         }
         // the delays of every stage and the buffer values of delays >= 1: lane
         // e < 2 S H takes stage e / 2H, side (e / H) % 2, point e % H of the
         // edge window
-        if (active && lane < 2 * S * H) {
+        if (active && hw == 0 && lane < 2 * S * H) {
             const int s = lane / (2 * H), side = (lane / H) & 1, h = lane % H;
             const int64_t nb = side == 0 ? (pe == 0 ? P - 1 : pe - 1) : (pe == P - 1 ? 0 : pe + 1);
             const int k = keff_at(a, n, s, pe, side);
             if (h == 0) {
                 if (log) log_delay(a, n, s, pe, side, k);
-                KS[(wid * S + s) * 2 + side] = k;
+                KS[(pw * S + s) * 2 + side] = k;
             }
             bool ok = true;  // the levels of a PE of the next CTA
-            if (MULTI && k >= 1 && (side == 0 ? wid == 0 : wid == nW - 1)) ok = wait(side);
+            if (MULTI && k >= 1 && (side == 0 ? pw == 0 : pw == nW - 1)) ok = wait(side);
             if (!ok) *fail = 1;
-            if (k >= 1 && ok) BV[((wid * S + s) * 2 + side) * H + h] = fused_buffer_old(a, n, s, k, nb, 1 - side, h);
+            if (k >= 1 && ok) BV[((pw * S + s) * 2 + side) * H + h] = fused_buffer_old(a, n, s, k, nb, 1 - side, h);
         }
-        // buffer lanes of the stages: left side on lanes 0..H-1, right side on H..2H-1
-        const bool buf = active && lane < 2 * H;
-        const int side = lane < H ? 0 : 1;
-        const int h = lane - side * H;
+        // buffer lanes of the stages: left side on lanes 0..H-1, right side on
+        // H..2H-1; with several warps a PE on lanes 0..H-1 of its first and last
+        const bool buf = active && (WPP == 1 ? lane < 2 * H : lane < H && (hw == 0 || hw == WPP - 1));
+        const int side = WPP == 1 ? (lane < H ? 0 : 1) : (hw == 0 ? 0 : 1);
+        const int h = WPP == 1 ? lane - side * H : lane;
 #pragma unroll
         for (int s = 0; s < S; ++s) {
             const int par = s & 1;
             double* R0 = ROW + par * W * RW;
             double* R1 = ROW + (par ^ 1) * W * RW;
-            double* Rw = R0 + wid * RW;
+            double* Rw = R0 + pw * RW;
             __syncthreads();  // the stage arguments of stage s, of every warp and strip
             if (MULTI && s == 0 && *(volatile int*)fail) return false;
             if (buf) {
-                const int k = KS[(wid * S + s) * 2 + side];
+                const int k = KS[(pw * S + s) * 2 + side];
                 // k = 0: the neighbour's stage argument at the point facing this
                 // PE (its point B-H+h on the left, h on the right)
                 double b;
                 if (k == 0) {
                     double cur;
                     if (side == 0)
-                        cur = wid > 0 ? R0[(wid - 1) * RW + H + B - H + h]
+                        cur = pw > 0 ? R0[(pw - 1) * RW + H + B - H + h]
                                       : SROW[(par * 2 + 0) * SW + H + D - H + h];
                     else
-                        cur = wid < nW - 1 ? R0[(wid + 1) * RW + H + h] : SROW[(par * 2 + 1) * SW + H + h];
+                        cur = pw < nW - 1 ? R0[(pw + 1) * RW + H + h] : SROW[(par * 2 + 1) * SW + H + h];
                     b = fused_extrap_cur(cur);
                 } else {
-                    b = BV[((wid * S + s) * 2 + side) * H + h];
+                    b = BV[((pw * S + s) * 2 + side) * H + h];
                 }
                 Rw[side == 0 ? h : H + B + h] = b;
             }
@@ -182,8 +190,8 @@ __device__ __forceinline__ bool fused_step(const StageArgs& a, const double* __r
             if (active) {
                 const bool last = s == S - 1;
 #pragma unroll
-                for (int i = 0; i < PPL; ++i) {
-                    const int j = lane + 32 * i;
+                for (int i = 0; i < PPW; ++i) {
+                    const int j = j0 + lane + 32 * i;
                     double K = 0.0;
 #pragma unroll
                     for (int o = -H; o <= H; ++o) K = fma(a.cm[o + H], Rw[H + j + o], K);
@@ -196,7 +204,7 @@ __device__ __forceinline__ bool fused_step(const StageArgs& a, const double* __r
                     if (last) {  // before the last step only the neighbours' strips read it
                         if (!MULTI || final || j < D || j >= B - D) uout[pe * B + j] = y;
                     } else
-                        R1[wid * RW + H + j] = y;
+                        R1[pw * RW + H + j] = y;
                     x[i] = y;
                 }
             }
@@ -278,7 +286,7 @@ __global__ void __launch_bounds__(32 * (W + 1)) step_fused_advdiff(const StageAr
 {
     extern __shared__ double sm[];
     double x[PPL];
-    fused_step<H, PPL, RK, W, false>(a, uin, uout, n, sm, blockIdx.x, x, true, true, nullptr,
+    fused_step<H, PPL, RK, W, 1, false>(a, uin, uout, n, sm, blockIdx.x, x, true, true, nullptr,
                                      [](int) { return true; });
 }
 
@@ -320,8 +328,11 @@ __device__ bool fused_wait_ge(const StageArgs& a, int64_t* ctr, int64_t target)
 // buffer that held u^{n-1}, which the neighbours read during their step n-1,
 // and the ring slots of levels n and n+1, which no CTA at step n or n+1 reads
 // (the CTAs are at most one step apart, the ring keeps k_max + q + 3 levels).
+// warps per PE of the multi-step kernel with W PEs a CTA
+__host__ __device__ constexpr int steps_wpp(int W, int ppl) { return W == 2 && ppl >= 2 ? 2 : 1; }
+
 template <int H, int PPL, int RK, int W>
-__global__ void __launch_bounds__(32 * (W + 1)) steps_fused_advdiff(const StageArgs a, double* __restrict__ b0,
+__global__ void __launch_bounds__(32 * (W * steps_wpp(W, PPL) + 1)) steps_fused_advdiff(const StageArgs a, double* __restrict__ b0,
                                                                     double* __restrict__ b1, int64_t level0,
                                                                     int64_t nsteps)
 {
@@ -331,16 +342,18 @@ __global__ void __launch_bounds__(32 * (W + 1)) steps_fused_advdiff(const StageA
     const int64_t cl = c == 0 ? C - 1 : c - 1, cr = c == C - 1 ? 0 : c + 1;
     const bool withheld = a.withhold_pe >= 0 && a.withhold_pe / W == c;  // fault injection: never publishes
     if (threadIdx.x == 0) s_fail = 0;
-    double x[PPL];
+    constexpr int WPP = steps_wpp(W, PPL), PPW = PPL / WPP;
+    double x[PPW];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int64_t pe = c * W + wid;
+    const int64_t pe = c * W + wid / WPP;
 #pragma unroll
-    for (int i = 0; i < PPL; ++i) x[i] = wid < W && pe < a.P ? b0[pe * (32 * PPL) + lane + 32 * i] : 0.0;
+    for (int i = 0; i < PPW; ++i)
+        x[i] = wid < W * WPP && pe < a.P ? b0[pe * (32 * PPL) + 32 * PPW * (wid % WPP) + lane + 32 * i] : 0.0;
     __syncthreads();
     for (int64_t i = 0; i < nsteps; ++i) {
         const int64_t n = level0 + i;
         const bool final = i == nsteps - 1;
-        const bool ok = fused_step<H, PPL, RK, W, true>(
+        const bool ok = fused_step<H, PPL, RK, W, WPP, true>(
             a, (i & 1) ? b1 : b0, (i & 1) ? b0 : b1, n, sm, c, x, final, final || a.trace, &s_fail,
             [&](int side) { return i == 0 || fused_wait_ge(a, a.done + (side == 0 ? cl : cr), n); });
         if (!ok) break;
@@ -398,7 +411,7 @@ void* fused_fn(int H, int rk, int ppl)
     return fused_fn_rk<3>(rk, ppl);
 }
 
-// the multi-step kernel with W = 4 or 8 PEs per CTA
+// the multi-step kernel with W = 2, 4 or 8 PEs per CTA
 template <int H, int RK, int W>
 void* fused_steps_fn_ppl(int ppl)
 {
@@ -428,7 +441,9 @@ void* fused_steps_fn_h(int H, int rk, int ppl)
 
 void* fused_steps_fn(int H, int rk, int ppl, int W)
 {
-    return W == 4 ? fused_steps_fn_h<4>(H, rk, ppl) : fused_steps_fn_h<8>(H, rk, ppl);
+    return W == 2   ? fused_steps_fn_h<2>(H, rk, ppl)
+           : W == 4 ? fused_steps_fn_h<4>(H, rk, ppl)
+                    : fused_steps_fn_h<8>(H, rk, ppl);
 }
 
 size_t fused_smem(int B, int H, int S, int W = kFusedW)
@@ -448,8 +463,10 @@ bool atk_fused_supported(int pde, int order, int B, int S)
     return pde == atk::ADVDIFF && (B == 32 || B == 64 || B == 128 || B == 256) && B >= S * (order / 2);
 }
 
-// CTAs (of W = 4 or 8 PEs) that one cooperative launch of the multi-step
+// CTAs (of W = 2, 4 or 8 PEs) that one cooperative launch of the multi-step
 // kernel holds at once (0: not available)
+int fused_steps_block(int B, int W) { return 32 * (W * atk::steps_wpp(W, B / 32) + 1); }
+
 int64_t atk_fused_capacity(int order, int rk, int B, int S, int W, int device)
 {
     const int H = order / 2;
@@ -460,7 +477,7 @@ int64_t atk_fused_capacity(int order, int rk, int B, int S, int W, int device)
         return 0;
     }
     int per_sm = 0, sms = 0, coop = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, 32 * (W + 1), smem) != cudaSuccess ||
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, fused_steps_block(B, W), smem) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
         cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, device) != cudaSuccess || !coop) {
         cudaGetLastError();
@@ -472,12 +489,16 @@ int64_t atk_fused_capacity(int order, int rk, int B, int S, int W, int device)
 int64_t atk_fused_ctas(int64_t P, int W) { return (P + W - 1) / W; }
 
 // PEs per CTA of the multi-step kernel for P PEs, or 0 when its CTAs do not
-// fit one cooperative launch: 4 where they fit (more SMs share the stages of
-// a small problem), else 8 (measured on GB300, PEs of 64 points, us per
-// step: 2^14 points 7.3 with 4 against 8.9 with 8; 2^18 points 20.6 with 8,
-// where 4 no longer fits and takes one launch per step: 22.5)
+// fit one cooperative launch: 2, on two warps each, where that is one CTA an SM
+// at most; 4 where they fit (more SMs share the stages of a small problem), else
+// 8 (measured on GB300, PEs of 64 points, us per step: 2^14 points 5.9 with 2, 7.4
+// with 4, 8.9 with 8; 2^18 points 20.6 with 8, where 4 no longer fits and takes
+// one launch per step: 22.5)
 int atk_fused_multi_w(int order, int rk, int B, int S, int64_t P, int device)
 {
+    int sms = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) return 0;
+    if (atk_fused_ctas(P, 2) <= sms && atk_fused_ctas(P, 2) <= atk_fused_capacity(order, rk, B, S, 2, device)) return 2;
     for (int W = 4; W <= 8; W += 4)
         if (atk_fused_ctas(P, W) <= atk_fused_capacity(order, rk, B, S, W, device)) return W;
     return 0;
@@ -500,7 +521,7 @@ cudaError_t atk_launch_fused_steps(const atk::StageArgs& a, int order, int W, in
     if (e != cudaSuccess) return e;
     atk::StageArgs args = a;
     void* params[] = {(void*)&args, (void*)&b0, (void*)&b1, (void*)&level0, (void*)&nsteps};
-    return cudaLaunchCooperativeKernel(fn, dim3((unsigned)C), dim3(32 * (W + 1)), params, smem, st);
+    return cudaLaunchCooperativeKernel(fn, dim3((unsigned)C), dim3(fused_steps_block(a.B, W)), params, smem, st);
 }
 
 // one step n: u^n from uin, u^{n+1} to uout (distinct buffers)
