@@ -160,37 +160,34 @@ __device__ __forceinline__ int keff(const StageArgs& a, int64_t pe, int side)
 }
 
 // exp(x) by Tang's table-driven method (P. T. P. Tang, ACM TOMS 15(2), 1989)
-// with 512 table entries: x = (512 M + j) ln2/512 + r, |r| <= ln2/1024, and
-// exp(x) = 2^M 2^(j/512) (1 + expm1(r)), expm1(r) by its Taylor polynomial of
-// degree 4 (the first omitted term, r^5/120, is below 2e-18).  The product
+// with 256 table entries: x = (256 M + j) ln2/256 + r, |r| <= ln2/512, and
+// exp(x) = 2^M 2^(j/256) (1 + expm1(r)), expm1(r) by its Taylor polynomial of
+// degree 4 (the first omitted term, r^5/120, is below 4e-17).  The product
 // with 2^M is an integer add to the exponent field, exact while the result is
 // normal, which the fast path |x| < 512 guarantees (tested on the high word
 // with integer instructions); every other x (and Inf, NaN) goes to exp().
-// What only needs FP32's 24 bits is done there (1 cycle against 64): the
-// nearest multiple (a slip by one at a tie leaves |r| a hair larger) and the
-// polynomial's terms above r^2/2, at most 6e-11 of the result, so that their
-// 3e-7 relative error is 2e-17.  Five FP64 instructions; within 2 ulp of the
-// correctly rounded value.
+// What needs no more than FP32's 24 bits is done there (1 cycle against 64): the
+// nearest multiple (a slip by one next to a tie leaves |r| a hair larger) and
+// the factor 1/6 + r/24 of r^3, whose 2^-23 relative error is 5e-17 of the
+// result.  Six FP64 instructions; within 2 ulp of the correctly rounded value.
 __device__ __forceinline__ double at_exp(double x)
 {
-    static_assert(AT_EXP_N == 512, "the table has 512 entries");
+    static_assert(AT_EXP_N == 256, "the table has 256 entries");
     const uint32_t hi = fx_hi(x), ah = hi & 0x7fffffffu;
     if (ah >= 0x40800000u) return exp(x);
-    const float xf = fx_float(x);
-    const float t = fmaf(xf, (float)AT_EXP_INV_L, 12582912.0f);  // 1.5 2^23: the integer lands in the low bits
-    const int n = __float_as_int(t) - 0x4b400000;                // 512 M + j
+    const float t = fmaf(fx_float(x), (float)AT_EXP_INV_L, 12582912.0f);  // 1.5 2^23: the integer lands in the low bits
+    const int n = __float_as_int(t) - 0x4b400000;                         // 256 M + j
     const uint32_t nb = __float_as_uint(t - 12582912.0f);
-    // -n as a double (at most 19 bits: its low word is zero)
+    // -n as a double (at most 18 bits: its low word is zero)
     const double nd = fx_double(n == 0 ? 0u : (((nb & 0x7fffffffu) >> 3) + 0x38000000u) | (~nb & 0x80000000u), 0u);
     double r = fma(nd, AT_EXP_L_HI, x);
     r = fma(nd, AT_EXP_L_LO, r);
-    const float rf = fx_float(r);
-    const uint32_t qb = __float_as_uint(rf * rf * fmaf(rf, 1.0f / 24.0f, 1.0f / 6.0f));  // r^2/6 + r^3/24
-    const double w = fma(0.5, r, fx_double((qb >> 3) + 0x38000000u, qb << 29));
-    const double em1 = fma(r, w, r);                // expm1(r)
-    const double tj = __ldg(&at_exp_tab[n & 511]);  // 2^(j/512)
+    const uint32_t cb = __float_as_uint(fmaf(fx_float(r), 1.0f / 24.0f, 1.0f / 6.0f));
+    const double c = fma(fx_double((cb >> 3) + 0x38000000u, cb << 29), r, 0.5);
+    const double em1 = fma(c, r * r, r);            // expm1(r)
+    const double tj = __ldg(&at_exp_tab[n & 255]);  // 2^(j/256)
     const double e = fma(tj, em1, tj);
-    return fx_double(fx_hi(e) + ((uint32_t)(n >> 9) << 20), fx_lo(e));
+    return fx_double(fx_hi(e) + ((uint32_t)(n >> 8) << 20), fx_lo(e));
 }
 
 // 1/x by two Newton-Raphson steps r <- r + r (1 - x r) from the hardware's

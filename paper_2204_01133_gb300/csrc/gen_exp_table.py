@@ -1,11 +1,11 @@
 """Write exp_table.h: the constants of the table-driven exponential in
-at_device.cuh (Tang's method, ACM TOMS 15(2), 1989, with 512 table entries).
+at_device.cuh (Tang's method, ACM TOMS 15(2), 1989, with 256 table entries).
 
 Every value is computed here from its mathematical definition in 60-digit
 decimal arithmetic and rounded once to the nearest double:
-  AT_EXP_INV_L = 512 / ln 2
-  AT_EXP_L_HI  = ln 2 / 512 rounded,  AT_EXP_L_LO = (ln 2 / 512 - AT_EXP_L_HI) rounded
-  at_exp_tab[j] = 2^(j/512), j = 0..511
+  AT_EXP_INV_L = 256 / ln 2
+  AT_EXP_L_HI  = ln 2 / 256 rounded,  AT_EXP_L_LO = (ln 2 / 256 - AT_EXP_L_HI) rounded
+  at_exp_tab[j] = 2^(j/256), j = 0..255
 Usage: python gen_exp_table.py > exp_table.h
 """
 from decimal import Decimal, getcontext
@@ -13,7 +13,7 @@ from decimal import Decimal, getcontext
 getcontext().prec = 60
 
 
-M = 512  # table entries
+M = 256  # table entries
 
 
 def main():
