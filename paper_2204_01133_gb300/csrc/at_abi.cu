@@ -230,7 +230,8 @@ int stage_window(const at_problem* pb, const Layout& L, int sms)
     if (!is_weno(pb->pde) || sms < 1) return L.Tw;
     int best = L.Tw;
     int64_t least = INT64_MAX;
-    for (int t = L.Tw; t >= 16 && t >= 2 * L.H; --t) {
+    // (longer windows than 128 gain nothing: atk_stage_block)
+    for (int t = std::min(L.Tw, 128); t >= 16 && t >= 2 * L.H; --t) {
         if (pb->pe_size % t) continue;
         const int64_t windows = pb->n / t, cost = (windows + sms - 1) / sms * (t + 8);
         if (cost < least) {

@@ -858,15 +858,15 @@ size_t atk_stage_smem_bytes(int pde, int Tw, int H)
 int atk_stage_block(int pde, int Tw)
 {
     int nv = (pde == atk::RNS || pde == atk::EULER) ? 4 : 1;
-    // WENO: a thread per (edge, variable)
+    // WENO: a thread per (edge, variable); where that is more than 256, 128 (more
+    // CTAs an SM, whose phases overlap: 2^23 points, windows of 128: 7.06 ms per
+    // step with 128 threads, 7.77 with 256; windows of 256 with 256: 7.17)
     int want = (pde == atk::EULER || pde == atk::ADV_WENO || pde == atk::BURGERS) ? nv * (Tw + 1) : nv * Tw;
-    // reacting N-S: half a thread per (point, variable) item, so that a CTA of
-    // 256 threads takes two whole-PE windows (below).  A window's fill has
-    // fewer items than its update (own points plus ring levels, against 4 per
-    // point), and two windows' fills keep more of the CTA busy before the
-    // barrier (measured on GB300 at N = 2^24, PEs of 64: 15.1 ms per step with
-    // one window per CTA, 13.7 with two or four)
-    if (pde == atk::RNS) want = nv * Tw / 2;
+    if (pde == atk::EULER && want > 256) want = 128;
+    // reacting N-S: a thread per point, two windows a CTA of 128 threads (below);
+    // its barriers then hold few warps (2^22 points, PEs of 64, ms per step: 1.90,
+    // with 128 threads a window 2.00, with 256 threads 2.43, with 32 1.97)
+    if (pde == atk::RNS) want = Tw;
     if (want > 256) want = 256;
     want = ((want + 31) / 32) * 32;
     return want < 32 ? 32 : want;
@@ -913,7 +913,7 @@ cudaError_t atk_launch_stage(const atk::StageArgs& a, int pde, int order, int sm
     int m = 1;
     if ((pde == atk::ADVDIFF || pde == atk::RNS || pde == atk::RNS_CHAIN) && a.wpp == 1) {
         for (int c = 4; c >= 2; c /= 2)
-            if (c * b1 <= 256 && windows % c == 0 && windows / c >= 4 * (int64_t)sms) {
+            if (c * b1 <= (pde == atk::RNS ? 128 : 256) && windows % c == 0 && windows / c >= 4 * (int64_t)sms) {
                 m = c;
                 break;
             }
