@@ -47,7 +47,7 @@ cudaError_t atk_launch_batch(int variant, const atk::StageArgs* tab, int64_t* lv
                              int n_order, int* queue, int64_t chunk, int grid, int block, size_t smem, cudaStream_t st);
 int atk_batch_max_ctas_per_sm(int variant, int block, size_t smem);
 cudaError_t atk_launch_batch_stage(int variant, const atk::StageArgs* tab, const int64_t* lvl, const int64_t* left,
-                                   const int* win_slot, const int* win_idx, int nwin, int stage, int block,
+                                   const int* win_slot, const int* win_idx, int nwin, int rk, int stage, int block,
                                    size_t smem, int win_smem, cudaStream_t st);
 cudaError_t atk_launch_batch_advance(int64_t* lvl, int64_t* left, const int* slots, int n, cudaStream_t st);
 cudaError_t atk_launch_batch_status(const atk::StageArgs* tab, const int* slots, int n, int* out, cudaStream_t st);
@@ -1283,6 +1283,7 @@ struct at_batch {
     int64_t bound_windows = 0;
     int64_t wbegin[kVariants + 1] = {0};
     int group_stages[kVariants] = {0};
+    int group_rk[kVariants] = {0};  // the RK scheme of the group's slots, -1 where they differ
     bool dirty = true;
     // graph of the last (chunk, order) configuration
     cudaGraphExec_t gexec = nullptr;
@@ -1324,7 +1325,7 @@ cudaError_t batch_upload_order(at_batch* b)
     for (int g = 0; g < kVariants; ++g) {
         b->wbegin[g] = (int64_t)b->wslot_h.size();
         const bool pairs = !variant_is_weno(g);
-        int smax = 0;
+        int smax = 0, rk = -2;
         for (int q = b->group_begin[g]; q < b->group_begin[g + 1]; ++q) {
             const int i = b->order_h[q];
             for (int64_t w = 0; w < b->windows[i];) {
@@ -1334,8 +1335,10 @@ cudaError_t batch_upload_order(at_batch* b)
                 w += two ? 2 : 1;
             }
             smax = std::max(smax, b->args[i].S);
+            rk = rk == -2 || rk == b->args[i].rk ? b->args[i].rk : -1;
         }
         b->group_stages[g] = smax;
+        b->group_rk[g] = rk < 0 ? -1 : rk;
     }
     b->wbegin[kVariants] = (int64_t)b->wslot_h.size();
     cudaError_t e = cudaSuccess;
@@ -1391,7 +1394,7 @@ cudaError_t batch_enqueue(at_batch* b, cudaStream_t st, int64_t chunk)
             const int* wi = (const int*)(b->tab + b->T.off_widx) + b->wbegin[g];
             for (int64_t step = 0; step < chunk && e == cudaSuccess; ++step) {
                 for (int stage = 0; stage < b->group_stages[g] && e == cudaSuccess; ++stage)
-                    e = atk_launch_batch_stage(g, tab, lvl, left, ws, wi, nwin, stage, b->block,
+                    e = atk_launch_batch_stage(g, tab, lvl, left, ws, wi, nwin, b->group_rk[g], stage, b->block,
                                                variant_is_weno(g) ? smem : 2 * smem, (int)(smem / sizeof(double)),
                                                b->branch[g]);
                 if (e == cudaSuccess) e = atk_launch_batch_advance(lvl, left, order, n, b->branch[g]);

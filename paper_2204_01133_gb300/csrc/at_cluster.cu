@@ -32,7 +32,8 @@ namespace cg = cooperative_groups;
 
 namespace atk {
 
-template <int H, int PPL, int WPP>
+// CLASSIC: four-stage RK4, known when compiled; else the scheme is read at run time
+template <int H, int PPL, int WPP, bool CLASSIC>
 __global__ void __launch_bounds__(256) cluster_advdiff(const StageArgs a, int64_t level0, int64_t nsteps)
 {
     constexpr int B = 32 * PPL;       // PE size
@@ -46,7 +47,7 @@ __global__ void __launch_bounds__(256) cluster_advdiff(const StageArgs a, int64_
     const int hw = wib - lp * WPP;                 // which share of the PE's points
     const int j0 = hw * SW;                        // first point of the share
     const int64_t pe = (int64_t)blockIdx.x * m + lp;
-    const int S = a.S, R = a.R;
+    const int S = CLASSIC ? 4 : a.S, R = a.R;
     extern __shared__ double sm[];
     double* U = sm;                                 // u^n                          [m][B]
     double* X = U + m * B;                          // stage argument, two parities [2][m][B]
@@ -158,7 +159,8 @@ __global__ void __launch_bounds__(256) cluster_advdiff(const StageArgs a, int64_
                 // the update of the per-stage kernels (rk_update), into shared memory
                 const double dt = a.dt, un = U[it], x = Wr[H + jw];
                 double y;
-                if (a.rk == RK4) {
+                const int rk = CLASSIC ? (int)RK4 : a.rk;
+                if (rk == RK4) {
                     if (s == 0) {
                         ACC[it] = K;
                         y = fma(a.hdt, K, un);
@@ -168,7 +170,7 @@ __global__ void __launch_bounds__(256) cluster_advdiff(const StageArgs a, int64_
                     } else {
                         y = fma(a.dt6, ACC[it] + K, un);
                     }
-                } else if (a.rk == RK3TVD) {
+                } else if (rk == RK3TVD) {
                     if (s == 0) y = fma(dt, K, x);
                     else if (s == 1) y = fma(0.75, un, 0.25 * fma(dt, K, x));
                     else y = fma(1.0 / 3.0, un, (2.0 / 3.0) * fma(dt, K, x));
@@ -224,33 +226,39 @@ int cluster_wpp(int B, int m)
     return w >= 8 ? 8 : w >= 4 ? 4 : w >= 2 ? 2 : 1;
 }
 
-void* cluster_fn(int H, int ppl, int wpp)
+template <bool C>
+void* cluster_fn_rk(int H, int ppl, int wpp)
 {
 #define AT_CL(HH)                                                                  \
     if (wpp == 1) {                                                                \
         switch (ppl) {                                                             \
-        case 1: return (void*)atk::cluster_advdiff<HH, 1, 1>;                      \
-        case 2: return (void*)atk::cluster_advdiff<HH, 2, 1>;                      \
-        case 4: return (void*)atk::cluster_advdiff<HH, 4, 1>;                      \
-        default: return (void*)atk::cluster_advdiff<HH, 8, 1>;                     \
+        case 1: return (void*)atk::cluster_advdiff<HH, 1, 1, C>;                      \
+        case 2: return (void*)atk::cluster_advdiff<HH, 2, 1, C>;                      \
+        case 4: return (void*)atk::cluster_advdiff<HH, 4, 1, C>;                      \
+        default: return (void*)atk::cluster_advdiff<HH, 8, 1, C>;                     \
         }                                                                          \
     }                                                                              \
     if (wpp == 2) {                                                                \
         switch (ppl) {                                                             \
-        case 2: return (void*)atk::cluster_advdiff<HH, 2, 2>;                      \
-        case 4: return (void*)atk::cluster_advdiff<HH, 4, 2>;                      \
-        default: return (void*)atk::cluster_advdiff<HH, 8, 2>;                     \
+        case 2: return (void*)atk::cluster_advdiff<HH, 2, 2, C>;                      \
+        case 4: return (void*)atk::cluster_advdiff<HH, 4, 2, C>;                      \
+        default: return (void*)atk::cluster_advdiff<HH, 8, 2, C>;                     \
         }                                                                          \
     }                                                                              \
     if (wpp == 4) {                                                                \
-        if (ppl == 4) return (void*)atk::cluster_advdiff<HH, 4, 4>;                \
-        return (void*)atk::cluster_advdiff<HH, 8, 4>;                              \
+        if (ppl == 4) return (void*)atk::cluster_advdiff<HH, 4, 4, C>;                \
+        return (void*)atk::cluster_advdiff<HH, 8, 4, C>;                              \
     }                                                                              \
-    return (void*)atk::cluster_advdiff<HH, 8, 8>;
+    return (void*)atk::cluster_advdiff<HH, 8, 8, C>;
     if (H == 1) { AT_CL(1) }
     if (H == 2) { AT_CL(2) }
     AT_CL(3)
 #undef AT_CL
+}
+
+void* cluster_fn(int H, int ppl, int wpp, int S)
+{
+    return S == 4 ? cluster_fn_rk<true>(H, ppl, wpp) : cluster_fn_rk<false>(H, ppl, wpp);
 }
 
 size_t cluster_smem(int B, int H, int m, int R, int S)
@@ -296,7 +304,7 @@ int atk_cluster_size(int pde, int order, int B, int64_t P, int R, int S, int dev
         }
     if (C == 0 || P / C > kClusterMaxPePerCta) return 0;
     const int m = (int)(P / C);
-    void* fn = cluster_fn(H, B / 32, cluster_wpp(B, m));
+    void* fn = cluster_fn(H, B / 32, cluster_wpp(B, m), S);
     const size_t smem = cluster_smem(B, H, m, R, S);
     if (cudaSetDevice(device) != cudaSuccess) return 0;
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
@@ -318,7 +326,7 @@ cudaError_t atk_launch_cluster(const atk::StageArgs& a, int order, int csize, in
                                cudaStream_t st)
 {
     const int H = order / 2, m = (int)(a.P / csize);
-    void* fn = cluster_fn(H, a.B / 32, cluster_wpp(a.B, m));
+    void* fn = cluster_fn(H, a.B / 32, cluster_wpp(a.B, m), a.S);
     const size_t smem = cluster_smem(a.B, H, m, a.R, a.S);
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

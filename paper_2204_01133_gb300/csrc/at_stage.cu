@@ -639,7 +639,8 @@ __global__ void __launch_bounds__(256) batch_run(const StageArgs* __restrict__ t
 // shared memory apiece: two windows' fill items then share the barrier phases
 // of one CTA, as on the per-stage path.
 constexpr int AT_BATCH_WIN_MASK = 0x3fffffff;
-template <int PDE, int H, bool WENO>
+// RKS: the stage's kind where every slot of the launch has the same RK scheme.
+template <int PDE, int H, bool WENO, int RKS = RKS_ANY>
 __global__ void __launch_bounds__(256, PDE == RNS ? 5 : 4) batch_stage(const StageArgs* __restrict__ tab, const int64_t* __restrict__ lvl,
                                                    const int64_t* __restrict__ left, const int* __restrict__ win_slot,
                                                    const int* __restrict__ win_idx, int stage, int win_smem)
@@ -655,14 +656,14 @@ __global__ void __launch_bounds__(256, PDE == RNS ? 5 : 4) batch_stage(const Sta
     const int e = win_idx[blockIdx.x];
     const int w0 = e & AT_BATCH_WIN_MASK;
     if constexpr (WENO) {
-        weno_window<PDE>(a, cx, w0, sm);
+        weno_window<PDE, RKS>(a, cx, w0, sm);
     } else {
         if (e >> 30) {
             const int half = blockDim.x >> 1;
             const int g = threadIdx.x >= half ? 1 : 0;
-            central_window<PDE, H>(a, cx, w0 + g, sm + (size_t)g * win_smem, threadIdx.x - g * half, half);
+            central_window<PDE, H, RKS>(a, cx, w0 + g, sm + (size_t)g * win_smem, threadIdx.x - g * half, half);
         } else {
-            central_window<PDE, H>(a, cx, w0, sm, threadIdx.x, blockDim.x);
+            central_window<PDE, H, RKS>(a, cx, w0, sm, threadIdx.x, blockDim.x);
         }
     }
 }
@@ -1068,8 +1069,17 @@ cudaError_t atk_launch_batch(int variant, const atk::StageArgs* tab, int64_t* lv
     return cudaLaunchKernel(fn, dim3(grid), dim3(block), params, smem, st);
 }
 
-static void* batch_stage_fn(int variant)
+// rk: the RK scheme of every slot of the launch, or -1 where they differ; the
+// configured combinations get one kernel per stage kind, as on the per-stage path
+static void* batch_stage_fn(int variant, int rk, int stage)
 {
+    const int kind = rk < 0 ? atk::RKS_ANY : atk::rk_stage_kind(rk, stage);
+    if (variant == 5 && kind == atk::RKS_RK4_0) return (void*)atk::batch_stage<atk::RNS, 3, false, atk::RKS_RK4_0>;
+    if (variant == 5 && kind == atk::RKS_RK4_MID) return (void*)atk::batch_stage<atk::RNS, 3, false, atk::RKS_RK4_MID>;
+    if (variant == 5 && kind == atk::RKS_RK4_LAST) return (void*)atk::batch_stage<atk::RNS, 3, false, atk::RKS_RK4_LAST>;
+    if (variant == 6 && kind == atk::RKS_RK3_0) return (void*)atk::batch_stage<atk::EULER, 3, true, atk::RKS_RK3_0>;
+    if (variant == 6 && kind == atk::RKS_RK3_1) return (void*)atk::batch_stage<atk::EULER, 3, true, atk::RKS_RK3_1>;
+    if (variant == 6 && kind == atk::RKS_RK3_2) return (void*)atk::batch_stage<atk::EULER, 3, true, atk::RKS_RK3_2>;
     switch (variant) {
     case 0: return (void*)atk::batch_stage<atk::ADVDIFF, 1, false>;
     case 1: return (void*)atk::batch_stage<atk::ADVDIFF, 2, false>;
@@ -1087,10 +1097,10 @@ static void* batch_stage_fn(int variant)
 }
 
 cudaError_t atk_launch_batch_stage(int variant, const atk::StageArgs* tab, const int64_t* lvl, const int64_t* left,
-                                   const int* win_slot, const int* win_idx, int nwin, int stage, int block,
+                                   const int* win_slot, const int* win_idx, int nwin, int rk, int stage, int block,
                                    size_t smem, int win_smem, cudaStream_t st)
 {
-    void* fn = batch_stage_fn(variant);
+    void* fn = batch_stage_fn(variant, rk, stage);
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     void* params[] = {(void*)&tab, (void*)&lvl, (void*)&left, (void*)&win_slot, (void*)&win_idx, (void*)&stage,
