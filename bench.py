@@ -60,30 +60,29 @@ DEFAULT = "detonation-n16777216"
 NOMINAL_FP64_TFLOPS = 1.25  # GB300 FP64 (vector and tensor), nominal, at 2070 MHz boost
 
 # FP64 flops per point per stage (FMA = 2, add/mul = 1) that the timed kernel
-# executes: ncu's DFMA/DADD/DMUL thread-instruction counts of one launch on
-# the large-N workloads (the persistent kernel on N = 16,384) divided by the
-# point-stages of the launch.  They include the AT halo work and the
-# instruction sequences of exp and the reciprocals, so achieved / peak is the
-# share of the FP64 roof the kernel's own arithmetic uses.
+# executes: ncu's DFMA/DADD/DMUL thread-instruction counts, mean over the RK
+# stages, on the large-N workloads (the persistent kernel on N = 16,384).  They
+# include the AT halo work.  The stencils of the reacting flow and the WENO
+# fluxes are integer arithmetic (csrc/at_fixed.cuh) and not in these counts, so
+# achieved / peak is the share of the FP64 roof that the FP64 part alone uses.
 FLOPS_PER_POINT_STAGE = {
-    ("rns", "stage"): 165.7,         # central6 + AT6, 4 variables (RK4 stage 1 counted)
-    ("rns", "persistent"): 165.8,    # same work, all K steps of one launch
-    ("detonation", "stage"): 500.3,  # WENO5 + AT-WENO5, 8 reconstructions per edge (RK3 stage 0)
+    ("rns", "stage"): 64.0,          # central6 + AT6, 4 variables (all in FP64: 165.7)
+    ("rns", "persistent"): 69.2,     # same work, all K steps of one launch
+    ("detonation", "stage"): 111.6,  # WENO5 + AT-WENO5, 8 reconstructions per edge (all in FP64: 500.3)
     ("advdiff", "stage"): 13.56,     # 5-tap merged stencil + RK4 update, mean of the 4 stages
     ("advdiff", "persistent"): 13.56,
-    ("advdiff", "fused"): 13.56,     # the method's work only (13.65 as executed, with the recomputed edge points)
-    ("rns", "fused"): 165.7,         # the method's work only (the tile-fused kernel also recomputes the strips)
-    ("detonation", "fused"): 500.3,  # likewise: the per-stage kernel's count
+    ("advdiff", "fused"): 13.56,     # the method's work only
+    ("rns", "fused"): 64.0,          # the per-stage kernel's count (the tile-fused kernel executes 67.3 with the strips)
+    ("detonation", "fused"): 111.6,  # likewise (144.7 with the strips)
 }
 # The method's own FP64 work per point per stage, by operation count (a
 # divide, square root or exponential counts as one operation): the
 # detonation's WENO5 + AT-WENO5 stage ~550 flops + 8 divides + 1 sqrt + 1 exp
 # (two reconstructions per variable and edge, the splitting, the Arrhenius
 # source, the update); the reacting flow's central6 stage ~150 flops + 4
-# divides + 1 exp; advection-diffusion 52 flops per RK4 step.  The executed
-# counts above also hold the instruction sequences of exp and the
-# reciprocals and the AT halo work; achieved / peak on this count is
-# roofline.frac_algorithmic.
+# divides + 1 exp; advection-diffusion 52 flops per RK4 step.  Achieved / peak
+# on this count is roofline.frac_algorithmic: above 1 where most of the work
+# does not run on the FP64 unit.
 ALG_FLOPS_PER_POINT_STAGE = {"detonation": 560.0, "rns": 155.0, "advdiff": 13.0}
 # Algorithmic HBM bytes per point per stage of the per-stage path: the arrays
 # a step reads and writes (RK4: 17 arrays, RK3-TVD: 8) x nvar x 8 B / stages.
@@ -91,9 +90,26 @@ BYTES_PER_POINT_STAGE = {"rns": 17 * 4 * 8 / 4, "detonation": 8 * 4 * 8 / 3, "ad
 # the step-fused path reads u^n and writes u^{n+1} once per step (+ the ring)
 BYTES_PER_POINT_STAGE_FUSED = {"advdiff": 2 * 8 / 4, "rns": 2 * 4 * 8 / 4, "detonation": 2 * 4 * 8 / 3}
 # DRAM bytes per launch of the timed kernel (dram__bytes_read.sum +
-# dram__bytes_write.sum) from ncu captures, by workload and path; a workload
-# without a capture of the current kernels has no entry.
-TRAFFIC_PER_LAUNCH = {}
+# dram__bytes_write.sum, mean over the RK stages) from the ncu captures of the
+# current kernels, by workload and path; the reacting flow and the detonation
+# were captured at N = 2^22, advection-diffusion at 2^25, and are scaled.
+TRAFFIC_PER_LAUNCH = {
+    ("rns-flame-n16384", "persistent"): 2.9916e+06,  # state and rings read once, writes stay in L2
+    ("rns-flame-n16777216", "stage"): 4 * 5.5312e+08,
+    ("rns-flame-n8388608", "stage"): 2 * 5.5312e+08,
+    ("detonation-n8388608", "stage"): 2 * 3.2141e+08,
+    ("detonation-n16777216", "stage"): 4 * 3.2141e+08,
+    ("advdiff-n134217728", "stage"): 4 * 1.1303e+09,
+    ("advdiff-n33554432", "stage"): 1.1303e+09,
+    ("advdiff-n134217728", "fused"): 4 * 5.5701e+08,  # one step: u^n, u^{n+1}, the ring
+    ("advdiff-n33554432", "fused"): 5.5701e+08,
+    ("advdiff-n2048", "persistent"): 7.5776e+04,  # one-cluster launch: state and ring read once
+    ("advdiff-n16384", "fused"): 2.4346e+05,  # cooperative fused launch: state and ring read once
+    ("rns-flame-n16777216", "fused"): 4 * 2.6627e+08,  # tile-fused step
+    ("rns-flame-n8388608", "fused"): 2 * 2.6627e+08,
+    ("detonation-n16777216", "fused"): 4 * 2.2820e+08,  # tile-fused step
+    ("detonation-n8388608", "fused"): 2 * 2.2820e+08,
+}
 
 
 # The kernel sources the captured counts above were taken from, per
@@ -106,7 +122,26 @@ KERNEL_FILES = {
     "persistent": ("at_cluster.cu", "at_device.cuh", "at_fixed.cuh", "at_persist.cu"),
     "fused": ("at_device.cuh", "at_fixed.cuh", "at_fused.cu", "at_tilefused.cu"),
 }
-PROFILED_SHA256 = {}
+_SHA_STAGE = "6e1003d69625f66ac04f5e517819a09bce1456e986aae19e8d6f5e8cc5a87e73"
+_SHA_PERSISTENT = "6dcb1913787d047c444bf2d51ef605ebc647a8f342f631cf4b456354bc2b5ec3"
+_SHA_FUSED = "07c561258ddafdf3ad19df60682fcf50bf59817393faa38b0375d6780655bf39"
+PROFILED_SHA256 = {
+    ("detonation-n16777216", "stage"): _SHA_STAGE,
+    ("detonation-n8388608", "stage"): _SHA_STAGE,
+    ("rns-flame-n16777216", "stage"): _SHA_STAGE,
+    ("rns-flame-n8388608", "stage"): _SHA_STAGE,
+    ("advdiff-n134217728", "stage"): _SHA_STAGE,
+    ("advdiff-n33554432", "stage"): _SHA_STAGE,
+    ("rns-flame-n16384", "persistent"): _SHA_PERSISTENT,
+    ("advdiff-n2048", "persistent"): _SHA_PERSISTENT,
+    ("advdiff-n134217728", "fused"): _SHA_FUSED,
+    ("advdiff-n33554432", "fused"): _SHA_FUSED,
+    ("advdiff-n16384", "fused"): _SHA_FUSED,
+    ("rns-flame-n16777216", "fused"): _SHA_FUSED,
+    ("rns-flame-n8388608", "fused"): _SHA_FUSED,
+    ("detonation-n16777216", "fused"): _SHA_FUSED,
+    ("detonation-n8388608", "fused"): _SHA_FUSED,
+}
 
 
 def sources_sha256(path: str) -> str:

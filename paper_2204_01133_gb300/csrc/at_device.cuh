@@ -196,9 +196,8 @@ __device__ __forceinline__ double at_exp(double x)
 // normal, finite, nonzero x the kernels divide by (densities, pressures,
 // temperatures, WENO weight sums).  Zero, Inf or subnormal x give Inf or
 // NaN, which the non-finite check reports.  Five FP64-pipe instructions, about
-// half of an IEEE division.  The kernels use at_rcp3 below (one instruction
-// fewer); this form is exported by the probe library beside it for the
-// reciprocal tests.
+// half of an IEEE division (at_rcp3 below: one fewer).  Exported by the probe
+// library beside the others for the reciprocal tests.
 __device__ __forceinline__ double at_rcp(double x)
 {
     double r;
@@ -215,8 +214,8 @@ __device__ __forceinline__ double at_rcp(double x)
 // "The Numerical Treatment of a Single Nonlinear Equation", 1970), one FP64
 // instruction fewer than at_rcp's two quadratic steps, within about an ulp
 // of 1/x for normal, finite, nonzero x (both are tested against 1/x).  The
-// kernels' reciprocals (densities, temperatures, pressures, WENO weight
-// sums) outside the normal range go through this one (at_rcpi below).
+// kernels' reciprocals are integer ones (at_rcpi) and come here only outside the
+// normal range.
 __device__ __forceinline__ double at_rcp3(double x)
 {
     double r;

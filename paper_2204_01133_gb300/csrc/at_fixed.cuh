@@ -450,7 +450,7 @@ AT_HD uint64_t fx_fixed(FxU a, int e)
 }
 
 // The sum of the corrections of the two WENO5 reconstructions of an edge, six
-// times (sum of num/den) - (s_1+ + s_1-) of weno5d and weno_flux, at_device.cuh,
+// times (sum of corrections) - (s_1+ + s_1-) of weno_flux, at_device.cuh,
 // from the first differences c of C and q of hl Q at the columns c-2..c+2.
 // With the ten differences aligned to their largest exponent (58 bits), the
 // split differences q + c and q - c, the second and third differences and
@@ -481,7 +481,7 @@ AT_HD double fx_weno_sum(const double* c, const double* q, FxU eps3)
     int64_t sum = 0;
 #pragma unroll
     for (int s = 0; s < 2; ++s) {
-        // f+ from the left, f- mirrored: a_1..a_4 of weno5d, below 2^59
+        // f+ from the left, f- mirrored: a_1..a_4, below 2^59
         const int64_t a1 = s ? Q[4] - C[4] : Q[0] + C[0], a2 = s ? Q[3] - C[3] : Q[1] + C[1];
         const int64_t a3 = s ? Q[2] - C[2] : Q[2] + C[2], a4 = s ? Q[1] - C[1] : Q[3] + C[3];
         const int64_t s0 = a2 - a1, s1 = a3 - a2, s2 = a4 - a3;  // below 2^60

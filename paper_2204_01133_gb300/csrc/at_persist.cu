@@ -133,20 +133,24 @@ __device__ __forceinline__ void bar_arrive_p(int p, int count)
 // GB300's FP64 unit spends the same time on a warp instruction whatever the
 // number of active lanes, so the work is laid out in whole, uniform warps
 // with fixed roles.  Stage t (= step n, stage s) of a PE:
-//   (A) derive warps: own-point derived quantities into G[t % 2] and the
-//       Arrhenius factor exp(-Ea/T) from the temperature among them;
+//   (A) derive warps: own-point derived quantities into G[t % 2] (the reacting
+//       flow's split for its integer differences); beside them, where there are
+//       enough, warps for the Arrhenius factor exp(-Ea/T);
 //   (C) all worker warps: stencil, source and RK update of every (point,
 //       variable), one variable per warp, the edge points straight into the
 //       ring; then the progress counter is published.
 // After a stage, warp 0 derives the new stage argument at the PE's 2H edge
 // points into a ring of derived quantities and publishes the stage.  The
 // halo warp runs one stage ahead of the workers: while they do stage t it
-// takes the delays of stage t + 1, waits (boundedly) for the neighbours'
-// data, reads their derived quantities of the delayed levels and writes the
-// weighted buffer values into the halo columns of G[(t + 1) % 2], so that
-// its latency hides behind the workers' arithmetic (a drawn delay of 0
+// takes the delays of stage t + 1, reads the neighbours' derived quantities of
+// the delayed levels and writes the weighted buffer values into the halo
+// columns of G[(t + 1) % 2], a side with delay 0 last, after a bounded wait, so
+// that its latency hides behind the workers' arithmetic (a drawn delay of 0
 // then costs the neighbour's edge derivation, not a derivation under the
-// contention of the receiving SM).  Named barriers, by
+// contention of the receiving SM).  What bounds it: the loop update (2,500
+// cycles) - edge derivation and release (2,800) - the neighbour's read and copy
+// (about 1,500) where delays of 0 chain; second differences on warps of their
+// own shortened the update but not the stage.  Named barriers, by
 // the parity p of the stage:
 //   1 + p  halo of stage t ready      (halo warp arrives, workers sync)
 //   3 + p  G[p] no longer read        (workers arrive after stage t, the

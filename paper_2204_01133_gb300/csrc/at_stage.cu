@@ -481,7 +481,7 @@ __global__ void __launch_bounds__(256, 4) stage_weno(const StageArgs a)
 // the right edge of f[2] from f[0..4] by the third-order interpolants
 // u0 = 3/8 f0 - 5/4 f1 + 15/8 f2, u1 = -1/8 f1 + 3/4 f2 + 3/8 f3,
 // u2 = 3/8 f2 + 3/4 f3 - 1/8 f4, ideal weights {1/16, 5/8, 5/16}, the
-// indicators of Eq. betaS and the weights of Eq. omg, arranged as weno5d():
+// indicators of Eq. betaS and the weights of Eq. omg, arranged as for weno_flux():
 // u0 - u1 = 3/8 (s_0 - s_1), u2 - u1 = 1/8 (s_1 - s_2), and with the common
 // factor E_0 E_1 E_2 and a scaling by 128,
 //   num = E_1 (3 E_2 (s_0 - s_1) + 5 E_0 (s_1 - s_2)),
@@ -901,15 +901,18 @@ cudaError_t atk_launch_stage(const atk::StageArgs& a, int pde, int order, int sm
     // the chain-rule form on few windows: a thread per fill item (own points and
     // buffer levels), so that the fill takes one pass
     const bool few = windows < 16 * (int64_t)sms;
-    if (pde == atk::RNS_CHAIN && few && a.Tw <= 192) b1 = (a.Tw + 2 * a.H * (a.q + 1) + 31) / 32 * 32 > 256 ? 256 : (a.Tw + 2 * a.H * (a.q + 1) + 31) / 32 * 32;
+    if (pde == atk::RNS_CHAIN && few && a.Tw <= 192) {
+        b1 = (a.Tw + 2 * a.H * (a.q + 1) + 31) / 32 * 32;
+        if (b1 > 256) b1 = 256;
+    }
     size_t smem1 = atk_stage_smem_bytes(pde, a.Tw, a.H);
     if (a.weno_interp) {  // G [ND][W2], SP, ARR [W2], LAM [E], REC [NV][2][E], HS with W2 = Tw + 8, E = Tw + 3
         const size_t nd = pde == atk::EULER ? 8 : 2, nv = nd / 2, W2 = a.Tw + 2 * a.H, E = a.Tw + 3;
         smem1 = sizeof(double) * (nd * W2 + 2 * W2 + E + 2 * nv * E + (size_t)2 * a.H * (AT_QMAX + 1) * nd);
     }
     // central stencils on small windows: several windows per CTA (whole PEs
-    // only, dividing the window count), so a CTA carries up to 256 threads, where
-    // that leaves four CTAs an SM (the chain-rule form at 16,384 points, 256
+    // only, dividing the window count), so a CTA carries up to 256 threads (the
+    // flame 128), where that leaves four CTAs an SM (the chain-rule form at 16,384 points, 256
     // windows: 15.2 us per stage with four windows a CTA, 12.9 with one)
     int m = 1;
     if ((pde == atk::ADVDIFF || pde == atk::RNS || pde == atk::RNS_CHAIN) && a.wpp == 1) {
