@@ -124,7 +124,7 @@ KERNEL_FILES = {
 }
 _SHA_STAGE = "6e1003d69625f66ac04f5e517819a09bce1456e986aae19e8d6f5e8cc5a87e73"
 _SHA_PERSISTENT = "6dcb1913787d047c444bf2d51ef605ebc647a8f342f631cf4b456354bc2b5ec3"
-_SHA_FUSED = "07c561258ddafdf3ad19df60682fcf50bf59817393faa38b0375d6780655bf39"
+_SHA_FUSED = "535ccbbe1ea52fd13c023dde16e7d073d3dbb73043d554add35ea67e78527a43"
 PROFILED_SHA256 = {
     ("detonation-n16777216", "stage"): _SHA_STAGE,
     ("detonation-n8388608", "stage"): _SHA_STAGE,

@@ -38,6 +38,18 @@ def test_pes_per_cta_of_the_multi_step_kernel(pe_size, pes):
     _same(_run(pb, u0, 25, "stage"), _run(pb, u0, 25, "fused"))
 
 
+@pytest.mark.parametrize("pes,order,rk", [(1, 4, "rk4"), (2, 6, "rk3tvd"), (101, 6, "rk3tvd"), (305, 4, "rk4"),
+                                          (2500, 4, "rk4"), (6001, 6, "rk4")])
+def test_pes_of_96_points(pes, order, rk):
+    """By the automatic rule (resident and one launch per step); the path asked
+    for by name still takes the sizes it took."""
+    from paper_2204_01133_gb300.api import AtError
+    pb, u0 = W.advdiff(n=96 * pes, pe_size=96, order=order, rk=rk, mode="at", k_max=3, seed=3, cfl=0.01)
+    _same(_run(pb, u0, 25, "stage"), _run(pb, u0, 25, "auto"))
+    with pytest.raises(AtError):
+        _run(pb, u0, 1, "fused")
+
+
 @pytest.mark.parametrize("pe_size,pes", [(512, 2), (480, 7), (480, 128), (96, 3), (1024, 60), (720, 300), (16, 5),
                                          (1021, 2), (22, 9)])
 def test_window_lengths_of_the_weno_kernels(pe_size, pes):
