@@ -122,7 +122,7 @@ KERNEL_FILES = {
     "persistent": ("at_cluster.cu", "at_device.cuh", "at_fixed.cuh", "at_persist.cu"),
     "fused": ("at_device.cuh", "at_fixed.cuh", "at_fused.cu", "at_tilefused.cu"),
 }
-_SHA_STAGE = "6e1003d69625f66ac04f5e517819a09bce1456e986aae19e8d6f5e8cc5a87e73"
+_SHA_STAGE = "2e82cec8708c49d8c0b717a92ef80de7f27a76226a8b015202d507f68faa638d"
 _SHA_PERSISTENT = "6dcb1913787d047c444bf2d51ef605ebc647a8f342f631cf4b456354bc2b5ec3"
 _SHA_FUSED = "535ccbbe1ea52fd13c023dde16e7d073d3dbb73043d554add35ea67e78527a43"
 PROFILED_SHA256 = {

@@ -230,10 +230,14 @@ int stage_window(const at_problem* pb, const Layout& L, int sms)
     if (!is_weno(pb->pde) || sms < 1) return L.Tw;
     int best = L.Tw;
     int64_t least = INT64_MAX;
-    // (longer windows than 128 gain nothing: atk_stage_block)
-    for (int t = std::min(L.Tw, 128); t >= 16 && t >= 2 * L.H; --t) {
+    // (longer windows than 128 gain nothing in the reconstruction form:
+    // atk_stage_block; the interpolation form, two edges and two halo points a
+    // window more, keeps 256 and pays 16 for a window)
+    const int longest = pb->weno == AT_WENO_INTERPOLATE ? 256 : 128;
+    const int extra = pb->weno == AT_WENO_INTERPOLATE ? 16 : 8;
+    for (int t = std::min(L.Tw, longest); t >= 16 && t >= 2 * L.H; --t) {
         if (pb->pe_size % t) continue;
-        const int64_t windows = pb->n / t, cost = (windows + sms - 1) / sms * (t + 8);
+        const int64_t windows = pb->n / t, cost = (windows + sms - 1) / sms * (t + extra);
         if (cost < least) {
             least = cost;
             best = t;

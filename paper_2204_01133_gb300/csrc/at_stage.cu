@@ -906,9 +906,10 @@ cudaError_t atk_launch_stage(const atk::StageArgs& a, int pde, int order, int sm
         if (b1 > 256) b1 = 256;
     }
     size_t smem1 = atk_stage_smem_bytes(pde, a.Tw, a.H);
-    if (a.weno_interp) {  // G [ND][W2], SP, ARR [W2], LAM [E], REC [NV][2][E], HS with W2 = Tw + 8, E = Tw + 3
+    if (a.weno_interp) {  // a thread per (edge, variable, sign); G [ND][W2], SP, ARR [W2], LAM [E], REC [NV][2][E], HS with W2 = Tw + 8, E = Tw + 3
         const size_t nd = pde == atk::EULER ? 8 : 2, nv = nd / 2, W2 = a.Tw + 2 * a.H, E = a.Tw + 3;
         smem1 = sizeof(double) * (nd * W2 + 2 * W2 + E + 2 * nv * E + (size_t)2 * a.H * (AT_QMAX + 1) * nd);
+        b1 = 2 * nv * E >= 256 ? 256 : (int)((2 * nv * E + 31) / 32 * 32);
     }
     // central stencils on small windows: several windows per CTA (whole PEs
     // only, dividing the window count), so a CTA carries up to 256 threads (the
