@@ -122,9 +122,9 @@ KERNEL_FILES = {
     "persistent": ("at_cluster.cu", "at_device.cuh", "at_fixed.cuh", "at_persist.cu"),
     "fused": ("at_device.cuh", "at_fixed.cuh", "at_fused.cu", "at_tilefused.cu"),
 }
-_SHA_STAGE = "2e82cec8708c49d8c0b717a92ef80de7f27a76226a8b015202d507f68faa638d"
-_SHA_PERSISTENT = "6dcb1913787d047c444bf2d51ef605ebc647a8f342f631cf4b456354bc2b5ec3"
-_SHA_FUSED = "535ccbbe1ea52fd13c023dde16e7d073d3dbb73043d554add35ea67e78527a43"
+_SHA_STAGE = "73d66cf4bb69b05e91a580d196a0d48ac7ce65d9ba4bf313e6f34e5587bfe78f"
+_SHA_PERSISTENT = "88de10f110aa4ac4ac19ec9bb1bcacc7d4eda71be70deacfa2d9b3271044aa64"
+_SHA_FUSED = "2cefcb626dc7bb58b28d69c0890ff7df8deab82dd05c1c0139b8f3b5ffec0c8f"
 PROFILED_SHA256 = {
     ("detonation-n16777216", "stage"): _SHA_STAGE,
     ("detonation-n8388608", "stage"): _SHA_STAGE,

@@ -369,7 +369,7 @@ atk::StageArgs build_args(const at_problem* pb, const at_delays* dl, const Layou
         }
     } else {
         a.k0 = 1.0 / dx;
-        a.k1 = 3.0 * pb->prm[pb->pde == AT_EULER ? 4 : 1];
+        a.eps3 = atk::fx_unpack(3.0 * pb->prm[pb->pde == AT_EULER ? 4 : 1]);
         a.weno_interp = pb->weno == AT_WENO_INTERPOLATE ? 1 : 0;
     }
     a.ext = (double*)(ws + L.off_ext);

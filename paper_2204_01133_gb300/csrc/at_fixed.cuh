@@ -273,8 +273,9 @@ AT_HD double fx_d2(const ROW& F)
 
 // ---------------------------------------------------------------------------
 // Products, sums and reciprocals of numbers with 64-bit mantissas: about 18 to
-// 25 issue cycles each against 64 for an FP64 instruction, and 57 or more
-// correct bits against 53.  m 2^e, cut towards zero.
+// 25 issue cycles each against 64 for an FP64 instruction.  m 2^e, cut towards
+// zero; a zero's exponent lies below every other, so that nothing is shifted
+// out beside it.
 // ---------------------------------------------------------------------------
 struct FxU {
     uint64_t m;
@@ -285,13 +286,7 @@ struct FxS {
     int e;
 };
 
-// a nonnegative double (a subnormal loses its scale, which is below 2^-1022)
-AT_HD FxU fx_unpack(double x)
-{
-    const uint32_t hi = fx_hi(x), t = hi & FX_EXP;
-    const uint64_t m = (uint64_t)((hi & 0xfffffu) | fx_min(t, 0x100000u)) << 32 | fx_lo(x);
-    return FxU{m << 11, (int)(t >> 20) - 1086};
-}
+constexpr int FX_TINY = -(1 << 20), FX_HUGE = 1 << 20;
 
 AT_HD FxU fx_mul(FxU a, FxU b) { return FxU{fx_mulhi(a.m, b.m), a.e + b.e + 64}; }
 
@@ -305,6 +300,16 @@ AT_HD FxU fx_normal(FxU a)
 {
     const int lz = fx_clz(a.m | 1u);
     return FxU{a.m << lz, a.e - lz};
+}
+
+// a nonnegative double; Inf and NaN have an exponent above every other, beside
+// which nothing is left
+AT_HD FxU fx_unpack(double x)
+{
+    const uint32_t hi = fx_hi(x), t = hi & FX_EXP;
+    const uint64_t m = (uint64_t)((hi & 0xfffffu) | fx_min(t, 0x100000u)) << 32 | fx_lo(x);
+    const FxU v = fx_normal(FxU{m << 11, (int)(fx_max(t, 0x100000u) >> 20) - 1086});
+    return t == FX_EXP ? FxU{0, FX_HUGE} : (m == 0 ? FxU{0, FX_TINY} : v);
 }
 
 AT_HD double fx_pack(FxS a)
@@ -432,6 +437,7 @@ AT_HD FxU fx_leading(uint64_t hi, uint64_t lo, int e)
         w0 = z ? 0u : w0;
         e -= z ? 32 : 0;
     }
+    if (w3 == 0) e = FX_TINY;
 #ifdef __CUDA_ARCH__
     const int lz = __clz((int)(w3 | 1u));
     return FxU{(uint64_t)__funnelshift_l(w2, w3, lz) << 32 | __funnelshift_l(w1, w2, lz), e - lz};
@@ -455,15 +461,18 @@ AT_HD uint64_t fx_fixed(FxU a, int e)
 // With the ten differences aligned to their largest exponent (58 bits), the
 // split differences q + c and q - c, the second and third differences and
 // 3 beta_i = s (4 s + 3 a) + 3 a^2 are exact integers; 3 (eps + beta_i) then has
-// a 64-bit mantissa of its own, and with E_i its square, A = 3 E_0 and
+// a 64-bit mantissa of its own (62 bits or more of it used, also where beta_i is
+// zero and eps alone is left), and with E_i its square, A = 3 E_0 and
 // den = E_1 (A + E_2) + 2 A E_2 the correction is
 //   (2 E_1 E_2 / den) (s_0 - s_1) + (E_1 A / den) (s_1 - s_2)
-// (the threes cancel), the two weights as fixed-point numbers.  About 1,600
-// issue cycles of integer work for an edge and variable stand beside seven FP64
-// instructions (448 cycles), in place of 66 of those (4,224).  Measured on
-// GB300: the detonation of 2^23 points 10.77 -> 7.19 ms per RK3 step (16.3 with
-// all of it in FP64), of 61,440 points 123 -> 105 us (168).  eps3 = 3 eps.  Not a number where a difference is not,
-// or where both denominators vanish (eps = 0 and no differences).
+// (the threes cancel), the two weights as fixed-point numbers.  The products are
+// not normalised: E_i keeps 60 bits or more, a product of two 55, a weight 53.
+// About 1,600 issue cycles of integer work for an edge and variable stand beside
+// seven FP64 instructions (448 cycles), in place of 66 of those (4,224).  Measured
+// on GB300: the detonation of 2^23 points 10.77 -> 7.19 ms per RK3 step (16.3 with
+// all of it in FP64), of 61,440 points 123 -> 105 us (168).  eps3 = 3 eps.  Not a
+// number where a difference or eps is not (or is infinite), or where a
+// denominator vanishes (eps = 0 and two indicators that are zero).
 AT_HD double fx_weno_sum(const double* c, const double* q, FxU eps3)
 {
     constexpr int G = 5;
