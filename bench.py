@@ -122,9 +122,9 @@ KERNEL_FILES = {
     "persistent": ("at_cluster.cu", "at_device.cuh", "at_fixed.cuh", "at_persist.cu"),
     "fused": ("at_device.cuh", "at_fixed.cuh", "at_fused.cu", "at_tilefused.cu"),
 }
-_SHA_STAGE = "73d66cf4bb69b05e91a580d196a0d48ac7ce65d9ba4bf313e6f34e5587bfe78f"
-_SHA_PERSISTENT = "88de10f110aa4ac4ac19ec9bb1bcacc7d4eda71be70deacfa2d9b3271044aa64"
-_SHA_FUSED = "2cefcb626dc7bb58b28d69c0890ff7df8deab82dd05c1c0139b8f3b5ffec0c8f"
+_SHA_STAGE = "28009148f9f42ed00de619e2c627b9c5efdb8b9c4a7b0ce996c270855a839452"
+_SHA_PERSISTENT = "cb4fe46b907f7fd270426eca69d61dcdb13cd3e55bd4cc881070debeddebe799"
+_SHA_FUSED = "575841c95d8c2f255dbd6d6ba93e0833ff28483dadf360e47092820fb5b5d5c4"
 PROFILED_SHA256 = {
     ("detonation-n16777216", "stage"): _SHA_STAGE,
     ("detonation-n8388608", "stage"): _SHA_STAGE,

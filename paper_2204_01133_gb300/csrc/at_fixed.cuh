@@ -117,8 +117,9 @@ constexpr uint32_t FX_EXP = 0x7ff00000u;
 constexpr int FX_GUARD = 3;  // bits kept below the last bit of the largest value
 
 // A double as a signed integer in units of 2^-FX_GUARD of its last place and its
-// exponent field (in place, bits 20..30 of the high word); a zero or subnormal
-// has no implicit bit.  Inf and NaN keep their bits, marked by the field.
+// exponent field (in place, bits 20..30 of the high word).  A zero or subnormal
+// has no implicit bit and the field of the smallest normal numbers, whose unit
+// is its own.  Inf and NaN keep their bits, marked by the field.
 struct FxV {
     int64_t m;
     uint32_t e;
@@ -130,7 +131,7 @@ AT_HD FxV fx_split(double x)
     const uint32_t hi = fx_hi(x), t = hi & FX_EXP;
     const uint64_t m = ((uint64_t)((hi & 0xfffffu) | fx_min(t, 0x100000u)) << 32 | fx_lo(x)) << GUARD;
     const int64_t s = (int32_t)hi >> 31;
-    return FxV{t == FX_EXP ? (int64_t)((uint64_t)hi << 32 | fx_lo(x)) : (int64_t)(m ^ (uint64_t)s) - s, t};
+    return FxV{t == FX_EXP ? (int64_t)((uint64_t)hi << 32 | fx_lo(x)) : (int64_t)(m ^ (uint64_t)s) - s, fx_max(t, 0x100000u)};
 }
 
 // the double that fx_split took apart (the sign of a zero aside)
@@ -138,7 +139,7 @@ AT_HD double fx_join(FxV v)
 {
     const uint64_t a = (v.m < 0 ? 0u - (uint64_t)v.m : (uint64_t)v.m) >> FX_GUARD;
     const uint32_t s = (uint32_t)((uint64_t)v.m >> 32) & 0x80000000u;
-    const uint64_t r = (a & 0xfffffffffffffull) | ((uint64_t)(v.e | s) << 32);
+    const uint64_t r = a + ((uint64_t)((v.e - 0x100000u) | s) << 32);  // the implicit bit, if any, adds one to the field
     const uint64_t x = v.e == FX_EXP ? (uint64_t)v.m : r;
     return fx_double((uint32_t)(x >> 32), (uint32_t)x);
 }
@@ -476,7 +477,7 @@ AT_HD uint64_t fx_fixed(FxU a, int e)
 AT_HD double fx_weno_sum(const double* c, const double* q, FxU eps3)
 {
     constexpr int G = 5;
-    uint32_t emax = 0;
+    uint32_t emax = 0x100000u;
 #pragma unroll
     for (int j = 0; j < 5; ++j) emax = fx_max(emax, fx_max(fx_hi(c[j]) & FX_EXP, fx_hi(q[j]) & FX_EXP));
     const int unit = (int)(emax >> 20) - 1075 - G;

@@ -59,3 +59,36 @@ def _indicator_counts(f):
         e = [x * x for x in d]
         out.append(e[1] * (3 * e[0] + e[2]) + 6 * e[0] * e[2])
     return out
+
+
+@pytest.mark.parametrize("h", (1, 2, 3))
+@pytest.mark.parametrize("k", (1, 2))
+def test_differences_of_subnormal_numbers(lib, k, h):
+    """No worse than a chain of FMAs may be: 2H + 1 roundings of partial sums,
+    each half a unit of the sum's last place."""
+    taps = (D1 if k == 1 else D2)[h]
+    rng = np.random.default_rng(8)
+    rows = [np.eye(2 * h + 1)[i] * v for i in range(2 * h + 1) for v in (5e-324, 1e-310, 2e-308, 3e-308)]
+    rows += [np.ldexp(rng.integers(-(1 << 53), 1 << 53, 2 * h + 1).astype(np.float64), -1074 - s)
+             for s in (0, 1, 2, 10, 30, 50) for _ in range(40)]
+    for f in rows:
+        exact = sum((t * Fraction(float(v)) for t, v in zip(taps, f)), Fraction(0))
+        got = _call(lib, k, f)
+        big = Fraction(float(np.abs(f).max()))
+        room = sum(abs(t) for t in taps) * big / 2 ** 53 + Fraction(2) ** -1075
+        assert abs(Fraction(got) - exact) <= (2 * h + 1) * room
+
+
+def test_join_undoes_split(tmp_path):
+    import ctypes
+    import os
+    import subprocess
+    from test_fixed_cpu import CSRC
+    src, so = tmp_path / "j.cpp", str(tmp_path / "j.so")
+    src.write_text('#include "at_fixed.cuh"\nextern "C" double j(double x) { return atk::fx_join(atk::fx_split(x)); }\n')
+    subprocess.run(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-I", CSRC, str(src), "-o", so], check=True)
+    f = ctypes.CDLL(so).j
+    f.restype, f.argtypes = ctypes.c_double, [ctypes.c_double]
+    for x in (0.0, 5e-324, 1e-310, math.nextafter(2.0 ** -1022, 0), 2.0 ** -1022, 1e-300, 1.0, 1.7e308, math.inf):
+        assert f(x) == x and f(-x) == -x
+    assert math.isnan(f(math.nan))
