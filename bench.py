@@ -122,9 +122,9 @@ KERNEL_FILES = {
     "persistent": ("at_cluster.cu", "at_device.cuh", "at_fixed.cuh", "at_persist.cu"),
     "fused": ("at_device.cuh", "at_fixed.cuh", "at_fused.cu", "at_tilefused.cu"),
 }
-_SHA_STAGE = "28009148f9f42ed00de619e2c627b9c5efdb8b9c4a7b0ce996c270855a839452"
-_SHA_PERSISTENT = "cb4fe46b907f7fd270426eca69d61dcdb13cd3e55bd4cc881070debeddebe799"
-_SHA_FUSED = "575841c95d8c2f255dbd6d6ba93e0833ff28483dadf360e47092820fb5b5d5c4"
+_SHA_STAGE = "d251e3de275ba9350c36377a4b13b6d046917112783a2db32a1d78018fce8a6f"
+_SHA_PERSISTENT = "a3740a6a97d23ea5cf76eadaf03cd208b52e89c88279a08fead7c30db8115762"
+_SHA_FUSED = "8966c90e35003880ca271e061236a319490b951b9b47d4d894f05803abb5a875"
 PROFILED_SHA256 = {
     ("detonation-n16777216", "stage"): _SHA_STAGE,
     ("detonation-n8388608", "stage"): _SHA_STAGE,

@@ -92,3 +92,69 @@ def test_join_undoes_split(tmp_path):
     for x in (0.0, 5e-324, 1e-310, math.nextafter(2.0 ** -1022, 0), 2.0 ** -1022, 1e-300, 1.0, 1.7e308, math.inf):
         assert f(x) == x and f(-x) == -x
     assert math.isnan(f(math.nan))
+
+
+def _chain(f, taps):
+    """the taps over the values by FMAs, each rounded as FP64 does"""
+    x = 0.0
+    for t, v in zip(taps, f):
+        if t:
+            x = float(t * Fraction(float(v)) + Fraction(x))
+    return x
+
+
+def _resolved(h, rng):
+    o = np.arange(-h, h + 1)
+    for g in (1.0, 1.2, 1.5, 2.0):  # a point, up and down
+        for s in (1, -1):
+            yield "%g^%d" % (g, s), lambda g=g, s=s: g ** (s * o) * (1 + 0.3 * rng.uniform(0, 1, len(o)))
+    for w in (0.1, 0.5, 2.0):
+        yield "sine %g" % w, lambda w=w: np.sin(w * o + rng.uniform(0, 6.28))
+    yield "ripple", lambda: 1 + 0.01 * np.sin(0.2 * o + rng.uniform(0, 6.28))
+    yield "bell", lambda: np.exp(-(o + rng.uniform(0, 6.28)) ** 2 / 50)
+    yield "random", lambda: rng.uniform(-1, 1, len(o))
+
+
+@pytest.mark.parametrize("h", (1, 2, 3))
+@pytest.mark.parametrize("k", (1, 2))
+def test_rows_of_a_few_binades_are_no_less_accurate_than_fmas(lib, k, h):
+    """Mean error against the exact sum, relative to the largest value: at most
+    that of the chain of FMAs on the same stencils (and two per cent: with H = 1
+    both are one rounding, and a value may be cut)."""
+    taps = (D1 if k == 1 else D2)[h]
+    rng = np.random.default_rng(12)
+    for name, row in _resolved(h, rng):
+        ours, fmas = Fraction(0), Fraction(0)
+        for _ in range(300):
+            f = row()
+            exact = sum((t * Fraction(float(v)) for t, v in zip(taps, f)), Fraction(0))
+            big = Fraction(float(np.abs(f).max()))
+            ours += abs(Fraction(_call(lib, k, f)) - exact) / big
+            fmas += abs(Fraction(_chain(f, taps)) - exact) / big
+        assert ours <= fmas * Fraction(102, 100), (name, float(ours / fmas))
+
+
+@pytest.mark.parametrize("h", (1, 2, 3))
+@pytest.mark.parametrize("k", (1, 2))
+def test_steep_rows_keep_the_absolute_bound(lib, k, h):
+    """Values growing up to 10^4 times a point: half an ulp of the result, and a
+    unit of 2^-55 of the largest value for every tap."""
+    taps = (D1 if k == 1 else D2)[h]
+    rng, o = np.random.default_rng(14), np.arange(-h, h + 1)
+    for g in (2.7, 4.0, 7.4, 16.0, 64.0, 1e4):
+        for i in range(200):
+            f = g ** ((1 if i % 2 else -1) * o) * (1 + 0.3 * rng.uniform(0, 1, len(o)))
+            exact = sum((t * Fraction(float(v)) for t, v in zip(taps, f)), Fraction(0))
+            big = Fraction(float(np.abs(f).max()))
+            room = Fraction(32 + sum(abs(t) for t in taps)) * big / 2 ** 55
+            assert abs(Fraction(_call(lib, k, f)) - exact) <= abs(exact) / 2 ** 53 + room
+
+
+def test_large_second_differences(lib):
+    """Values of one exponent, nothing cut: half an ulp, and 2^-50 of the largest
+    value where the sum does not fit 64 bits."""
+    rng = np.random.default_rng(13)
+    for _ in range(3000):
+        f = rng.uniform(1.0, 2.0, 7) * rng.choice([-1.0, 1.0], 7)
+        exact = sum((t * Fraction(float(v)) for t, v in zip(D2[3], f)), Fraction(0))
+        assert abs(Fraction(_call(lib, 2, f)) - exact) <= abs(exact) * Fraction(1001, 1000) / 2 ** 53 + Fraction(2) ** -49
