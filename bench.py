@@ -122,9 +122,9 @@ KERNEL_FILES = {
     "persistent": ("at_cluster.cu", "at_device.cuh", "at_fixed.cuh", "at_persist.cu"),
     "fused": ("at_device.cuh", "at_fixed.cuh", "at_fused.cu", "at_tilefused.cu"),
 }
-_SHA_STAGE = "d251e3de275ba9350c36377a4b13b6d046917112783a2db32a1d78018fce8a6f"
-_SHA_PERSISTENT = "a3740a6a97d23ea5cf76eadaf03cd208b52e89c88279a08fead7c30db8115762"
-_SHA_FUSED = "8966c90e35003880ca271e061236a319490b951b9b47d4d894f05803abb5a875"
+_SHA_STAGE = "6e784c929c16a6d751d35abe7a4d62e209453830427fb470dbc828ec5c52f3fa"
+_SHA_PERSISTENT = "fb9e5b73f0d501498a0e85ccf9e3a519b7101855cb5784487c8b7391eed81324"
+_SHA_FUSED = "a2353bf33374fa56e050de38aa1370357b223d3d0b75913c5475e50c1216a403"
 PROFILED_SHA256 = {
     ("detonation-n16777216", "stage"): _SHA_STAGE,
     ("detonation-n8388608", "stage"): _SHA_STAGE,

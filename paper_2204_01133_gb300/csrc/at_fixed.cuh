@@ -159,10 +159,15 @@ AT_HD double fx_join(FxV v)
 // its integer at the exponent field emax (at least its own), cut downwards
 AT_HD int64_t fx_at(FxV v, uint32_t emax) { return v.m >> fx_min((emax - v.e) >> 20, 63u); }
 
+// Inf and NaN aside, fx_at of fx_split in fewer instructions, for values read
+// once: i is the implicit bit, 0 for a subnormal, whose field then counts as 1
 template <int GUARD>
 AT_HD int64_t fx_align(double x, uint32_t emax)
 {
-    return fx_at(fx_split<GUARD>(x), emax);
+    const uint32_t hi = fx_hi(x), t = hi & FX_EXP, i = fx_min(t, 0x100000u);
+    const uint64_t m = ((uint64_t)((hi & 0xfffffu) | i) << 32 | fx_lo(x)) << GUARD;
+    const int64_t s = (int32_t)hi >> 31;
+    return ((int64_t)(m ^ (uint64_t)s) - s) >> fx_min((emax - 0x100000u - t + i) >> 20, 63u);
 }
 
 // the integer x in fx_at's units as a double, rounded to nearest; *ok is
@@ -466,15 +471,14 @@ AT_HD FxU fx_leading(uint64_t hi, uint64_t lo, int e)
         w0 = z ? 0u : w0;
         e -= z ? 32 : 0;
     }
-    if (w3 == 0) e = FX_TINY;
 #ifdef __CUDA_ARCH__
-    const int lz = __clz((int)(w3 | 1u));
-    return FxU{(uint64_t)__funnelshift_l(w2, w3, lz) << 32 | __funnelshift_l(w1, w2, lz), e - lz};
+    const int lz = __clz((int)w3);  // 32 for zero
+    const uint64_t m = (uint64_t)__funnelshift_l(w2, w3, lz) << 32 | __funnelshift_l(w1, w2, lz);
 #else
-    const int lz = __builtin_clz(w3 | 1u);
-    const uint64_t v = (uint64_t)w3 << 32 | w2;
-    return FxU{(v << lz) | (lz ? w1 >> (32 - lz) : 0u), e - lz};
+    const int lz = w3 ? __builtin_clz(w3) : 32;
+    const uint64_t m = (((uint64_t)w3 << 32 | w2) << lz) | (lz ? w1 >> (32 - lz) : 0u);
 #endif
+    return FxU{m, e - lz - ((lz & 32) << 15)};  // zero: 2^20 further down
 }
 
 // a in units of 2^e, less than 2^64 of them

@@ -158,3 +158,19 @@ def test_large_second_differences(lib):
         f = rng.uniform(1.0, 2.0, 7) * rng.choice([-1.0, 1.0], 7)
         exact = sum((t * Fraction(float(v)) for t, v in zip(D2[3], f)), Fraction(0))
         assert abs(Fraction(_call(lib, 2, f)) - exact) <= abs(exact) * Fraction(1001, 1000) / 2 ** 53 + Fraction(2) ** -49
+
+
+def test_weno_sum_of_differences_next_to_the_subnormal_range(soft):
+    """Subnormal differences beside small normal ones, and subnormal ones alone;
+    eps in proportion.  The general bound, and the result's own last place (a
+    result below the normal range is zero)."""
+    rng = np.random.default_rng(15)
+    for i in range(400):
+        c, q = (np.ldexp(rng.uniform(-1, 1, 5), rng.integers(-1030, (-1021, -1005, -980)[i % 3], 5)) for _ in range(2))
+        got = Fraction(_weno(soft, c, q, 1e-6))
+        big = Fraction(float(max(np.abs(c).max(), np.abs(q).max())))
+        exact = _weno_exact(c, q, 1e-6)
+        if abs(exact) < Fraction(2) ** -1022:
+            assert got == 0 or abs(got - exact) <= 32 * big / 2 ** 53 + Fraction(2) ** -1074
+        else:
+            assert abs(got - exact) <= 32 * big / 2 ** 53 + Fraction(2) ** -1074
