@@ -123,7 +123,7 @@ KERNEL_FILES = {
     "fused": ("at_device.cuh", "at_fixed.cuh", "at_fused.cu", "at_tilefused.cu"),
 }
 _SHA_STAGE = "6e784c929c16a6d751d35abe7a4d62e209453830427fb470dbc828ec5c52f3fa"
-_SHA_PERSISTENT = "fb9e5b73f0d501498a0e85ccf9e3a519b7101855cb5784487c8b7391eed81324"
+_SHA_PERSISTENT = "7f3ab37ef47676a1fa3618d9e21771d44ee55d0c21031ac6fd964add8773a377"
 _SHA_FUSED = "a2353bf33374fa56e050de38aa1370357b223d3d0b75913c5475e50c1216a403"
 PROFILED_SHA256 = {
     ("detonation-n16777216", "stage"): _SHA_STAGE,

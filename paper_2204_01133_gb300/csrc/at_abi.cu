@@ -27,7 +27,7 @@ cudaError_t atk_launch_reset(const atk::StageArgs& a, const atk::ResetArgs& z, c
 cudaError_t atk_launch_ring_recompute(const atk::StageArgs& a, int pde, int order, int rk, const double* um,
                                       int64_t m, cudaStream_t st);
 cudaError_t atk_set_smem_limits();
-int64_t atk_persist_capacity(int pde, int order, int B, int device);
+int64_t atk_persist_capacity(int pde, int order, int B, int variant, int device);
 int atk_cluster_size(int pde, int order, int B, int64_t P, int R, int S, int device);
 cudaError_t atk_launch_cluster(const atk::StageArgs& a, int order, int csize, int64_t level0, int64_t nsteps,
                                cudaStream_t st);
@@ -40,7 +40,7 @@ cudaError_t atk_launch_tile_fused(const atk::StageArgs& a, int pde, int order, i
                                   double* uout, cudaStream_t st);
 cudaError_t atk_launch_fused(const atk::StageArgs& a, int order, int64_t n, const double* uin, double* uout,
                              cudaStream_t st);
-cudaError_t atk_launch_persist(const atk::StageArgs& a, int pde, int order, int64_t level0, int64_t nsteps,
+cudaError_t atk_launch_persist(const atk::StageArgs& a, int pde, int order, int variant, int64_t level0, int64_t nsteps,
                                cudaStream_t st);
 int atk_batch_variant(int pde, int order);
 cudaError_t atk_launch_batch(int variant, const atk::StageArgs* tab, int64_t* lvl, int64_t* left, const int* order,
@@ -409,6 +409,8 @@ struct at_ctx {
     int path = AT_PATH_AUTO;       // at_set_option(AT_OPT_PATH)
     int last_path = 0;             // path of the last at_step
     int64_t persist_cap = 0;       // PEs one cooperative launch can hold (0: unavailable)
+    int persist_variant = 0;       // the variant of the kernel that holds this problem's PEs
+    bool persist_auto = false;     // whether the automatic rule takes it
     int cluster_c = 0;             // CTAs of the one-cluster kernel for this problem (0: not used)
     int sms = 0;                   // SMs of the device
     int64_t fit_key[8] = {-1};     // what the capacities below were asked for
@@ -577,10 +579,20 @@ int at_set_delays(at_ctx* c, const at_delays* dl)
     if (std::memcmp(key, c->fit_key, sizeof key) != 0) {
         if (c->sms == 0) cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device);
         c->stage_tw = stage_window(&c->pb, L, c->sms);
-        c->persist_cap = (c->pb.pde == AT_ADVDIFF || c->pb.pde == AT_RNS)
-                             ? atk_persist_capacity(c->pb.pde, c->pb.order, c->pb.pe_size, c->device)
-                             : 0;
-        if (c->persist_cap > kPersistMaxPE) c->persist_cap = kPersistMaxPE;
+        c->persist_cap = 0;
+        for (int v = 0; v < 3 && (v == 0 || L.P > c->persist_cap); ++v) {
+            const int64_t cap = std::min(
+                atk_persist_capacity(c->pb.pde, c->pb.order, c->pb.pe_size, v, c->device), kPersistMaxPE);
+            if (cap <= c->persist_cap) continue;
+            c->persist_cap = cap;
+            c->persist_variant = v;
+        }
+        // large PEs of the reacting flow are no faster resident than with one
+        // launch per stage (us per step, resident and per stage: 152 PEs of 600
+        // points 56.3 and 55.5, of 749 68.8 and 64.2, 150 of 800 73.5 and 66.0, 304
+        // of 480, dense, 81.7 and 73.9): the automatic rule leaves them there from
+        // 750 points on and where only dense rows fit
+        c->persist_auto = c->pb.pde == AT_ADVDIFF || (c->persist_variant < 2 && c->pb.pe_size < 750);
         c->cluster_c = c->pb.pde == AT_ADVDIFF
                            ? atk_cluster_size(c->pb.pde, c->pb.order, c->pb.pe_size, L.P, L.R, L.S, c->device)
                            : 0;
@@ -634,7 +646,8 @@ int at_step(at_ctx* c, int64_t nsteps)
                          atk_tile_fused_supported(c->pb.pde, c->pb.order, c->pb.pe_size, c->pb.rk, L.q) &&
                          (!is_weno(c->pb.pde) || L.wpp == 1 || L.Tw >= L.S * L.H);
     const bool cluster_ok = c->cluster_c > 0 && !c->arrival && c->withhold_pe < 0;
-    bool persist = c->path == AT_PATH_PERSISTENT || (c->path == AT_PATH_AUTO && can_persist);
+    bool persist = c->path == AT_PATH_PERSISTENT ||
+                   (c->path == AT_PATH_AUTO && can_persist && (c->persist_auto || c->arrival || c->withhold_pe >= 0));
     // advection-diffusion beyond one thread-block cluster: the step-fused
     // kernel is faster than the neighbour-wait kernel (measured on GB300 at
     // 256 PEs of 64 points: 10.3 against 13.1 us per step); delays by arrival
@@ -719,7 +732,8 @@ int at_step(at_ctx* c, int64_t nsteps)
         e = record(c, true);
         if (e == cudaSuccess)
             e = cluster ? atk_launch_cluster(a, c->pb.order, c->cluster_c, c->level, nsteps, c->stream)
-                        : atk_launch_persist(a, c->pb.pde, c->pb.order, c->level, nsteps, c->stream);
+                        : atk_launch_persist(a, c->pb.pde, c->pb.order, c->persist_variant, c->level, nsteps,
+                                             c->stream);
         if (e != cudaSuccess) return cuda_fail(e, "persistent kernel launch");
         e = record(c, false);
         if (e != cudaSuccess) return cuda_fail(e, "profiling event");

@@ -160,11 +160,20 @@ __device__ __forceinline__ void bar_arrive_p(int p, int count)
 // A failed wait records the stage in s_abort_at before the halo warp
 // arrives; the workers stop at that stage and the halo warp matches the one
 // arrival it would otherwise have consumed, so every barrier completes.
-template <int PDE, int H>
-__global__ void __launch_bounds__(288, 2) persist_central(const StageArgs a, int64_t level0, int64_t nsteps)
+//
+// How many PEs fit the chip is registers and shared memory.  CTAS = 2 of 288
+// threads an SM leaves the registers the code wants (85 at order 6); CTAS = 3 holds
+// it to 72 for more PEs (none spilt, 3 to 6 % slower where both fit: 304 PEs of
+// 64 points 19.1 and 20.8 us per step; 456 of them 24.7, one launch per stage
+// 40.3).  DENSE has the reacting flow's rows as doubles, split where they are
+// read, in 27 words a point instead of 34, for large PEs that no other holds (100
+// of 400 points 52.9 us against 39.9).
+template <int PDE, int H, int CTAS, bool DENSE>
+__global__ void __launch_bounds__(288, CTAS) persist_central(const StageArgs a, int64_t level0, int64_t nsteps)
 {
     using P = Phys<PDE>;
     constexpr int NV = P::NV, ND = P::ND;
+    constexpr bool SPLITROWS = P::SPLIT > 0 && !DENSE;
     const int B = a.B, W2 = B + 2 * H, S = a.S;
     const int64_t pe = place_rank(a);
     const int64_t nbr[2] = {pe == 0 ? a.P - 1 : pe - 1, pe == a.P - 1 ? 0 : pe + 1};
@@ -176,9 +185,9 @@ __global__ void __launch_bounds__(288, 2) persist_central(const StageArgs a, int
     double* G2 = E + B;            // derived rows by stage parity: [2][W2] doubles, or the
                                    // reacting flow's split rows
     constexpr int NG = P::SPLIT > 0 ? P::SPLIT : ND;
-    const int gwords = P::SPLIT > 0 ? split_words(NG, W2) : NG * W2;
+    const int gwords = SPLITROWS ? split_words(NG, W2) : NG * W2;
     auto rows = [&](int p) {
-        if constexpr (P::SPLIT > 0) {
+        if constexpr (SPLITROWS) {
             int64_t* m = (int64_t*)(G2 + p * gwords);
             return SplitRows{m, (uint32_t*)(m + NG * W2), W2};
         } else {
@@ -461,40 +470,47 @@ __global__ void counters_set(int64_t* done, int64_t P, int64_t value, int* abort
     }
 }
 
-template <int PDE, int H>
-void* persist_fn()
-{
-    return (void*)persist_central<PDE, H>;
-}
-
 } // namespace atk
 
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
 namespace {
-void* persist_kernel(int pde, int order)
+// the variants of the kernel, in the order in which they are preferred
+constexpr int kVariants = 3;
+
+template <int H>
+void* persist_fn(int pde, int variant)
 {
-    if (pde == atk::ADVDIFF) {
-        if (order == 2) return atk::persist_fn<atk::ADVDIFF, 1>();
-        if (order == 4) return atk::persist_fn<atk::ADVDIFF, 2>();
-        return atk::persist_fn<atk::ADVDIFF, 3>();
-    }
-    if (pde == atk::RNS) {
-        if (order == 2) return atk::persist_fn<atk::RNS, 1>();
-        if (order == 4) return atk::persist_fn<atk::RNS, 2>();
-        return atk::persist_fn<atk::RNS, 3>();
-    }
-    return nullptr;
+    if (pde == atk::ADVDIFF) return variant == 0 ? (void*)atk::persist_central<atk::ADVDIFF, H, 2, false> : nullptr;
+    if (pde != atk::RNS) return nullptr;
+    return variant == 0   ? (void*)atk::persist_central<atk::RNS, H, 2, false>
+           : variant == 1 ? (void*)atk::persist_central<atk::RNS, H, 3, false>
+                          : (void*)atk::persist_central<atk::RNS, H, 3, true>;
+}
+
+void* persist_kernel(int pde, int order, int variant)
+{
+    return order == 2 ? persist_fn<1>(pde, variant) : order == 4 ? persist_fn<2>(pde, variant) : persist_fn<3>(pde, variant);
+}
+
+size_t persist_smem_bytes(int pde, int B, int H, int variant)
+{
+    const int W2 = B + 2 * H, nv = pde == atk::RNS ? 4 : 1, rows = pde == atk::RNS ? atk::Phys<atk::RNS>::SPLIT : 1;
+    const size_t words = pde == atk::RNS && variant < 2 ? atk::split_words(rows, W2) : rows * W2;
+    return sizeof(double) * ((size_t)3 * nv * B + 2 * words + (size_t)B);
+}
+
+// The PE sizes the path takes: u, argument and accumulator, eight (one) rows of
+// derived quantities by stage parity, their halo levels and a factor for each
+// point within 200 KB (the reacting flow at order 6: up to 872 points).
+bool persist_takes(int pde, int B, int H)
+{
+    const int nv = pde == atk::RNS ? 4 : 1, nd = pde == atk::RNS ? 8 : 1;
+    return sizeof(double) * ((size_t)3 * nv * B + (size_t)2 * nd * (B + 2 * H) + (size_t)2 * H * (AT_QMAX + 1) * nd +
+                             (size_t)B) <= 200 * 1024;
 }
 } // namespace
-
-size_t atk_persist_smem_bytes(int pde, int B, int H)
-{
-    const int nv = pde == atk::RNS ? 4 : 1, W2 = B + 2 * H;
-    const size_t rows = pde == atk::RNS ? atk::split_words(atk::Phys<atk::RNS>::SPLIT, W2) : W2;
-    return sizeof(double) * ((size_t)3 * nv * B + 2 * rows + (size_t)B);
-}
 
 // worker warps for the PE's points (at least two roles' worth for phase A)
 // plus one halo warp
@@ -509,14 +525,14 @@ int atk_persist_block(int pde, int B)
     return want + 32;
 }
 
-// how many PEs one cooperative launch can hold (0: not available)
-int64_t atk_persist_capacity(int pde, int order, int B, int device)
+// how many PEs one cooperative launch of a variant can hold (0: not available)
+int64_t atk_persist_capacity(int pde, int order, int B, int variant, int device)
 {
-    void* fn = persist_kernel(pde, order);
-    if (!fn) return 0;
+    void* fn = variant < kVariants ? persist_kernel(pde, order, variant) : nullptr;
     const int H = order / 2;
-    const size_t smem = atk_persist_smem_bytes(pde, B, H);
-    if (smem > 200 * 1024) return 0;
+    if (!fn || !persist_takes(pde, B, H)) return 0;
+    const size_t smem = persist_smem_bytes(pde, B, H, variant);
+    if (smem > 226 * 1024) return 0;
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
     int per_sm = 0, sms = 0, coop = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, atk_persist_block(pde, B), smem) != cudaSuccess)
@@ -526,16 +542,16 @@ int64_t atk_persist_capacity(int pde, int order, int B, int device)
     return (int64_t)per_sm * sms;
 }
 
-cudaError_t atk_launch_persist(const atk::StageArgs& a, int pde, int order, int64_t level0, int64_t nsteps,
+cudaError_t atk_launch_persist(const atk::StageArgs& a, int pde, int order, int variant, int64_t level0, int64_t nsteps,
                                cudaStream_t st)
 {
-    void* fn = persist_kernel(pde, order);
+    void* fn = persist_kernel(pde, order, variant);
     if (!fn) return cudaErrorInvalidValue;
     atk::counters_set<<<(unsigned)((a.P + 255) / 256 < 1024 ? (a.P + 255) / 256 : 1024), 256, 0, st>>>(
         a.done, a.P, (level0 - a.R) * a.S, a.abort_flag, a.place_count);  // raised to level0 S by each PE's prologue
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const size_t smem = atk_persist_smem_bytes(pde, a.B, order / 2);
+    const size_t smem = persist_smem_bytes(pde, a.B, order / 2, variant);
     // the attribute is per kernel, not per context: set it for this launch
     e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;

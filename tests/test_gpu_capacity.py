@@ -1,0 +1,66 @@
+"""How many PEs the resident kernels hold on a GB300 (152 SMs), at the edges of
+what each variant of them takes.  All give the bits of the per-stage path."""
+import numpy as np
+import pytest
+
+from paper_2204_01133_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+OPT_ARRIVAL = 3
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _gpu():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("the counts are those of 152 SMs")
+    from paper_2204_01133_gb300 import build
+    build.build()
+
+
+def _run(pb, u0, steps, path):
+    from paper_2204_01133_gb300.api import Solver
+    s = Solver(pb, u0, path=path)
+    s.run(steps)
+    out = s.read_state(), s.read_delays(), s.stats()
+    s.close()
+    return out
+
+
+@pytest.mark.parametrize("order", [2, 4, 6])
+@pytest.mark.parametrize("pe_size,pes", [(16, 1368), (24, 1064), (32, 760), (48, 608), (64, 304), (64, 305), (64, 456),
+                                         (280, 456), (320, 456), (421, 304), (488, 304), (749, 152), (750, 152),
+                                         (850, 152), (872, 152)])
+def test_flames_on_the_persistent_path(order, pe_size, pes):
+    pb, u0 = W.rns(case="flame", n=pe_size * pes, pe_size=pe_size, order=order, mode="at", k_max=3, seed=2)
+    a, b = _run(pb, u0, 3, "persistent"), _run(pb, u0, 3, "stage")
+    assert a[2].path == 2
+    assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
+
+
+@pytest.mark.parametrize("pe_size,pes", [(64, 456), (320, 456), (872, 20)])
+def test_delays_by_arrival(pe_size, pes):
+    """They have no other path."""
+    from paper_2204_01133_gb300.api import Solver
+    pb, u0 = W.rns(case="flame", n=pe_size * pes, pe_size=pe_size, mode="at", k_max=3, seed=2)
+    s = Solver(pb, u0)
+    s.set_option(OPT_ARRIVAL, 1)
+    s.run(5)
+    assert s.stats().path == 2 and np.isfinite(s.read_state()).all()
+    s.close()
+
+
+@pytest.mark.parametrize("pe_size,pes", [(32, 760), (64, 384), (64, 456), (200, 456)])
+def test_the_automatic_rule_keeps_them_resident(pe_size, pes):
+    pb, u0 = W.rns(case="flame", n=pe_size * pes, pe_size=pe_size, mode="at", k_max=3, seed=2)
+    assert _run(pb, u0, 2, "auto")[2].path == 2
+
+
+@pytest.mark.parametrize("pe_size", [873, 900])
+def test_larger_pes_are_refused(pe_size):
+    from paper_2204_01133_gb300.api import AtError
+    pb, u0 = W.rns(case="flame", n=pe_size * 4, pe_size=pe_size, mode="at", k_max=3, seed=2)
+    with pytest.raises(AtError):
+        _run(pb, u0, 1, "persistent")
