@@ -32,8 +32,8 @@ int atk_cluster_size(int pde, int order, int B, int64_t P, int R, int S, int dev
 cudaError_t atk_launch_cluster(const atk::StageArgs& a, int order, int csize, int64_t level0, int64_t nsteps,
                                cudaStream_t st);
 bool atk_fused_supported(int pde, int order, int B, int S);
-int atk_fused_multi_w(int order, int rk, int B, int S, int64_t P, int device);
-cudaError_t atk_launch_fused_steps(const atk::StageArgs& a, int order, int W, int64_t level0, int64_t nsteps,
+int atk_fused_multi(int order, int rk, int B, int S, int64_t P, int device);
+cudaError_t atk_launch_fused_steps(const atk::StageArgs& a, int order, int variant, int64_t level0, int64_t nsteps,
                                    double* b0, double* b1, cudaStream_t st);
 bool atk_tile_fused_supported(int pde, int order, int B, int rk, int q);
 cudaError_t atk_launch_tile_fused(const atk::StageArgs& a, int pde, int order, int64_t n, const double* uin,
@@ -415,7 +415,7 @@ struct at_ctx {
     int sms = 0;                   // SMs of the device
     int64_t fit_key[8] = {-1};     // what the capacities below were asked for
     int stage_tw = 0;              // window length of the per-stage kernels (stage_window)
-    int fused_multi_w = 0;         // PEs per CTA when the fused path's steps fit one cooperative launch
+    int fused_multi = 0;           // variant of the multi-step kernel that holds the fused path's CTAs at once (0: none)
     int64_t wait_limit = 4000000;  // polls of a bounded wait
     int64_t withhold_pe = -1;
     int arrival = 0;               // at_set_option(AT_OPT_ARRIVAL)
@@ -596,9 +596,9 @@ int at_set_delays(at_ctx* c, const at_delays* dl)
         c->cluster_c = c->pb.pde == AT_ADVDIFF
                            ? atk_cluster_size(c->pb.pde, c->pb.order, c->pb.pe_size, L.P, L.R, L.S, c->device)
                            : 0;
-        c->fused_multi_w = atk_fused_supported(c->pb.pde, c->pb.order, c->pb.pe_size, L.S)
-                               ? atk_fused_multi_w(c->pb.order, c->pb.rk, c->pb.pe_size, L.S, L.P, c->device)
-                               : 0;
+        c->fused_multi = atk_fused_supported(c->pb.pde, c->pb.order, c->pb.pe_size, L.S)
+                             ? atk_fused_multi(c->pb.order, c->pb.rk, c->pb.pe_size, L.S, L.P, c->device)
+                             : 0;
         std::memcpy(c->fit_key, key, sizeof key);
     }
     cudaGetLastError();  // an unavailable persistent path is not an error
@@ -672,7 +672,7 @@ int at_step(at_ctx* c, int64_t nsteps)
         // after an odd number of steps the result is copied back
         const double* cur = u;
         double* nxt = A;
-        if (c->fused_multi_w > 0 && nsteps > 0) {
+        if (c->fused_multi > 0 && nsteps > 0) {
             // every CTA resident: all steps in one cooperative launch
             atk::StageArgs a = c->base;
             a.level = c->level;
@@ -680,7 +680,7 @@ int at_step(at_ctx* c, int64_t nsteps)
             a.withhold_pe = c->withhold_pe;
             e = record(c, true);
             if (e == cudaSuccess)
-                e = atk_launch_fused_steps(a, c->pb.order, c->fused_multi_w, c->level, nsteps, u, A, c->stream);
+                e = atk_launch_fused_steps(a, c->pb.order, c->fused_multi, c->level, nsteps, u, A, c->stream);
             if (e != cudaSuccess) return cuda_fail(e, "fused multi-step kernel launch");
             e = record(c, false);
             if (e != cudaSuccess) return cuda_fail(e, "profiling event");

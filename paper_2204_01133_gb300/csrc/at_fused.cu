@@ -331,10 +331,18 @@ __device__ bool fused_wait_ge(const StageArgs& a, int64_t* ctr, int64_t target)
 // warps per PE of the multi-step kernel with W PEs a CTA
 __host__ __device__ constexpr int steps_wpp(int W, int ppl) { return W == 2 && ppl >= 2 ? (ppl == 3 ? 3 : 2) : 1; }
 
-template <int H, int PPL, int RK, int W>
-__global__ void __launch_bounds__(32 * (W * steps_wpp(W, PPL) + 1)) steps_fused_advdiff(const StageArgs a, double* __restrict__ b0,
-                                                                    double* __restrict__ b1, int64_t level0,
-                                                                    int64_t nsteps)
+// CTAs an SM that the full variant of W = 8 keeps registers for: those that fitted
+// before u^n stayed in registers from step to step (56 of them a thread for PEs
+// of 32 and 64 points, 72 for 96 and 128)
+__host__ __device__ constexpr int steps_min_ctas(int H, int ppl)
+{
+    return ppl <= 2 ? 4 : (ppl <= 4 ? (H == 1 ? 4 : 3) : (H == 1 ? 3 : 0));
+}
+
+// CTAS: so many an SM at least (0: as the registers fall)
+template <int H, int PPL, int RK, int W, int CTAS>
+__global__ void __launch_bounds__(32 * (W * steps_wpp(W, PPL) + 1), CTAS)
+    steps_fused_advdiff(const StageArgs a, double* __restrict__ b0, double* __restrict__ b1, int64_t level0, int64_t nsteps)
 {
     extern __shared__ double sm[];
     __shared__ int s_fail;
@@ -412,40 +420,45 @@ void* fused_fn(int H, int rk, int ppl)
     return fused_fn_rk<3>(rk, ppl);
 }
 
-// the multi-step kernel with W = 2, 4 or 8 PEs per CTA
-template <int H, int RK, int W>
-void* fused_steps_fn_ppl(int ppl)
+// the variants of the multi-step kernel, in the order in which they are preferred
+// (0: none): 2, 4 and 8 PEs a CTA, and 8 with registers for more CTAs an SM
+constexpr int kStepsVariants = 4;
+constexpr int steps_w(int variant) { return variant == 1 ? 2 : (variant == 2 ? 4 : 8); }
+
+template <int H, int RK, int PPL>
+void* fused_steps_fn_v(int variant)
+{
+    if (variant == 1) return (void*)atk::steps_fused_advdiff<H, PPL, RK, 2, 0>;
+    if (variant == 2) return (void*)atk::steps_fused_advdiff<H, PPL, RK, 4, 0>;
+    if (variant == 3) return (void*)atk::steps_fused_advdiff<H, PPL, RK, 8, 0>;
+    return (void*)atk::steps_fused_advdiff<H, PPL, RK, 8, atk::steps_min_ctas(H, PPL)>;
+}
+
+template <int H, int RK>
+void* fused_steps_fn_ppl(int ppl, int variant)
 {
     switch (ppl) {
-    case 1: return (void*)atk::steps_fused_advdiff<H, 1, RK, W>;
-    case 2: return (void*)atk::steps_fused_advdiff<H, 2, RK, W>;
-    case 3: return (void*)atk::steps_fused_advdiff<H, 3, RK, W>;
-    case 4: return (void*)atk::steps_fused_advdiff<H, 4, RK, W>;
-    default: return (void*)atk::steps_fused_advdiff<H, 8, RK, W>;
+    case 1: return fused_steps_fn_v<H, RK, 1>(variant);
+    case 2: return fused_steps_fn_v<H, RK, 2>(variant);
+    case 3: return fused_steps_fn_v<H, RK, 3>(variant);
+    case 4: return fused_steps_fn_v<H, RK, 4>(variant);
+    default: return fused_steps_fn_v<H, RK, 8>(variant);
     }
 }
 
-template <int H, int W>
-void* fused_steps_fn_rk(int rk, int ppl)
+template <int H>
+void* fused_steps_fn_rk(int rk, int ppl, int variant)
 {
-    if (rk == atk::RK4) return fused_steps_fn_ppl<H, atk::RK4, W>(ppl);
-    if (rk == atk::RK3TVD) return fused_steps_fn_ppl<H, atk::RK3TVD, W>(ppl);
-    return fused_steps_fn_ppl<H, atk::RK2, W>(ppl);
+    if (rk == atk::RK4) return fused_steps_fn_ppl<H, atk::RK4>(ppl, variant);
+    if (rk == atk::RK3TVD) return fused_steps_fn_ppl<H, atk::RK3TVD>(ppl, variant);
+    return fused_steps_fn_ppl<H, atk::RK2>(ppl, variant);
 }
 
-template <int W>
-void* fused_steps_fn_h(int H, int rk, int ppl)
+void* fused_steps_fn(int H, int rk, int ppl, int variant)
 {
-    if (H == 1) return fused_steps_fn_rk<1, W>(rk, ppl);
-    if (H == 2) return fused_steps_fn_rk<2, W>(rk, ppl);
-    return fused_steps_fn_rk<3, W>(rk, ppl);
-}
-
-void* fused_steps_fn(int H, int rk, int ppl, int W)
-{
-    return W == 2   ? fused_steps_fn_h<2>(H, rk, ppl)
-           : W == 4 ? fused_steps_fn_h<4>(H, rk, ppl)
-                    : fused_steps_fn_h<8>(H, rk, ppl);
+    if (H == 1) return fused_steps_fn_rk<1>(rk, ppl, variant);
+    if (H == 2) return fused_steps_fn_rk<2>(rk, ppl, variant);
+    return fused_steps_fn_rk<3>(rk, ppl, variant);
 }
 
 size_t fused_smem(int B, int H, int S, int W = kFusedW)
@@ -467,14 +480,14 @@ bool atk_fused_supported(int pde, int order, int B, int S)
     return pde == atk::ADVDIFF && (B == 32 || B == 64 || B == 96 || B == 128 || B == 256) && B >= S * (order / 2);
 }
 
-// CTAs (of W = 2, 4 or 8 PEs) that one cooperative launch of the multi-step
-// kernel holds at once (0: not available)
 int fused_steps_block(int B, int W) { return 32 * (W * atk::steps_wpp(W, B / 32) + 1); }
 
-int64_t atk_fused_capacity(int order, int rk, int B, int S, int W, int device)
+// CTAs that one cooperative launch of a variant of the multi-step kernel holds
+// at once (0: not available)
+int64_t atk_fused_capacity(int order, int rk, int B, int S, int variant, int device)
 {
-    const int H = order / 2;
-    void* fn = fused_steps_fn(H, rk, B / 32, W);
+    const int H = order / 2, W = steps_w(variant);
+    void* fn = fused_steps_fn(H, rk, B / 32, variant);
     const size_t smem = fused_smem(B, H, S, W);
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
         cudaGetLastError();
@@ -490,32 +503,32 @@ int64_t atk_fused_capacity(int order, int rk, int B, int S, int W, int device)
     return (int64_t)per_sm * sms;
 }
 
-int64_t atk_fused_ctas(int64_t P, int W) { return (P + W - 1) / W; }
-
-// PEs per CTA of the multi-step kernel for P PEs, or 0 when its CTAs do not
-// fit one cooperative launch: 2, on two warps each, where that is one CTA an SM
-// at most; 4 where they fit (more SMs share the stages of a small problem), else
-// 8 (measured on GB300, PEs of 64 points, us per step: 2^14 points 5.9 with 2, 7.4
-// with 4, 8.9 with 8; 2^18 points 20.6 with 8, where 4 no longer fits and takes
-// one launch per step: 22.5)
-int atk_fused_multi_w(int order, int rk, int B, int S, int64_t P, int device)
+// Variant of the multi-step kernel for P PEs, or 0 when none holds them in one
+// cooperative launch: 2 PEs a CTA, on two warps each, where that is one CTA an SM at
+// most; 4 where they fit (more SMs share the stages of a small problem); 8; 8 with
+// registers for more CTAs an SM (measured on GB300, PEs of 64 points, us per step:
+// 2^14 points 5.9 with 2, 7.4 with 4, 8.9 with 8; 3,000 PEs 16.4 with 8, 16.9 with
+// the registers of the last; 4,096 PEs 21.2 with those, 22.6 with one launch per
+// step)
+int atk_fused_multi(int order, int rk, int B, int S, int64_t P, int device)
 {
     int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) return 0;
-    if (atk_fused_ctas(P, 2) <= sms && atk_fused_ctas(P, 2) <= atk_fused_capacity(order, rk, B, S, 2, device)) return 2;
-    for (int W = 4; W <= 8; W += 4)
-        if (atk_fused_ctas(P, W) <= atk_fused_capacity(order, rk, B, S, W, device)) return W;
+    for (int v = 1; v <= kStepsVariants; ++v) {
+        const int64_t ctas = (P + steps_w(v) - 1) / steps_w(v);
+        if (v == 1 && ctas > sms) continue;
+        if (ctas <= atk_fused_capacity(order, rk, B, S, v, device)) return v;
+    }
     return 0;
 }
 
-// steps level0 .. level0 + nsteps - 1 in one cooperative launch of CTAs of W
-// PEs: u^{level0} in b0, the result in b0 (even nsteps) or b1 (odd)
-cudaError_t atk_launch_fused_steps(const atk::StageArgs& a, int order, int W, int64_t level0, int64_t nsteps,
+// steps level0 .. level0 + nsteps - 1 in one cooperative launch of a variant: u^{level0} in b0, the result in b0 (even nsteps) or b1 (odd)
+cudaError_t atk_launch_fused_steps(const atk::StageArgs& a, int order, int variant, int64_t level0, int64_t nsteps,
                                    double* b0, double* b1, cudaStream_t st)
 {
-    const int H = order / 2;
-    const int64_t C = atk_fused_ctas(a.P, W);
-    void* fn = fused_steps_fn(H, a.rk, a.B / 32, W);
+    const int H = order / 2, W = steps_w(variant);
+    const int64_t C = (a.P + W - 1) / W;
+    void* fn = fused_steps_fn(H, a.rk, a.B / 32, variant);
     const size_t smem = fused_smem(a.B, H, a.S, W);
     atk::fused_counters_set<<<(unsigned)((C + 255) / 256 < 1024 ? (C + 255) / 256 : 1024), 256, 0, st>>>(
         a.done, C, level0, a.abort_flag, a.place_count);

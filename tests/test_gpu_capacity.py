@@ -64,3 +64,17 @@ def test_larger_pes_are_refused(pe_size):
     pb, u0 = W.rns(case="flame", n=pe_size * 4, pe_size=pe_size, mode="at", k_max=3, seed=2)
     with pytest.raises(AtError):
         _run(pb, u0, 1, "persistent")
+
+
+@pytest.mark.parametrize("order,rk,pe_size,pes", [
+    (2, "rk4", 32, 4864), (2, "rk4", 64, 4864), (2, "rk4", 128, 3648), (4, "rk4", 32, 4864), (4, "rk4", 64, 4096),
+    (4, "rk4", 64, 4864), (4, "rk4", 128, 3648), (6, "rk4", 32, 4864), (6, "rk4", 64, 3648), (6, "rk4", 128, 3648),
+    (2, "rk3tvd", 64, 4864), (2, "rk3tvd", 128, 3648), (2, "rk3tvd", 256, 3648), (4, "rk3tvd", 64, 4864),
+    (4, "rk3tvd", 128, 3648), (6, "rk3tvd", 64, 4864), (6, "rk3tvd", 128, 3648), (2, "rk2", 128, 4864),
+    (2, "rk2", 256, 3648), (4, "rk2", 64, 4864), (4, "rk2", 128, 3648), (6, "rk2", 64, 4864), (6, "rk2", 128, 2432),
+    (4, "rk4", 256, 1824), (6, "rk4", 256, 1824)])
+def test_advection_diffusion_in_one_launch(order, rk, pe_size, pes):
+    pb, u0 = W.advdiff(n=pe_size * pes, pe_size=pe_size, order=order, rk=rk, mode="at", k_max=3, seed=3, cfl=0.01)
+    a, b = _run(pb, u0, 7, "fused"), _run(pb, u0, 7, "stage")
+    assert a[2].kernels_launched == 2  # the counters' reset and the kernel
+    assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
