@@ -124,7 +124,7 @@ KERNEL_FILES = {
 }
 _SHA_STAGE = "6e784c929c16a6d751d35abe7a4d62e209453830427fb470dbc828ec5c52f3fa"
 _SHA_PERSISTENT = "7f3ab37ef47676a1fa3618d9e21771d44ee55d0c21031ac6fd964add8773a377"
-_SHA_FUSED = "1d948f2a1b3516ef1cd1dfa42559a3ee9d5883327c766ccb6963c99d2483556b"
+_SHA_FUSED = "308c373af45eb4e84007d4c4672744281a7d691a8dc441b68684e567ed24c37f"
 PROFILED_SHA256 = {
     ("detonation-n16777216", "stage"): _SHA_STAGE,
     ("detonation-n8388608", "stage"): _SHA_STAGE,

@@ -91,7 +91,8 @@ enum { AT_READ_STATE = 0, AT_READ_DELAYS = 1, AT_READ_RING = 2, AT_READ_STATS = 
  * CTA: all steps of the call in one cooperative launch whose CTAs wait only
  * for their neighbour CTAs' previous step when they fit on the GPU at once,
  * else one launch per step (advection-diffusion, PEs of 32, 64, 128 or 256
- * points and at least stages x halo points; the reacting flow in flux form,
+ * points, by AT_PATH_AUTO also of 96, 160, 192 or 224, and at least stages x
+ * halo points; the reacting flow in flux form,
  * one launch per step over tiles of up to 8 PEs with recomputed strips of
  * the outer neighbours, PEs of at least stages x halo points; the WENO PDEs
  * in the reconstruction form, one launch per step over the per-stage

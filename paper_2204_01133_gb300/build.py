@@ -19,7 +19,9 @@ OUT = os.path.join(HERE, "libat_gb300.so")
 PROBE = os.path.join(HERE, "libat_probe.so")
 BUILD = os.path.join(HERE, "_build")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-SOURCES = ["at_abi.cu", "at_stage.cu", "at_persist.cu", "at_cluster.cu", "at_fused.cu", "at_tilefused.cu"]
+# one object each; the step-fused kernels by halo width (the longest to compile)
+SOURCES = ["at_fused.cu:-DAT_FUSED_H=1", "at_fused.cu:-DAT_FUSED_H=2", "at_fused.cu:-DAT_FUSED_H=3", "at_fused.cu",
+           "at_stage.cu", "at_abi.cu", "at_persist.cu", "at_cluster.cu", "at_tilefused.cu"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--fmad=true", "-Xptxas", "-O3"]
 
 
@@ -46,9 +48,10 @@ def build(force: bool = False, verbose: bool = False, extra=()) -> str:
     os.makedirs(BUILD, exist_ok=True)
     cc = nvcc()
 
-    def compile_one(src):
-        obj = os.path.join(BUILD, src.replace(".cu", ".o"))
-        cmd = [cc, *ARCH, *FLAGS, *extra, "-c", os.path.join(CSRC, src), "-o", obj]
+    def compile_one(unit):
+        src, *defs = unit.split(":")
+        obj = os.path.join(BUILD, src.replace(".cu", "") + "".join(d[-1] for d in defs) + ".o")
+        cmd = [cc, *ARCH, *FLAGS, *extra, *defs, "-c", os.path.join(CSRC, src), "-o", obj]
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError("nvcc failed on %s:\n%s%s" % (src, r.stdout, r.stderr))

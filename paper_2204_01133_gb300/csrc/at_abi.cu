@@ -658,8 +658,10 @@ int at_step(at_ctx* c, int64_t nsteps)
         return fail(AT_EINVAL, "delays by arrival need the persistent path (a central PDE and at most %lld PEs)",
                     (long long)c->persist_cap);
     if (c->path == AT_PATH_FUSED || (c->path == AT_PATH_AUTO && !persist && !c->arrival && fused_ok)) {
-        // (PEs of 96 points take it by the automatic rule only)
-        if ((!fused_ok && !tile_ok) || (c->path == AT_PATH_FUSED && c->pb.pde == AT_ADVDIFF && c->pb.pe_size == 96))
+        // advection-diffusion on PEs whose size is no power of two takes it by the
+        // automatic rule only
+        const bool by_name = c->path == AT_PATH_FUSED;
+        if ((!fused_ok && !tile_ok) || (by_name && fused_ok && (c->pb.pe_size & (c->pb.pe_size - 1)) != 0))
             return fail(AT_EINVAL, "the fused path takes advection-diffusion with PEs of 32, 64, 128 or 256 points, "
                                    "the reacting flow in flux form or a WENO PDE in the reconstruction form, with at "
                                    "least stages x halo points per PE");

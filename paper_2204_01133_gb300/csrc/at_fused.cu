@@ -25,6 +25,9 @@
 // The step reads u^n from one buffer and writes u^{n+1} to another (a
 // neighbouring CTA may still read the edge points of u^n); the host
 // alternates the two.
+//
+// The file is compiled four times (build.py): the kernels of one halo width each
+// with AT_FUSED_H = 1, 2, 3, and the host side without it.
 #include <cuda/atomic>
 #include <cuda_runtime.h>
 
@@ -304,7 +307,7 @@ __device__ __forceinline__ void fused_store_release(int64_t* p, int64_t v)
 
 // bounded wait for *ctr >= target; false if it ran out (status bit 2, abort
 // flag raised) or another CTA's wait did
-__device__ bool fused_wait_ge(const StageArgs& a, int64_t* ctr, int64_t target)
+static __device__ bool fused_wait_ge(const StageArgs& a, int64_t* ctr, int64_t target)
 {
     if (fused_load_acquire(ctr) >= target) return true;
     for (int64_t it = 0; it < a.wait_limit; ++it) {
@@ -328,15 +331,19 @@ __device__ bool fused_wait_ge(const StageArgs& a, int64_t* ctr, int64_t target)
 // buffer that held u^{n-1}, which the neighbours read during their step n-1,
 // and the ring slots of levels n and n+1, which no CTA at step n or n+1 reads
 // (the CTAs are at most one step apart, the ring keeps k_max + q + 3 levels).
-// warps per PE of the multi-step kernel with W PEs a CTA
-__host__ __device__ constexpr int steps_wpp(int W, int ppl) { return W == 2 && ppl >= 2 ? (ppl == 3 ? 3 : 2) : 1; }
+// warps per PE of the multi-step kernel with W PEs a CTA: with 2 the fewest that
+// share its points evenly
+__host__ __device__ constexpr int steps_wpp(int W, int ppl)
+{
+    return W != 2 || ppl == 1 ? 1 : (ppl % 2 == 0 ? 2 : ppl);
+}
 
 // CTAs an SM that the full variant of W = 8 keeps registers for: those that fitted
 // before u^n stayed in registers from step to step (56 of them a thread for PEs
 // of 32 and 64 points, 72 for 96 and 128)
 __host__ __device__ constexpr int steps_min_ctas(int H, int ppl)
 {
-    return ppl <= 2 ? 4 : (ppl <= 4 ? (H == 1 ? 4 : 3) : (H == 1 ? 3 : 0));
+    return ppl <= 2 ? 4 : (ppl <= 4 ? (H == 1 ? 4 : 3) : (H == 1 ? 3 : (ppl < 8 ? 2 : 0)));
 }
 
 // CTAS: so many an SM at least (0: as the registers fall)
@@ -373,26 +380,17 @@ __global__ void __launch_bounds__(32 * (W * steps_wpp(W, PPL) + 1), CTAS)
     }
 }
 
-// done[c] = level0 for the CTAs of a launch, the abort flag and the placement count cleared
-__global__ void fused_counters_set(int64_t* done, int64_t C, int64_t level0, int* abort_flag, int* place_count)
-{
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < C; i += (int64_t)gridDim.x * blockDim.x)
-        done[i] = level0;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        *abort_flag = 0;
-        *place_count = 0;
-    }
-}
-
 } // namespace atk
 
-// ---------------------------------------------------------------------------
-// host side
-// ---------------------------------------------------------------------------
 namespace {
-
 constexpr int kFusedW = 8;  // PEs per CTA (measured on GB300: 8 ahead of 4 and 16)
 
+// the variants of the multi-step kernel, in the order in which they are preferred
+// (0: none): 2, 4 and 8 PEs a CTA, and 8 with registers for more CTAs an SM
+constexpr int kStepsVariants = 4;
+constexpr int steps_w(int variant) { return variant == 1 ? 2 : (variant == 2 ? 4 : 8); }
+
+#ifdef AT_FUSED_H
 template <int H, int RK>
 void* fused_fn_ppl(int ppl)
 {
@@ -401,7 +399,11 @@ void* fused_fn_ppl(int ppl)
     case 2: return (void*)atk::step_fused_advdiff<H, 2, RK, kFusedW>;
     case 3: return (void*)atk::step_fused_advdiff<H, 3, RK, kFusedW>;
     case 4: return (void*)atk::step_fused_advdiff<H, 4, RK, kFusedW>;
-    default: return (void*)atk::step_fused_advdiff<H, 8, RK, kFusedW>;
+    case 5: return (void*)atk::step_fused_advdiff<H, 5, RK, kFusedW>;
+    case 6: return (void*)atk::step_fused_advdiff<H, 6, RK, kFusedW>;
+    case 7: return (void*)atk::step_fused_advdiff<H, 7, RK, kFusedW>;
+    case 8: return (void*)atk::step_fused_advdiff<H, 8, RK, kFusedW>;
+    default: return nullptr;
     }
 }
 
@@ -412,18 +414,6 @@ void* fused_fn_rk(int rk, int ppl)
     if (rk == atk::RK3TVD) return fused_fn_ppl<H, atk::RK3TVD>(ppl);
     return fused_fn_ppl<H, atk::RK2>(ppl);
 }
-
-void* fused_fn(int H, int rk, int ppl)
-{
-    if (H == 1) return fused_fn_rk<1>(rk, ppl);
-    if (H == 2) return fused_fn_rk<2>(rk, ppl);
-    return fused_fn_rk<3>(rk, ppl);
-}
-
-// the variants of the multi-step kernel, in the order in which they are preferred
-// (0: none): 2, 4 and 8 PEs a CTA, and 8 with registers for more CTAs an SM
-constexpr int kStepsVariants = 4;
-constexpr int steps_w(int variant) { return variant == 1 ? 2 : (variant == 2 ? 4 : 8); }
 
 template <int H, int RK, int PPL>
 void* fused_steps_fn_v(int variant)
@@ -442,7 +432,11 @@ void* fused_steps_fn_ppl(int ppl, int variant)
     case 2: return fused_steps_fn_v<H, RK, 2>(variant);
     case 3: return fused_steps_fn_v<H, RK, 3>(variant);
     case 4: return fused_steps_fn_v<H, RK, 4>(variant);
-    default: return fused_steps_fn_v<H, RK, 8>(variant);
+    case 5: return fused_steps_fn_v<H, RK, 5>(variant);
+    case 6: return fused_steps_fn_v<H, RK, 6>(variant);
+    case 7: return fused_steps_fn_v<H, RK, 7>(variant);
+    case 8: return fused_steps_fn_v<H, RK, 8>(variant);
+    default: return nullptr;
     }
 }
 
@@ -454,11 +448,55 @@ void* fused_steps_fn_rk(int rk, int ppl, int variant)
     return fused_steps_fn_ppl<H, atk::RK2>(ppl, variant);
 }
 
+} // namespace
+
+#define AT_CAT2(a, b) a##b
+#define AT_CAT(a, b) AT_CAT2(a, b)
+// the kernels of this halo width for PEs of 32 ppl points: one step; many steps by variant
+void* AT_CAT(atk_fused_fn_, AT_FUSED_H)(int rk, int ppl) { return fused_fn_rk<AT_FUSED_H>(rk, ppl); }
+void* AT_CAT(atk_fused_steps_fn_, AT_FUSED_H)(int rk, int ppl, int variant)
+{
+    return fused_steps_fn_rk<AT_FUSED_H>(rk, ppl, variant);
+}
+
+#else
+} // namespace
+
+void* atk_fused_fn_1(int rk, int ppl);
+void* atk_fused_fn_2(int rk, int ppl);
+void* atk_fused_fn_3(int rk, int ppl);
+void* atk_fused_steps_fn_1(int rk, int ppl, int variant);
+void* atk_fused_steps_fn_2(int rk, int ppl, int variant);
+void* atk_fused_steps_fn_3(int rk, int ppl, int variant);
+
+namespace atk {
+// done[c] = level0 for the CTAs of a launch, the abort flag and the placement count cleared
+__global__ void fused_counters_set(int64_t* done, int64_t C, int64_t level0, int* abort_flag, int* place_count)
+{
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < C; i += (int64_t)gridDim.x * blockDim.x)
+        done[i] = level0;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        *abort_flag = 0;
+        *place_count = 0;
+    }
+}
+
+} // namespace atk
+
+// ---------------------------------------------------------------------------
+// host side
+// ---------------------------------------------------------------------------
+namespace {
+
+void* fused_fn(int H, int rk, int ppl)
+{
+    return H == 1 ? atk_fused_fn_1(rk, ppl) : (H == 2 ? atk_fused_fn_2(rk, ppl) : atk_fused_fn_3(rk, ppl));
+}
+
 void* fused_steps_fn(int H, int rk, int ppl, int variant)
 {
-    if (H == 1) return fused_steps_fn_rk<1>(rk, ppl, variant);
-    if (H == 2) return fused_steps_fn_rk<2>(rk, ppl, variant);
-    return fused_steps_fn_rk<3>(rk, ppl, variant);
+    return H == 1 ? atk_fused_steps_fn_1(rk, ppl, variant)
+                  : (H == 2 ? atk_fused_steps_fn_2(rk, ppl, variant) : atk_fused_steps_fn_3(rk, ppl, variant));
 }
 
 size_t fused_smem(int B, int H, int S, int W = kFusedW)
@@ -472,12 +510,12 @@ size_t fused_smem(int B, int H, int S, int W = kFusedW)
 } // namespace
 
 // whether the fused path takes this problem: advection-diffusion with
-// central stencils, PEs of 32, 64, 96, 128 or 256 points, at least S H points
-// (96: 9,696 points, AT6, RK3: 6.4 us per step against 10.8 with the kernel that
-// hands off every stage)
+// central stencils, PEs of a multiple of 32 points (a lane has the same number of
+// them in every warp) up to 256 (u^n and the accumulator of 8 points a lane in
+// registers), at least S H points
 bool atk_fused_supported(int pde, int order, int B, int S)
 {
-    return pde == atk::ADVDIFF && (B == 32 || B == 64 || B == 96 || B == 128 || B == 256) && B >= S * (order / 2);
+    return pde == atk::ADVDIFF && B % 32 == 0 && B <= 256 && B >= S * (order / 2);
 }
 
 int fused_steps_block(int B, int W) { return 32 * (W * atk::steps_wpp(W, B / 32) + 1); }
@@ -488,6 +526,7 @@ int64_t atk_fused_capacity(int order, int rk, int B, int S, int variant, int dev
 {
     const int H = order / 2, W = steps_w(variant);
     void* fn = fused_steps_fn(H, rk, B / 32, variant);
+    if (!fn) return 0;
     const size_t smem = fused_smem(B, H, S, W);
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
         cudaGetLastError();
@@ -529,6 +568,7 @@ cudaError_t atk_launch_fused_steps(const atk::StageArgs& a, int order, int varia
     const int H = order / 2, W = steps_w(variant);
     const int64_t C = (a.P + W - 1) / W;
     void* fn = fused_steps_fn(H, a.rk, a.B / 32, variant);
+    if (!fn) return cudaErrorInvalidValue;
     const size_t smem = fused_smem(a.B, H, a.S, W);
     atk::fused_counters_set<<<(unsigned)((C + 255) / 256 < 1024 ? (C + 255) / 256 : 1024), 256, 0, st>>>(
         a.done, C, level0, a.abort_flag, a.place_count);
@@ -547,6 +587,7 @@ cudaError_t atk_launch_fused(const atk::StageArgs& a, int order, int64_t n, cons
 {
     const int H = order / 2;
     void* fn = fused_fn(H, a.rk, a.B / 32);
+    if (!fn) return cudaErrorInvalidValue;
     const size_t smem = fused_smem(a.B, H, a.S);
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -555,3 +596,4 @@ cudaError_t atk_launch_fused(const atk::StageArgs& a, int order, int64_t n, cons
     void* params[] = {(void*)&args, (void*)&uin, (void*)&uout, (void*)&n};
     return cudaLaunchKernel(fn, dim3((unsigned)grid), dim3(32 * (kFusedW + 1)), params, smem, st);
 }
+#endif

@@ -78,3 +78,18 @@ def test_advection_diffusion_in_one_launch(order, rk, pe_size, pes):
     a, b = _run(pb, u0, 7, "fused"), _run(pb, u0, 7, "stage")
     assert a[2].kernels_launched == 2  # the counters' reset and the kernel
     assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
+
+
+@pytest.mark.parametrize("pe_size", [96, 160, 192, 224])
+@pytest.mark.parametrize("pes,order,rk", [(1, 4, "rk4"), (2, 6, "rk3tvd"), (3, 2, "rk2"), (101, 6, "rk4"), (305, 4, "rk4"),
+                                          (1216, 6, "rk2"), (2500, 4, "rk4"), (6001, 6, "rk3tvd")])
+def test_pes_of_any_multiple_of_32(pe_size, pes, order, rk):
+    """By the automatic rule, in one launch or one a step; asked for by name the
+    path takes the powers of two, as ever."""
+    from paper_2204_01133_gb300.api import AtError
+    pb, u0 = W.advdiff(n=pe_size * pes, pe_size=pe_size, order=order, rk=rk, mode="at", k_max=3, seed=3, cfl=0.01)
+    a, b = _run(pb, u0, 7, "auto"), _run(pb, u0, 7, "stage")
+    assert a[2].path == 3
+    assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
+    with pytest.raises(AtError):
+        _run(pb, u0, 1, "fused")
