@@ -861,9 +861,12 @@ int atk_stage_block(int pde, int Tw)
     int nv = (pde == atk::RNS || pde == atk::EULER) ? 4 : 1;
     // WENO: a thread per (edge, variable); where that is more than 256, 128 (more
     // CTAs an SM, whose phases overlap: 2^23 points, windows of 128: 7.06 ms per
-    // step with 128 threads, 7.77 with 256; windows of 256 with 256: 7.17)
+    // step with 128 threads, 7.77 with 256), and 256 for windows from 192 points on
+    // (PE sizes without a divisor from 16 to 128), of which few fit an SM (us per
+    // step with 128 and 256 threads: 3,000 windows of 139 points 413 and 433, of 199
+    // 566 and 565, 4,000 of 509 2,398 and 1,917, of 1,021 7,520 and 5,165)
     int want = (pde == atk::EULER || pde == atk::ADV_WENO || pde == atk::BURGERS) ? nv * (Tw + 1) : nv * Tw;
-    if (pde == atk::EULER && want > 256) want = 128;
+    if (pde == atk::EULER && want > 256) want = Tw < 192 ? 128 : 256;
     // reacting N-S: a thread per point, two windows a CTA of 128 threads (below);
     // its barriers then hold few warps (2^22 points, PEs of 64, ms per step: 1.90,
     // with 128 threads a window 2.00, with 256 threads 2.43, with 32 1.97)
