@@ -93,3 +93,15 @@ def test_pes_of_any_multiple_of_32(pe_size, pes, order, rk):
     assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
     with pytest.raises(AtError):
         _run(pb, u0, 1, "fused")
+
+
+@pytest.mark.parametrize("variant", [7, 8], ids=["advection", "burgers"])
+def test_batched_scalar_weno_solves_hold_the_ctas_a_batch_asks_for(variant):
+    import ctypes
+    from paper_2204_01133_gb300 import api
+    L = api.lib()
+    smem = L._Z20atk_stage_smem_bytesiii  # size_t atk_stage_smem_bytes(int pde, int Tw, int H)
+    smem.restype, smem.argtypes = ctypes.c_size_t, [ctypes.c_int] * 3
+    ctas = L._Z25atk_batch_max_ctas_per_smiim  # int atk_batch_max_ctas_per_sm(int variant, int block, size_t smem)
+    ctas.restype, ctas.argtypes = ctypes.c_int, [ctypes.c_int, ctypes.c_int, ctypes.c_size_t]
+    assert ctas(variant, 256, smem({7: 3, 8: 4}[variant], 64, 3)) >= 3

@@ -6,7 +6,8 @@ import pytest
 
 @pytest.fixture(scope="module")
 def block():
-    from paper_2204_01133_gb300 import api
+    from paper_2204_01133_gb300 import api, build
+    build.build()
     f = api.lib()._Z15atk_stage_blockii  # int atk_stage_block(int pde, int Tw)
     f.restype, f.argtypes = ctypes.c_int, [ctypes.c_int, ctypes.c_int]
     return f
