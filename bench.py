@@ -122,7 +122,7 @@ KERNEL_FILES = {
     "persistent": ("at_cluster.cu", "at_device.cuh", "at_fixed.cuh", "at_persist.cu"),
     "fused": ("at_device.cuh", "at_fixed.cuh", "at_fused.cu", "at_tilefused.cu"),
 }
-_SHA_STAGE = "8a3be86847be71e094de5858227e4a06a04017d96f026e8f228f54be12010597"
+_SHA_STAGE = "640fd0c7e36121918783c3e61999f8401dfe3c0052ef0b4a6c20813fdc3b8821"
 _SHA_PERSISTENT = "7f3ab37ef47676a1fa3618d9e21771d44ee55d0c21031ac6fd964add8773a377"
 _SHA_FUSED = "308c373af45eb4e84007d4c4672744281a7d691a8dc441b68684e567ed24c37f"
 PROFILED_SHA256 = {

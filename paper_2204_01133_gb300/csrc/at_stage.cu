@@ -879,6 +879,17 @@ int atk_stage_block(int pde, int Tw)
     return want < 32 ? 32 : want;
 }
 
+// The flame on few windows, at most four an SM: a thread per (point, variable), up
+// to 256, since nothing else fills the SM while a window's items wait for one
+// another (us per step with Tw, 2 Tw and 4 Tw threads, 200 PEs of 64 points: order 6
+// 38.9, 30.2, 27.3; order 4 38.3, 28.1, 25.1, where FP64 throughout took 33.0 with
+// 2 Tw; 512 PEs 44.5, 34.1, 33.0; 1,000, more than four an SM, 53.8 with Tw).
+int atk_flame_threads(int Tw, int64_t windows, int sms)
+{
+    const int b = atk_stage_block(atk::RNS, Tw);
+    return windows > 4 * (int64_t)sms ? b : (4 * b < 256 ? 4 * b : 256);
+}
+
 namespace {
 // One stage kernel, allowed to come up before its predecessor on the stream has
 // ended (stage_begin waits for that).
@@ -903,7 +914,7 @@ cudaError_t atk_launch_stage(const atk::StageArgs& a, int pde, int order, int sm
 {
     const int64_t windows = a.P * a.wpp;
     cudaError_t e = cudaErrorInvalidValue;
-    int b1 = atk_stage_block(pde, a.Tw);
+    int b1 = pde == atk::RNS ? atk_flame_threads(a.Tw, windows, sms) : atk_stage_block(pde, a.Tw);
     // the chain-rule form on few windows: a thread per fill item (own points and
     // buffer levels), so that the fill takes one pass
     const bool few = windows < 16 * (int64_t)sms;
