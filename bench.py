@@ -122,9 +122,9 @@ KERNEL_FILES = {
     "persistent": ("at_cluster.cu", "at_device.cuh", "at_fixed.cuh", "at_persist.cu"),
     "fused": ("at_device.cuh", "at_fixed.cuh", "at_fused.cu", "at_tilefused.cu"),
 }
-_SHA_STAGE = "640fd0c7e36121918783c3e61999f8401dfe3c0052ef0b4a6c20813fdc3b8821"
-_SHA_PERSISTENT = "7f3ab37ef47676a1fa3618d9e21771d44ee55d0c21031ac6fd964add8773a377"
-_SHA_FUSED = "308c373af45eb4e84007d4c4672744281a7d691a8dc441b68684e567ed24c37f"
+_SHA_STAGE = "51b4ce2a1772202faebc6d022f243953a4aecfc5335e7e6074fa6ee5c0a2ce00"
+_SHA_PERSISTENT = "8cbc082d1fa8163013566239a8193a4150ff8956d1cc605e8cc9b8412d0e233d"
+_SHA_FUSED = "634228a5b063efb4c93c7243978697675d9c373d3cf3696891bb43782dbef2cf"
 PROFILED_SHA256 = {
     ("detonation-n16777216", "stage"): _SHA_STAGE,
     ("detonation-n8388608", "stage"): _SHA_STAGE,

@@ -19,6 +19,7 @@
 
 #include "../../include/at.h"
 #include "at_device.cuh"
+#include "at_fit.h"
 
 size_t atk_stage_smem_bytes(int pde, int Tw, int H);
 int atk_stage_block(int pde, int Tw);
@@ -32,7 +33,7 @@ int atk_cluster_size(int pde, int order, int B, int64_t P, int R, int S, int dev
 cudaError_t atk_launch_cluster(const atk::StageArgs& a, int order, int csize, int64_t level0, int64_t nsteps,
                                cudaStream_t st);
 bool atk_fused_supported(int pde, int order, int B, int S);
-int atk_fused_multi(int order, int rk, int B, int S, int64_t P, int device);
+int atk_fused_multi(int order, int rk, int B, int S, int64_t P, int device, bool* failed);
 cudaError_t atk_launch_fused_steps(const atk::StageArgs& a, int order, int variant, int64_t level0, int64_t nsteps,
                                    double* b0, double* b1, cudaStream_t st);
 bool atk_tile_fused_supported(int pde, int order, int B, int rk, int q);
@@ -413,7 +414,7 @@ struct at_ctx {
     bool persist_auto = false;     // whether the automatic rule takes it
     int cluster_c = 0;             // CTAs of the one-cluster kernel for this problem (0: not used)
     int sms = 0;                   // SMs of the device
-    int64_t fit_key[8] = {-1};     // what the capacities below were asked for
+    atk::FitCache fit;             // what the capacities below were asked for
     int stage_tw = 0;              // window length of the per-stage kernels (stage_window)
     int fused_multi = 0;           // variant of the multi-step kernel that holds the fused path's CTAs at once (0: none)
     int64_t wait_limit = 4000000;  // polls of a bounded wait
@@ -573,16 +574,19 @@ int at_set_delays(at_ctx* c, const at_delays* dl)
     if (e != cudaSuccess) return cuda_fail(e, "reset launch");
     c->level = 0;
     c->hist_level = -1;  // reading A recomputes level 0 at the first at_step
-    // what fits on the device depends on these alone: asked again only when one
-    // of them changes (the occupancy queries take some tens of microseconds)
+    // what fits on the device depends on these alone
     const int64_t key[8] = {c->pb.pde, c->pb.order, c->pb.rk, c->pb.pe_size, c->pb.n, c->pb.weno, L.R, L.S};
-    if (std::memcmp(key, c->fit_key, sizeof key) != 0) {
-        if (c->sms == 0) cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device);
+    if (!c->fit.knows(key)) {
+        c->fit.ask(key);
+        if (c->sms == 0) {
+            e = cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device);
+            if (e != cudaSuccess) c->fit.take(atk::fit_error(e));
+        }
         c->stage_tw = stage_window(&c->pb, L, c->sms);
         c->persist_cap = 0;
         for (int v = 0; v < 3 && (v == 0 || L.P > c->persist_cap); ++v) {
             const int64_t cap = std::min(
-                atk_persist_capacity(c->pb.pde, c->pb.order, c->pb.pe_size, v, c->device), kPersistMaxPE);
+                c->fit.take(atk_persist_capacity(c->pb.pde, c->pb.order, c->pb.pe_size, v, c->device)), kPersistMaxPE);
             if (cap <= c->persist_cap) continue;
             c->persist_cap = cap;
             c->persist_variant = v;
@@ -593,13 +597,15 @@ int at_set_delays(at_ctx* c, const at_delays* dl)
         // of 480, dense, 81.7 and 73.9): the automatic rule leaves them there from
         // 750 points on and where only dense rows fit
         c->persist_auto = c->pb.pde == AT_ADVDIFF || (c->persist_variant < 2 && c->pb.pe_size < 750);
-        c->cluster_c = c->pb.pde == AT_ADVDIFF
-                           ? atk_cluster_size(c->pb.pde, c->pb.order, c->pb.pe_size, L.P, L.R, L.S, c->device)
-                           : 0;
+        c->cluster_c = (int)c->fit.take(
+            c->pb.pde == AT_ADVDIFF
+                ? atk_cluster_size(c->pb.pde, c->pb.order, c->pb.pe_size, L.P, L.R, L.S, c->device)
+                : 0);
+        bool failed = false;
         c->fused_multi = atk_fused_supported(c->pb.pde, c->pb.order, c->pb.pe_size, L.S)
-                             ? atk_fused_multi(c->pb.order, c->pb.rk, c->pb.pe_size, L.S, L.P, c->device)
+                             ? atk_fused_multi(c->pb.order, c->pb.rk, c->pb.pe_size, L.S, L.P, c->device, &failed)
                              : 0;
-        std::memcpy(c->fit_key, key, sizeof key);
+        if (failed) c->fit.take(-1);
     }
     cudaGetLastError();  // an unavailable persistent path is not an error
     c->have_delays = true;

@@ -287,8 +287,8 @@ cudaLaunchConfig_t cluster_config(int B, int csize, int m, size_t smem, cudaStre
 } // namespace
 
 // CTAs of the cluster (one per SM) for P PEs of B points of advection-
-// diffusion, or 0 when the cluster path does not apply: B of 32..256 points
-// (a multiple of 32), at most 4 PEs per CTA, at most 16 CTAs (sizes above 8
+// diffusion, or 0 when the cluster path does not apply (-1: a query failed): B of
+// 32, 64, 128 or 256 points, at most 4 PEs per CTA, at most 16 CTAs (sizes above 8
 // are non-portable; every size is checked with the occupancy query).
 int atk_cluster_size(int pde, int order, int B, int64_t P, int R, int S, int device)
 {
@@ -306,20 +306,15 @@ int atk_cluster_size(int pde, int order, int B, int64_t P, int R, int S, int dev
     const int m = (int)(P / C);
     void* fn = cluster_fn(H, B / 32, cluster_wpp(B, m), S);
     const size_t smem = cluster_smem(B, H, m, R, S);
-    if (cudaSetDevice(device) != cudaSuccess) return 0;
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
-        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
-        cudaGetLastError();
-        return 0;
-    }
+    cudaError_t e = cudaSetDevice(device);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     cudaLaunchAttribute attr[1];
     cudaLaunchConfig_t cfg = cluster_config(B, C, m, smem, 0, attr);
     int nclusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&nclusters, fn, &cfg) != cudaSuccess || nclusters < 1) {
-        cudaGetLastError();
-        return 0;
-    }
-    return C;
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&nclusters, fn, &cfg);
+    if (e != cudaSuccess) return (int)atk::fit_error(e);
+    return nclusters < 1 ? 0 : C;
 }
 
 cudaError_t atk_launch_cluster(const atk::StageArgs& a, int order, int csize, int64_t level0, int64_t nsteps,

@@ -81,6 +81,14 @@ struct StageArgs {
     double* state;
 };
 
+// The answer of a capacity query that ended with an error: 0, the kernel does not
+// fit, where the launch shape itself is refused; -1, unknown, otherwise.
+inline int64_t fit_error(cudaError_t e)
+{
+    cudaGetLastError();
+    return e == cudaErrorInvalidValue ? 0 : -1;
+}
+
 // what a solve's reset takes besides its StageArgs
 struct ResetArgs {
     int64_t ring_elems, ext_elems;

@@ -521,42 +521,44 @@ bool atk_fused_supported(int pde, int order, int B, int S)
 int fused_steps_block(int B, int W) { return 32 * (W * atk::steps_wpp(W, B / 32) + 1); }
 
 // CTAs that one cooperative launch of a variant of the multi-step kernel holds
-// at once (0: not available)
+// at once (0: not available, -1: the query failed)
 int64_t atk_fused_capacity(int order, int rk, int B, int S, int variant, int device)
 {
     const int H = order / 2, W = steps_w(variant);
     void* fn = fused_steps_fn(H, rk, B / 32, variant);
     if (!fn) return 0;
     const size_t smem = fused_smem(B, H, S, W);
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
-        cudaGetLastError();
-        return 0;
-    }
     int per_sm = 0, sms = 0, coop = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, fused_steps_block(B, W), smem) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
-        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, device) != cudaSuccess || !coop) {
-        cudaGetLastError();
-        return 0;
-    }
-    return (int64_t)per_sm * sms;
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, fused_steps_block(B, W), smem);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, device);
+    if (e != cudaSuccess) return atk::fit_error(e);
+    return coop ? (int64_t)per_sm * sms : 0;
 }
 
 // Variant of the multi-step kernel for P PEs, or 0 when none holds them in one
-// cooperative launch: 2 PEs a CTA, on two warps each, where that is one CTA an SM at
+// cooperative launch (*failed: a query on the way failed): 2 PEs a CTA, on two warps each, where that is one CTA an SM at
 // most; 4 where they fit (more SMs share the stages of a small problem); 8; 8 with
 // registers for more CTAs an SM (measured on GB300, PEs of 64 points, us per step:
 // 2^14 points 5.9 with 2, 7.4 with 4, 8.9 with 8; 3,000 PEs 16.4 with 8, 16.9 with
 // the registers of the last; 4,096 PEs 21.2 with those, 22.6 with one launch per
 // step)
-int atk_fused_multi(int order, int rk, int B, int S, int64_t P, int device)
+int atk_fused_multi(int order, int rk, int B, int S, int64_t P, int device, bool* failed)
 {
     int sms = 0;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) return 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) {
+        cudaGetLastError();
+        *failed = true;
+        return 0;
+    }
     for (int v = 1; v <= kStepsVariants; ++v) {
         const int64_t ctas = (P + steps_w(v) - 1) / steps_w(v);
         if (v == 1 && ctas > sms) continue;
-        if (ctas <= atk_fused_capacity(order, rk, B, S, v, device)) return v;
+        const int64_t cap = atk_fused_capacity(order, rk, B, S, v, device);
+        if (cap < 0) *failed = true;
+        if (ctas <= cap) return v;
     }
     return 0;
 }

@@ -525,7 +525,7 @@ int atk_persist_block(int pde, int B)
     return want + 32;
 }
 
-// how many PEs one cooperative launch of a variant can hold (0: not available)
+// how many PEs one cooperative launch of a variant can hold (0: not available, -1: the query failed)
 int64_t atk_persist_capacity(int pde, int order, int B, int variant, int device)
 {
     void* fn = variant < kVariants ? persist_kernel(pde, order, variant) : nullptr;
@@ -533,13 +533,14 @@ int64_t atk_persist_capacity(int pde, int order, int B, int variant, int device)
     if (!fn || !persist_takes(pde, B, H)) return 0;
     const size_t smem = persist_smem_bytes(pde, B, H, variant);
     if (smem > 226 * 1024) return 0;
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
     int per_sm = 0, sms = 0, coop = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, atk_persist_block(pde, B), smem) != cudaSuccess)
-        return 0;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) return 0;
-    if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, device) != cudaSuccess || !coop) return 0;
-    return (int64_t)per_sm * sms;
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, atk_persist_block(pde, B), smem);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, device);
+    if (e != cudaSuccess) return atk::fit_error(e);
+    return coop ? (int64_t)per_sm * sms : 0;
 }
 
 cudaError_t atk_launch_persist(const atk::StageArgs& a, int pde, int order, int variant, int64_t level0, int64_t nsteps,
