@@ -39,3 +39,33 @@ def test_weno_front_beside_a_uniform_state(amp, eps):
         out.append(s.read_state())
         s.close()
     assert np.array_equal(*out)
+
+
+@pytest.mark.parametrize("which", [5, 6], ids=["reciprocal", "root"])
+def test_reciprocal_and_root_outside_the_normal_range(which):
+    """Each by itself: no wrong finite value, and the signs of zeros and of
+    infinities as in IEEE arithmetic where a value is defined (the probe test of
+    the normal range checks only part of them)."""
+    import ctypes
+    import os
+    import torch
+    from paper_2204_01133_gb300 import build
+    L = ctypes.CDLL(os.path.join(os.path.dirname(build.__file__), "libat_probe.so"))
+    L.at_probe_fn.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int64, ctypes.c_int]
+    x = np.array([0.0, np.inf, np.nan, -1.0, 1e-310, 5e-324, 2.0 ** -1022, 1.7e308, 2.0 ** 1022])
+    xd = torch.from_numpy(x).cuda()
+    yd = torch.empty_like(xd)
+    assert L.at_probe_fn(xd.data_ptr(), yd.data_ptr(), xd.numel(), which) == 0
+    zero, inf, nan, neg, sub, least, normal, most, big = yd.cpu().numpy().tolist()
+    assert np.isnan(nan)
+    if which == 5:
+        assert not np.isfinite(zero)
+        assert inf == 0.0 or np.isnan(inf)
+        assert neg == -1.0
+        assert not np.isfinite(sub) and not np.isfinite(least)  # above the largest number
+        assert normal == 2.0 ** 1022 and big == 2.0 ** -1022
+        assert abs(most - 1 / 1.7e308) <= 2.0 ** -1022 * 2.0 ** -50 or most == 0.0 or np.isnan(most)
+    else:
+        assert zero == 0.0 and inf == np.inf and np.isnan(neg)
+        assert sub == np.sqrt(1e-310) and least == np.sqrt(5e-324) and normal == 2.0 ** -511
+        assert abs(most - np.sqrt(1.7e308)) <= np.spacing(most) and big == 2.0 ** 511
