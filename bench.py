@@ -123,7 +123,7 @@ KERNEL_FILES = {
     "fused": ("at_device.cuh", "at_fixed.cuh", "at_fused.cu", "at_tilefused.cu"),
 }
 _SHA_STAGE = "51b4ce2a1772202faebc6d022f243953a4aecfc5335e7e6074fa6ee5c0a2ce00"
-_SHA_PERSISTENT = "8cbc082d1fa8163013566239a8193a4150ff8956d1cc605e8cc9b8412d0e233d"
+_SHA_PERSISTENT = "80b64dc32c286c96c2c99834a8633f64098fe8a5b9accc82f5af63a83d610858"
 _SHA_FUSED = "634228a5b063efb4c93c7243978697675d9c373d3cf3696891bb43782dbef2cf"
 PROFILED_SHA256 = {
     ("detonation-n16777216", "stage"): _SHA_STAGE,
