@@ -122,9 +122,9 @@ KERNEL_FILES = {
     "persistent": ("at_cluster.cu", "at_device.cuh", "at_fixed.cuh", "at_persist.cu"),
     "fused": ("at_device.cuh", "at_fixed.cuh", "at_fused.cu", "at_tilefused.cu"),
 }
-_SHA_STAGE = "51b4ce2a1772202faebc6d022f243953a4aecfc5335e7e6074fa6ee5c0a2ce00"
-_SHA_PERSISTENT = "80b64dc32c286c96c2c99834a8633f64098fe8a5b9accc82f5af63a83d610858"
-_SHA_FUSED = "634228a5b063efb4c93c7243978697675d9c373d3cf3696891bb43782dbef2cf"
+_SHA_STAGE = "3ddceba4ffdd56910ac24509f7bc19514ea1b15d1ff7ac38da55b4eb0cffd3e4"
+_SHA_PERSISTENT = "dfd7937f4f4ae3eab48a26547235a678ecbdc6bbd825a223192ab6d8ba9563a1"
+_SHA_FUSED = "a6a64ff1f16634e1e06eecad0e6929e43e82f594a7354244e024165d44d8d458"
 PROFILED_SHA256 = {
     ("detonation-n16777216", "stage"): _SHA_STAGE,
     ("detonation-n8388608", "stage"): _SHA_STAGE,

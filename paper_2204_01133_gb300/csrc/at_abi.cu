@@ -584,19 +584,18 @@ int at_set_delays(at_ctx* c, const at_delays* dl)
         }
         c->stage_tw = stage_window(&c->pb, L, c->sms);
         c->persist_cap = 0;
-        for (int v = 0; v < 3 && (v == 0 || L.P > c->persist_cap); ++v) {
+        for (int v = 0; v < 4 && (c->persist_cap == 0 || L.P > c->persist_cap); ++v) {
             const int64_t cap = std::min(
                 c->fit.take(atk_persist_capacity(c->pb.pde, c->pb.order, c->pb.pe_size, v, c->device)), kPersistMaxPE);
             if (cap <= c->persist_cap) continue;
             c->persist_cap = cap;
             c->persist_variant = v;
         }
-        // large PEs of the reacting flow are no faster resident than with one
-        // launch per stage (us per step, resident and per stage: 152 PEs of 600
-        // points 56.3 and 55.5, of 749 68.8 and 64.2, 150 of 800 73.5 and 66.0, 304
-        // of 480, dense, 81.7 and 73.9): the automatic rule leaves them there from
-        // 750 points on and where only dense rows fit
-        c->persist_auto = c->pb.pde == AT_ADVDIFF || (c->persist_variant < 2 && c->pb.pe_size < 750);
+        // large PEs of the reacting flow that fit as dense rows only are faster with
+        // one launch per stage (us per step, resident and per stage: 304 PEs of 480
+        // points 81.3 and 73.8, 100 of 870 104.5 and 57.3; with split rows 152 of 760
+        // 55.6 and 66.5, 456 of 64 23.5 and 30.3): the automatic rule leaves them there
+        c->persist_auto = c->pb.pde == AT_ADVDIFF || c->persist_variant < 3;
         c->cluster_c = (int)c->fit.take(
             c->pb.pde == AT_ADVDIFF
                 ? atk_cluster_size(c->pb.pde, c->pb.order, c->pb.pe_size, L.P, L.R, L.S, c->device)
@@ -656,7 +655,7 @@ int at_step(at_ctx* c, int64_t nsteps)
                    (c->path == AT_PATH_AUTO && can_persist && (c->persist_auto || c->arrival || c->withhold_pe >= 0));
     // advection-diffusion beyond one thread-block cluster: the step-fused
     // kernel is faster than the neighbour-wait kernel (measured on GB300 at
-    // 256 PEs of 64 points: 10.3 against 13.1 us per step); delays by arrival
+    // 256 PEs of 64 points: 5.6 against 12.0 us per step); delays by arrival
     // and withheld progress need the neighbour waits
     if (c->path == AT_PATH_AUTO && persist && !cluster_ok && fused_ok && !c->arrival && c->withhold_pe < 0)
         persist = false;

@@ -502,8 +502,8 @@ AT_HD uint64_t fx_fixed(FxU a, int e)
 // not normalised: E_i keeps 60 bits or more, a product of two 55, a weight 53.
 // About 1,600 issue cycles of integer work for an edge and variable stand beside
 // seven FP64 instructions (448 cycles), in place of 66 of those (4,224).  Measured
-// on GB300: the detonation of 2^23 points 10.77 -> 7.19 ms per RK3 step (16.3 with
-// all of it in FP64), of 61,440 points 123 -> 105 us (168).  eps3 = 3 eps.  Not a
+// on GB300: the detonation of 2^23 points 10.77 -> 6.83 ms per RK3 step (16.3 with
+// all of it in FP64), of 61,440 points 123 -> 91 us (168).  eps3 = 3 eps.  Not a
 // number where a difference or eps is not (or is infinite), or where a
 // denominator vanishes (eps = 0 and two indicators that are zero).
 AT_HD double fx_weno_sum(const double* c, const double* q, FxU eps3)

@@ -164,12 +164,13 @@ __device__ __forceinline__ void bar_arrive_p(int p, int count)
 // How many PEs fit the chip is registers and shared memory.  CTAS = 2 of 288
 // threads an SM leaves the registers the code wants (85 at order 6); CTAS = 3 holds
 // it to 72 for more PEs (none spilt, 3 to 6 % slower where both fit: 304 PEs of
-// 64 points 19.1 and 20.8 us per step; 456 of them 24.7, one launch per stage
-// 40.3).  DENSE has the reacting flow's rows as doubles, split where they are
-// read, in 27 words a point instead of 34, for large PEs that no other holds (100
-// of 400 points 52.9 us against 39.9).
+// 64 points 18.7 and 20.0 us per step; 456 of them 23.5, one launch per stage
+// 30.3).  CTAS = 1 has sixteen worker warps instead of eight, for some PE sizes where
+// every PE has an SM to itself (persist_wide).  DENSE has the reacting flow's rows
+// as doubles, split where they are read, in 27 words a point instead of 34, for
+// large PEs that no other holds (100 of 400 points 52.9 us against 39.9).
 template <int PDE, int H, int CTAS, bool DENSE>
-__global__ void __launch_bounds__(288, CTAS) persist_central(const StageArgs a, int64_t level0, int64_t nsteps)
+__global__ void __launch_bounds__(CTAS == 1 ? 544 : 288, CTAS) persist_central(const StageArgs a, int64_t level0, int64_t nsteps)
 {
     using P = Phys<PDE>;
     constexpr int NV = P::NV, ND = P::ND;
@@ -282,8 +283,12 @@ __global__ void __launch_bounds__(288, CTAS) persist_central(const StageArgs a, 
             if (lane < 2 && a.arrival) {
                 const int kc = kcap_at(a, n);
                 const int64_t need = (n - kc) * S + s;
-                ok = wait_ge(a, a.done + nbr[lane], need > free_at ? need : free_at);
+                const int64_t target = need > free_at ? need : free_at;
                 seen = load_acquire(a.done + nbr[lane]);
+                if (seen < target) {
+                    ok = wait_ge(a, a.done + nbr[lane], target);
+                    seen = load_acquire(a.done + nbr[lane]);
+                }
                 const int64_t m = (seen - s) / S;
                 k = m >= n ? 0 : (int)(n - m);
                 if (k > kc) k = kc;  // only if the wait gave up
@@ -480,15 +485,16 @@ __global__ void counters_set(int64_t* done, int64_t P, int64_t value, int* abort
 // ---------------------------------------------------------------------------
 namespace {
 // the variants of the kernel, in the order in which they are preferred
-constexpr int kVariants = 3;
+constexpr int kVariants = 4;
 
 template <int H>
 void* persist_fn(int pde, int variant)
 {
-    if (pde == atk::ADVDIFF) return variant == 0 ? (void*)atk::persist_central<atk::ADVDIFF, H, 2, false> : nullptr;
+    if (pde == atk::ADVDIFF) return variant == 1 ? (void*)atk::persist_central<atk::ADVDIFF, H, 2, false> : nullptr;
     if (pde != atk::RNS) return nullptr;
-    return variant == 0   ? (void*)atk::persist_central<atk::RNS, H, 2, false>
-           : variant == 1 ? (void*)atk::persist_central<atk::RNS, H, 3, false>
+    return variant == 0   ? (void*)atk::persist_central<atk::RNS, H, 1, false>
+           : variant == 1 ? (void*)atk::persist_central<atk::RNS, H, 2, false>
+           : variant == 2 ? (void*)atk::persist_central<atk::RNS, H, 3, false>
                           : (void*)atk::persist_central<atk::RNS, H, 3, true>;
 }
 
@@ -500,7 +506,7 @@ void* persist_kernel(int pde, int order, int variant)
 size_t persist_smem_bytes(int pde, int B, int H, int variant)
 {
     const int W2 = B + 2 * H, nv = pde == atk::RNS ? 4 : 1, rows = pde == atk::RNS ? atk::Phys<atk::RNS>::SPLIT : 1;
-    const size_t words = pde == atk::RNS && variant < 2 ? atk::split_words(rows, W2) : rows * W2;
+    const size_t words = pde == atk::RNS && variant < 3 ? atk::split_words(rows, W2) : rows * W2;
     return sizeof(double) * ((size_t)3 * nv * B + 2 * words + (size_t)B);
 }
 
@@ -513,33 +519,42 @@ bool persist_takes(int pde, int B, int H)
     return sizeof(double) * ((size_t)3 * nv * B + (size_t)2 * nd * (B + 2 * H) + (size_t)2 * H * (AT_QMAX + 1) * nd +
                              (size_t)B) <= 200 * 1024;
 }
-} // namespace
+// Whether the variant with sixteen worker warps is the faster one for PEs of B
+// points, each with an SM to itself: from 65 to 96 points eight warps have a second,
+// mostly empty round of (point, variable) items, and from 224 on half as many rounds
+// are left; between, waiting for twice the warps costs more than it saves.  us per
+// step with eight and sixteen, order 6: 72 points 17.8 and 16.3, 96 18.2 and 16.3,
+// 150 21.9 and 22.4, 192 25.2 and 26.1, 256 37.8 and 27.9 (FP64 throughout 36.3), 600
+// 59.5 and 50.8; order 4: 96 16.7 and 15.6, 150 19.4 and 21.0, 224 24.0 and 24.1, 256
+// 32.8 and 26.0 (FP64 31.4)
+bool persist_wide(int pde, int B) { return pde == atk::RNS && ((B > 64 && B <= 96) || B >= 224); }
 
 // worker warps for the PE's points (at least two roles' worth for phase A)
 // plus one halo warp
-int atk_persist_block(int pde, int B)
+int persist_block(int pde, int B, int variant)
 {
-    const int nv = pde == atk::RNS ? 4 : 1;
+    const int nv = pde == atk::RNS ? 4 : 1, most = variant == 0 ? 512 : 256;
     const int bw = (B + 31) / 32;
     int want = ((nv * B + 31) / 32) * 32;
-    if (want > 256) want = 256;
+    if (want > most) want = most;
     if (want < 64 * bw) want = 64 * bw;
-    if (want > 256) want = 256;
+    if (want > most) want = most;
     return want + 32;
 }
+} // namespace
 
 // how many PEs one cooperative launch of a variant can hold (0: not available, -1: the query failed)
 int64_t atk_persist_capacity(int pde, int order, int B, int variant, int device)
 {
     void* fn = variant < kVariants ? persist_kernel(pde, order, variant) : nullptr;
     const int H = order / 2;
-    if (!fn || !persist_takes(pde, B, H)) return 0;
+    if (!fn || !persist_takes(pde, B, H) || (variant == 0 && !persist_wide(pde, B))) return 0;
     const size_t smem = persist_smem_bytes(pde, B, H, variant);
-    if (smem > 226 * 1024) return 0;
+    if (smem > 227 * 1024 - 64) return 0;  // (64 for the kernel's own shared variables)
     int per_sm = 0, sms = 0, coop = 0;
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, atk_persist_block(pde, B), smem);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, persist_block(pde, B, variant), smem);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, device);
     if (e != cudaSuccess) return atk::fit_error(e);
@@ -561,5 +576,5 @@ cudaError_t atk_launch_persist(const atk::StageArgs& a, int pde, int order, int 
     if (e != cudaSuccess) return e;
     atk::StageArgs args = a;
     void* params[] = {(void*)&args, (void*)&level0, (void*)&nsteps};
-    return cudaLaunchCooperativeKernel(fn, dim3((unsigned)a.P), dim3(atk_persist_block(pde, a.B)), params, smem, st);
+    return cudaLaunchCooperativeKernel(fn, dim3((unsigned)a.P), dim3(persist_block(pde, a.B, variant)), params, smem, st);
 }

@@ -863,8 +863,8 @@ int atk_stage_block(int pde, int Tw)
 {
     int nv = (pde == atk::RNS || pde == atk::EULER) ? 4 : 1;
     // WENO: a thread per (edge, variable); where that is more than 256, 128 (more
-    // CTAs an SM, whose phases overlap: 2^23 points, windows of 128: 7.06 ms per
-    // step with 128 threads, 7.77 with 256), and 256 for windows from 192 points on
+    // CTAs an SM, whose phases overlap: 2^23 points, windows of 128: 6.83 ms per
+    // step with 128 threads, 10 % more with 256), and 256 for windows from 192 points on
     // (PE sizes without a divisor from 16 to 128), of which few fit an SM (us per
     // step with 128 and 256 threads: 3,000 windows of 139 points 413 and 433, of 199
     // 566 and 565, 4,000 of 509 2,398 and 1,917, of 1,021 7,520 and 5,165)
@@ -973,8 +973,10 @@ cudaError_t atk_launch_stage(const atk::StageArgs& a, int pde, int order, int sm
 #undef AT_WARP_LAUNCH
         return e;
     }
-    // the benchmarked combinations (6th-order reacting N-S with RK4, reactive
-    // Euler with RK3-TVD) get one kernel per RK stage kind
+    // one kernel per RK stage kind for the scheme each PDE is run with in earnest:
+    // the sixth-order reacting flow with RK4, the detonation with RK3-TVD; the others
+    // read the scheme at run time and pay the issue slots of the FP64 instructions
+    // predicated off (a kernel a kind, order and scheme would be 60 more to build)
     const int kind = atk::rk_stage_kind(a.rk, a.stage);
     constexpr int ANY = atk::RKS_ANY;
     switch (pde) {
@@ -1090,8 +1092,8 @@ cudaError_t atk_launch_batch(int variant, const atk::StageArgs* tab, int64_t* lv
     return cudaLaunchKernel(fn, dim3(grid), dim3(block), params, smem, st);
 }
 
-// rk: the RK scheme of every slot of the launch, or -1 where they differ; the
-// configured combinations get one kernel per stage kind, as on the per-stage path
+// rk: the RK scheme of every slot of the launch, or -1 where they differ; a kernel
+// per stage kind for the pairs of PDE and scheme that have one on the per-stage path
 static void* batch_stage_fn(int variant, int rk, int stage)
 {
     const int kind = rk < 0 ? atk::RKS_ANY : atk::rk_stage_kind(rk, stage);

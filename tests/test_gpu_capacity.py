@@ -31,7 +31,8 @@ def _run(pb, u0, steps, path):
 
 @pytest.mark.parametrize("order", [2, 4, 6])
 @pytest.mark.parametrize("pe_size,pes", [(16, 1368), (24, 1064), (32, 760), (48, 608), (64, 304), (64, 305), (64, 456),
-                                         (280, 456), (320, 456), (421, 304), (488, 304), (749, 152), (750, 152),
+                                         (65, 152), (96, 152), (96, 153), (97, 152), (223, 100), (224, 152),
+                                         (224, 153), (256, 1), (280, 456), (320, 456), (421, 304), (488, 304), (749, 152), (750, 152),
                                          (850, 152), (872, 152)])
 def test_flames_on_the_persistent_path(order, pe_size, pes):
     pb, u0 = W.rns(case="flame", n=pe_size * pes, pe_size=pe_size, order=order, mode="at", k_max=3, seed=2)
@@ -52,7 +53,7 @@ def test_delays_by_arrival(pe_size, pes):
     s.close()
 
 
-@pytest.mark.parametrize("pe_size,pes", [(32, 760), (64, 384), (64, 456), (200, 456)])
+@pytest.mark.parametrize("pe_size,pes", [(32, 760), (64, 384), (64, 456), (200, 456), (800, 100)])
 def test_the_automatic_rule_keeps_them_resident(pe_size, pes):
     pb, u0 = W.rns(case="flame", n=pe_size * pes, pe_size=pe_size, mode="at", k_max=3, seed=2)
     assert _run(pb, u0, 2, "auto")[2].path == 2
