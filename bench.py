@@ -122,9 +122,9 @@ KERNEL_FILES = {
     "persistent": ("at_cluster.cu", "at_device.cuh", "at_fixed.cuh", "at_persist.cu"),
     "fused": ("at_device.cuh", "at_fixed.cuh", "at_fused.cu", "at_tilefused.cu"),
 }
-_SHA_STAGE = "3ddceba4ffdd56910ac24509f7bc19514ea1b15d1ff7ac38da55b4eb0cffd3e4"
-_SHA_PERSISTENT = "dfd7937f4f4ae3eab48a26547235a678ecbdc6bbd825a223192ab6d8ba9563a1"
-_SHA_FUSED = "a6a64ff1f16634e1e06eecad0e6929e43e82f594a7354244e024165d44d8d458"
+_SHA_STAGE = "fa2d7fae87f415af36fe13968e6d947e7b4dd29239846e19caf7f96f605f5ed8"
+_SHA_PERSISTENT = "3c598fce9c1be11e79bbff566fb976e6834c3e700e2fc899e11968470dbff4e6"
+_SHA_FUSED = "7322801f4b0e8288a0c207cd736b97af3e6cd9fcded4c3f73bc281215fe26189"
 PROFILED_SHA256 = {
     ("detonation-n16777216", "stage"): _SHA_STAGE,
     ("detonation-n8388608", "stage"): _SHA_STAGE,

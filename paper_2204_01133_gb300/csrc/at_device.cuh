@@ -47,13 +47,18 @@ struct StageArgs {
     double s2;                                // 1 / (D2 dx^2): scales fx_d2
     double cm[2 * AT_HMAX + 1];               // merged advection-diffusion taps
     double prm[16];                           // physics constants (see at.h)
-    double k0, k1, k2, k3;                    // derived physics constants (WENO: k0 = 1/dx)
+    double k0;                                // derived physics constants (WENO: k0 = 1/dx, 3 eps)
+    union {
+        struct {
+            double k1, k2, k3;
+        };
+        FxU eps3;
+    };
     // reacting flow: the diffusion rows are u, the energy term over lambda and
     // Y, with the constants in the scale: s2v[v-1] = s2 times (4/3) mu,
     // lambda, lambda / (cp Le) for v = 1, 2, 3; kd1 = k1 / k2, kd3 = qc k3 / k2
     double s2v[3];
     double kd1, kd3;
-    FxU eps3;                                 // WENO: 3 eps
     // persistent path only
     int64_t* done;       // per PE: stages completed, as the index n*S + s + 1 [P]
     double* gring;       // derived quantities of the edge windows [R][S][P][2][H][ND]
