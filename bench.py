@@ -67,13 +67,13 @@ NOMINAL_FP64_TFLOPS = 1.25  # GB300 FP64 (vector and tensor), nominal, at 2070 M
 # achieved / peak is the share of the FP64 roof that the FP64 part alone uses.
 FLOPS_PER_POINT_STAGE = {
     ("rns", "stage"): 64.0,          # central6 + AT6, 4 variables (all in FP64: 165.7)
-    ("rns", "persistent"): 69.2,     # same work, all K steps of one launch
+    ("rns", "persistent"): 68.5,     # same work, all K steps of one launch
     ("detonation", "stage"): 111.6,  # WENO5 + AT-WENO5, 8 reconstructions per edge (all in FP64: 500.3)
     ("advdiff", "stage"): 13.56,     # 5-tap merged stencil + RK4 update, mean of the 4 stages
     ("advdiff", "persistent"): 13.56,
     ("advdiff", "fused"): 13.56,     # the method's work only
     ("rns", "fused"): 64.0,          # the per-stage kernel's count (the tile-fused kernel executes 67.3 with the strips)
-    ("detonation", "fused"): 111.6,  # likewise (144.7 with the strips)
+    ("detonation", "fused"): 111.6,  # likewise (146.2 with the strips)
 }
 # The method's own FP64 work per point per stage, by operation count (a
 # divide, square root or exponential counts as one operation): the
@@ -94,21 +94,21 @@ BYTES_PER_POINT_STAGE_FUSED = {"advdiff": 2 * 8 / 4, "rns": 2 * 4 * 8 / 4, "deto
 # current kernels, by workload and path; the reacting flow and the detonation
 # were captured at N = 2^22, advection-diffusion at 2^25, and are scaled.
 TRAFFIC_PER_LAUNCH = {
-    ("rns-flame-n16384", "persistent"): 2.9916e+06,  # state and rings read once, writes stay in L2
-    ("rns-flame-n16777216", "stage"): 4 * 5.5312e+08,
-    ("rns-flame-n8388608", "stage"): 2 * 5.5312e+08,
-    ("detonation-n8388608", "stage"): 2 * 3.2141e+08,
-    ("detonation-n16777216", "stage"): 4 * 3.2141e+08,
-    ("advdiff-n134217728", "stage"): 4 * 1.1303e+09,
-    ("advdiff-n33554432", "stage"): 1.1303e+09,
-    ("advdiff-n134217728", "fused"): 4 * 5.5701e+08,  # one step: u^n, u^{n+1}, the ring
-    ("advdiff-n33554432", "fused"): 5.5701e+08,
-    ("advdiff-n2048", "persistent"): 7.5776e+04,  # one-cluster launch: state and ring read once
-    ("advdiff-n16384", "fused"): 2.4346e+05,  # cooperative fused launch: state and ring read once
-    ("rns-flame-n16777216", "fused"): 4 * 2.6627e+08,  # tile-fused step
-    ("rns-flame-n8388608", "fused"): 2 * 2.6627e+08,
-    ("detonation-n16777216", "fused"): 4 * 2.2820e+08,  # tile-fused step
-    ("detonation-n8388608", "fused"): 2 * 2.2820e+08,
+    ("rns-flame-n16384", "persistent"): 3.0062e+06,  # state and rings read once, writes stay in L2
+    ("rns-flame-n16777216", "stage"): 4 * 5.5318e+08,
+    ("rns-flame-n8388608", "stage"): 2 * 5.5318e+08,
+    ("detonation-n8388608", "stage"): 2 * 3.2157e+08,
+    ("detonation-n16777216", "stage"): 4 * 3.2157e+08,
+    ("advdiff-n134217728", "stage"): 4 * 1.1301e+09,
+    ("advdiff-n33554432", "stage"): 1.1301e+09,
+    ("advdiff-n134217728", "fused"): 4 * 5.5704e+08,  # one step: u^n, u^{n+1}, the ring
+    ("advdiff-n33554432", "fused"): 5.5704e+08,
+    ("advdiff-n2048", "persistent"): 1.3722e+05,  # one-cluster launch: state and ring read once
+    ("advdiff-n16384", "fused"): 2.5907e+05,  # cooperative fused launch: state and ring read once
+    ("rns-flame-n16777216", "fused"): 4 * 2.6617e+08,  # tile-fused step
+    ("rns-flame-n8388608", "fused"): 2 * 2.6617e+08,
+    ("detonation-n16777216", "fused"): 4 * 2.2932e+08,  # tile-fused step
+    ("detonation-n8388608", "fused"): 2 * 2.2932e+08,
 }
 
 
