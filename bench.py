@@ -122,9 +122,9 @@ KERNEL_FILES = {
     "persistent": ("at_cluster.cu", "at_device.cuh", "at_fixed.cuh", "at_persist.cu"),
     "fused": ("at_device.cuh", "at_fixed.cuh", "at_fused.cu", "at_tilefused.cu"),
 }
-_SHA_STAGE = "fa2d7fae87f415af36fe13968e6d947e7b4dd29239846e19caf7f96f605f5ed8"
-_SHA_PERSISTENT = "3c598fce9c1be11e79bbff566fb976e6834c3e700e2fc899e11968470dbff4e6"
-_SHA_FUSED = "7322801f4b0e8288a0c207cd736b97af3e6cd9fcded4c3f73bc281215fe26189"
+_SHA_STAGE = "42c9217c669c84c42fb523461f2597be634afa8e89e9ef97213dda06c24e8eee"
+_SHA_PERSISTENT = "de61aa93f92627dc0d8bf1b4b0b8274051d4351e87d40b7de299ee8ab280ef0a"
+_SHA_FUSED = "be6cccd5d2c9deb59f10f9712529a23610fc9e69117f9dcea6539c56be65c50f"
 PROFILED_SHA256 = {
     ("detonation-n16777216", "stage"): _SHA_STAGE,
     ("detonation-n8388608", "stage"): _SHA_STAGE,

@@ -131,7 +131,8 @@ constexpr int FX_GUARD = 3;  // bits kept below the last bit of the largest valu
 // A double as a signed integer in units of 2^-FX_GUARD of its last place and its
 // exponent field (in place, bits 20..30 of the high word).  A zero or subnormal
 // has no implicit bit and the field of the smallest normal numbers, whose unit
-// is its own.  Inf and NaN keep their bits, marked by the field.
+// is its own.  Inf and NaN are their bits with an implicit one, marked by the field;
+// fx_join gives them back like any other number.
 struct FxV {
     int64_t m;
     uint32_t e;
@@ -143,7 +144,7 @@ AT_HD FxV fx_split(double x)
     const uint32_t hi = fx_hi(x), t = hi & FX_EXP;
     const uint64_t m = ((uint64_t)((hi & 0xfffffu) | fx_min(t, 0x100000u)) << 32 | fx_lo(x)) << GUARD;
     const int64_t s = (int32_t)hi >> 31;
-    return FxV{t == FX_EXP ? (int64_t)((uint64_t)hi << 32 | fx_lo(x)) : (int64_t)(m ^ (uint64_t)s) - s, fx_max(t, 0x100000u)};
+    return FxV{(int64_t)(m ^ (uint64_t)s) - s, fx_max(t, 0x100000u)};
 }
 
 // the double that fx_split took apart (the sign of a zero aside)
@@ -151,16 +152,15 @@ AT_HD double fx_join(FxV v)
 {
     const uint64_t a = (v.m < 0 ? 0u - (uint64_t)v.m : (uint64_t)v.m) >> FX_GUARD;
     const uint32_t s = (uint32_t)((uint64_t)v.m >> 32) & 0x80000000u;
-    const uint64_t r = a + ((uint64_t)((v.e - 0x100000u) | s) << 32);  // the implicit bit, if any, adds one to the field
-    const uint64_t x = v.e == FX_EXP ? (uint64_t)v.m : r;
+    const uint64_t x = a + ((uint64_t)((v.e - 0x100000u) | s) << 32);  // the implicit bit, if any, adds one to the field
     return fx_double((uint32_t)(x >> 32), (uint32_t)x);
 }
 
 // its integer at the exponent field emax (at least its own), cut downwards
 AT_HD int64_t fx_at(FxV v, uint32_t emax) { return v.m >> fx_min((emax - v.e) >> 20, 63u); }
 
-// Inf and NaN aside, fx_at of fx_split in fewer instructions, for values read
-// once: i is the implicit bit, 0 for a subnormal, whose field then counts as 1
+// fx_at of fx_split in fewer instructions, for values read once: i is the implicit
+// bit, 0 for a subnormal, whose field then counts as 1
 template <int GUARD>
 AT_HD int64_t fx_align(double x, uint32_t emax)
 {

@@ -589,11 +589,12 @@ __global__ void __launch_bounds__(256, 4) stage_weno_interp(const StageArgs a)
 // stages, none between CTAs).  Per-slot level and remaining steps live on
 // the device, so a launch is the same from one chunk of steps to the next.
 // ---------------------------------------------------------------------------
-// Scalar WENO solves: registers for three CTAs an SM, the number a batch asks for
-// by default (900 solves of 512 to 1,024 points: 406 us per step; 549 with two, as
-// the registers fall, 427 with four, which spill).
+// Scalar WENO solves and flames of orders 2 and 4: registers for three CTAs an SM, the
+// number a batch asks for by default (as the registers fall, two: 900 scalar solves of
+// 512 to 1,024 points 549 instead of 406 us per step, 456 flames of those sizes, order
+// 4, 377 instead of 318; four spill: 427 for the scalar ones).
 template <int PDE, int H, bool WENO>
-__global__ void __launch_bounds__(256, WENO && Phys<PDE>::NV == 1 ? 3 : 0)
+__global__ void __launch_bounds__(256, (WENO && Phys<PDE>::NV == 1) || (PDE == RNS && H < 3) ? 3 : 0)
     batch_run(const StageArgs* __restrict__ tab, int64_t* lvl, int64_t* left, const int* __restrict__ order, int n_order,
               int* queue, int64_t chunk)
 {

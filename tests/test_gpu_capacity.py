@@ -106,3 +106,14 @@ def test_batched_scalar_weno_solves_hold_the_ctas_a_batch_asks_for(variant):
     ctas = L._Z25atk_batch_max_ctas_per_smiim  # int atk_batch_max_ctas_per_sm(int variant, int block, size_t smem)
     ctas.restype, ctas.argtypes = ctypes.c_int, [ctypes.c_int, ctypes.c_int, ctypes.c_size_t]
     assert ctas(variant, 256, smem({7: 3, 8: 4}[variant], 64, 3)) >= 3
+
+
+@pytest.mark.parametrize("variant,halo", [(3, 1), (4, 2)], ids=["order 2", "order 4"])
+def test_batched_flames_hold_the_ctas_a_batch_asks_for(variant, halo):
+    import ctypes
+    from paper_2204_01133_gb300 import api
+    L = api.lib()
+    smem, ctas = L._Z20atk_stage_smem_bytesiii, L._Z25atk_batch_max_ctas_per_smiim
+    smem.restype, smem.argtypes = ctypes.c_size_t, [ctypes.c_int] * 3
+    ctas.restype, ctas.argtypes = ctypes.c_int, [ctypes.c_int, ctypes.c_int, ctypes.c_size_t]
+    assert ctas(variant, 256, smem(1, 64, halo)) >= 3
