@@ -123,7 +123,7 @@ KERNEL_FILES = {
     "fused": ("at_device.cuh", "at_fixed.cuh", "at_fused.cu", "at_tilefused.cu"),
 }
 _SHA_STAGE = "42c9217c669c84c42fb523461f2597be634afa8e89e9ef97213dda06c24e8eee"
-_SHA_PERSISTENT = "de61aa93f92627dc0d8bf1b4b0b8274051d4351e87d40b7de299ee8ab280ef0a"
+_SHA_PERSISTENT = "19ffd25b3b92929698abb5790247020c60226fd559e37cd980ca6bebae2e223c"
 _SHA_FUSED = "be6cccd5d2c9deb59f10f9712529a23610fc9e69117f9dcea6539c56be65c50f"
 PROFILED_SHA256 = {
     ("detonation-n16777216", "stage"): _SHA_STAGE,

@@ -591,10 +591,11 @@ int at_set_delays(at_ctx* c, const at_delays* dl)
             c->persist_cap = cap;
             c->persist_variant = v;
         }
-        // large PEs of the reacting flow that fit as dense rows only are faster with
-        // one launch per stage (us per step, resident and per stage: 304 PEs of 480
-        // points 81.3 and 73.8, 100 of 870 104.5 and 57.3; with split rows 152 of 760
-        // 55.6 and 66.5, 456 of 64 23.5 and 30.3): the automatic rule leaves them there
+        // large PEs of the reacting flow that fit as dense rows only are mostly faster
+        // with one launch per stage (us per step, resident and per stage: 304 PEs of 480
+        // points 76.1 and 73.2, 100 of 870 90.9 and 56.5, but 456 of 300 69.8 and 75.7;
+        // with split rows 152 of 760 54.9 and 65.9, 456 of 64 23.6 and 30.0): the
+        // automatic rule leaves them there
         c->persist_auto = c->pb.pde == AT_ADVDIFF || c->persist_variant < 3;
         c->cluster_c = (int)c->fit.take(
             c->pb.pde == AT_ADVDIFF

@@ -162,13 +162,13 @@ __device__ __forceinline__ void bar_arrive_p(int p, int count)
 // arrival it would otherwise have consumed, so every barrier completes.
 //
 // How many PEs fit the chip is registers and shared memory.  CTAS = 2 of 288
-// threads an SM leaves the registers the code wants (85 at order 6); CTAS = 3 holds
-// it to 72 for more PEs (none spilt, 3 to 6 % slower where both fit: 304 PEs of
-// 64 points 18.7 and 20.0 us per step; 456 of them 23.5, one launch per stage
-// 30.3).  CTAS = 1 has sixteen worker warps instead of eight, for some PE sizes where
-// every PE has an SM to itself (persist_wide).  DENSE has the reacting flow's rows
-// as doubles, split where they are read, in 27 words a point instead of 34, for
-// large PEs that no other holds (100 of 400 points 52.9 us against 39.9).
+// threads an SM leaves the registers the code wants (86 at order 6); CTAS = 3 holds
+// it to 72 for more PEs (none spilt, 3 to 6 % slower where both fit; 456 PEs of 64
+// points 23.6 us per step, one launch per stage 30.0).  CTAS = 1 has sixteen worker
+// warps instead of eight, for some PE sizes where every PE has an SM to itself
+// (persist_wide).  DENSE has the reacting flow's rows as doubles, split where they
+// are read, in 27 words a point instead of 34, for large PEs that no other holds
+// (456 of 300 points 69.8 us; per stage 75.7).
 template <int PDE, int H, int CTAS, bool DENSE>
 __global__ void __launch_bounds__(CTAS == 1 ? 544 : 288, CTAS) persist_central(const StageArgs a, int64_t level0, int64_t nsteps)
 {
@@ -520,14 +520,18 @@ bool persist_takes(int pde, int B, int H)
                              (size_t)B) <= 200 * 1024;
 }
 // Whether the variant with sixteen worker warps is the faster one for PEs of B
-// points, each with an SM to itself: from 65 to 96 points eight warps have a second,
-// mostly empty round of (point, variable) items, and from 224 on half as many rounds
-// are left; between, waiting for twice the warps costs more than it saves.  us per
-// step with eight and sixteen, order 6: 72 points 17.8 and 16.3, 96 18.2 and 16.3,
-// 150 21.9 and 22.4, 192 25.2 and 26.1, 256 37.8 and 27.9 (FP64 throughout 36.3), 600
-// 59.5 and 50.8; order 4: 96 16.7 and 15.6, 150 19.4 and 21.0, 224 24.0 and 24.1, 256
-// 32.8 and 26.0 (FP64 31.4)
-bool persist_wide(int pde, int B) { return pde == atk::RNS && ((B > 64 && B <= 96) || B >= 224); }
+// points, each with an SM to itself: from 65 points on eight warps have a second
+// round of (point, variable) items, mostly empty up to 96, and from 224 on half as
+// many rounds are left; between, waiting for twice the warps costs more than it saves
+// (order 6, whose items are longer, gains up to 128).  us per step with eight and
+// sixteen, order 6: 72 points 17.8 and 16.3, 96 18.2 and 16.3, 128 21.3 and 20.2 (by
+// arrival 20.6 and 17.9, FP64 throughout 17.7), 150 21.9 and 22.4, 192 25.2 and 26.1,
+// 256 37.8 and 27.9 (FP64 36.3), 600 59.5 and 50.8; order 4: 96 16.7 and 15.6, 128 17.9
+// and 18.0, 150 19.4 and 21.0, 224 24.0 and 24.1, 256 32.8 and 26.0 (FP64 31.4)
+bool persist_wide(int pde, int B, int H)
+{
+    return pde == atk::RNS && ((B > 64 && B <= (H == 3 ? 128 : 96)) || B >= 224);
+}
 
 // worker warps for the PE's points (at least two roles' worth for phase A)
 // plus one halo warp
@@ -548,7 +552,7 @@ int64_t atk_persist_capacity(int pde, int order, int B, int variant, int device)
 {
     void* fn = variant < kVariants ? persist_kernel(pde, order, variant) : nullptr;
     const int H = order / 2;
-    if (!fn || !persist_takes(pde, B, H) || (variant == 0 && !persist_wide(pde, B))) return 0;
+    if (!fn || !persist_takes(pde, B, H) || (variant == 0 && !persist_wide(pde, B, H))) return 0;
     const size_t smem = persist_smem_bytes(pde, B, H, variant);
     if (smem > 227 * 1024 - 64) return 0;  // (64 for the kernel's own shared variables)
     int per_sm = 0, sms = 0, coop = 0;

@@ -31,7 +31,7 @@ def _run(pb, u0, steps, path):
 
 @pytest.mark.parametrize("order", [2, 4, 6])
 @pytest.mark.parametrize("pe_size,pes", [(16, 1368), (24, 1064), (32, 760), (48, 608), (64, 304), (64, 305), (64, 456),
-                                         (65, 152), (96, 152), (96, 153), (97, 152), (223, 100), (224, 152),
+                                         (65, 152), (96, 152), (96, 153), (97, 152), (128, 152), (128, 153), (129, 152), (223, 100), (224, 152),
                                          (224, 153), (256, 1), (280, 456), (320, 456), (421, 304), (488, 304), (749, 152), (750, 152),
                                          (850, 152), (872, 152)])
 def test_flames_on_the_persistent_path(order, pe_size, pes):
